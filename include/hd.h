@@ -104,9 +104,14 @@ typedef struct hd_opts {
                                 (in the checkerboard of Sec. II.B a pass reads
                                 one cell row beyond its own cells and a rebuild
                                 moves a disk by at most one cell).  Same chain.
-                                0: automatic (16 when the colour pass is 1.5 to
-                                3.5 waves of resident blocks deep, 8 when it is
-                                deeper, none when it is shallower);
+                                0: the library chooses the order of the launches,
+                                of hd_sweep too: where cells hold up to four disks,
+                                the sweeps of a draw table (up to 256) run as one
+                                launch, of a box that fits one block's shared
+                                memory or of tiles of cells staged there (FP64: up
+                                to 655,360 cells); else strips, 16 when the colour
+                                pass is 1.5 to 3.5 waves of resident blocks deep, 8
+                                when it is deeper, none when it is shallower;
                                 1: none; 2 .. 64: K strips (at most m / 2, and
                                 only for one replica, the split kernels and one
                                 thread per cell; else HD_ERR_ARG) [0]          */
@@ -116,10 +121,14 @@ typedef struct hd_opts {
                                 one-replica launches, the replicas' chains
                                 concurrently (independent chains, Sec. IV.A's
                                 scan); the measurement stays one batched launch.
-                                Same chains.  0: automatic (on where it applies);
-                                1: off [0]                                      */
+                                Same chains.  0: the library chooses (the one-launch
+                                sweeps as for strips 0, up to 1024 replicas; else
+                                branches where they apply); 1: one batched launch
+                                per phase [0]                                   */
 } hd_opts;
 
+/* The one-launch sweeps of strips = 0 and replica_branches = 0 wait for
+ * neighbouring tiles with a bound; a wait that gives up sets HD_ERR_TIMEOUT. */
 enum { HD_SWEEP_SPLIT = 0, HD_SWEEP_FUSED = 1, HD_SWEEP_TMA = 2, HD_SWEEP_PERSISTENT = 3 };
 
 /* Geometry of one replica as realised by the library. */
@@ -266,8 +275,8 @@ int32_t hd_replicas(const hd_ctx *ctx);
  * hd_psi6_local_device.  Each distinct step is captured once as a CUDA graph
  * and replayed, its sweeps on concurrent branches where hd_opts asks for strips
  * or replica branches (graph_branches of hd_get_geometry); while profiling is
- * enabled the graph instead runs every kernel in order, with a timing event
- * before and after it, and each replay is followed by a synchronisation that
+ * enabled the graph instead runs the split kernels in order, with a timing event
+ * before and after each, and each replay is followed by a synchronisation that
  * adds the kernels' times to hd_kernel_times.  Capturing and instantiating a
  * step graph is a one-time cost per distinct step (at N = 2^20 about 6 ms
  * serial, about 0.13 s as 16 strips, whose graph holds ~8000 kernel nodes per
@@ -460,7 +469,7 @@ typedef enum hd_kernel_class {
     HD_K_PSI6 = 5,       /* local psi_6                                       */
     HD_K_PSI6_REDUCE = 6,/* global Psi_6 reduction                            */
     HD_K_POSITIONS = 7,  /* cell frame to global positions                    */
-    HD_K_SWEEP = 8,      /* whole sweeps in one launch (fused or persistent)  */
+    HD_K_SWEEP = 8,      /* whole sweeps in one launch (boxes, tiles, fused or persistent) */
     HD_K_ANALYSIS = 9,   /* Psi_6 autocorrelation, correlation time, field    */
     HD_KERNEL_CLASSES = 10
 } hd_kernel_class;

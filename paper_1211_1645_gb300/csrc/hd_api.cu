@@ -16,6 +16,7 @@
 #include "hd_analysis.h"
 #include "hd_bin.h"
 #include "hd_bounds.h"
+#include "hd_tile.h"
 
 using hd::CellBufs;
 using hd::Frame;
@@ -40,6 +41,8 @@ constexpr int kMaxStrips = 64;    // strips of a one-replica graph wavefront
 constexpr int kAutoStrips = 16;   // strips chosen when the colour pass is 1.5 to 3.5 waves deep
 constexpr int kAutoStripsDeep = 8;  // ... and when it is deeper
 constexpr int kMaxBranches = 64;  // replicas on concurrent branches of a captured step
+constexpr int kMaxTiledReplicas = 1024;       // replicas of a context on the tile or box sweep (bounds its scratch)
+constexpr int64_t kTileCells64 = 640 * 1024;  // cells of an FP64 context up to which the tile sweep is the faster
 
 struct Plan {
     Rep rep;
@@ -64,6 +67,12 @@ struct hd_ctx {
     int bands = 0;          // bands of two cell rows over all replicas
     uint32_t* persist_sync = nullptr;  // ticket, abort word and per-band progress of the persistent sweep
     int persist_blocks = 0;            // its grid: the blocks resident at once
+    // the tile sweep (hd_tile.cu): the sweeps of contexts whose options leave
+    // the order of the launches to the library
+    bool tiled = false;
+    std::vector<hd::TileGrid> tiles;   // [R]
+    hd::TileCfg tile_cfg{};
+    void* box_spill = nullptr;         // set: the boxes are small enough for one block each (launch_sweeps_box)
     bool persist_stall = false;        // test hook (HD_TEST_PERSIST_STALL=1 at creation)
     // analysis scratch, grown on demand and freed with the context
     double2* acf = nullptr;     // [R][max_lag + 1]
@@ -225,6 +234,38 @@ void set_hist_f32_bounds(Rep& r, double e0, double eK) {
     r.psi_m = std::nextafter(float(hd::cells_f32_margin(r.w, 2)), HUGE_VALF);
 }
 
+// Tiles of every replica for the tile sweep (see hd_tile.h); false where it
+// cannot run (a box of fewer than six half-cells) or another order of the
+// sweeps is faster.  As few tiles as the staged region allows, since every
+// tile also updates some cells around it; one replica that would leave SMs
+// idle is split further, its longer side first, down to tiles of 16 cells
+// (N = 65,536: 144 tiles 8.8 us per sweep, 72 tiles 10.8).
+bool plan_tiles(hd_ctx* ctx, int sms) {
+    // The FP64 form stages twice the bytes per cell in tiles half as large, and
+    // its frame changes are FP64-bound: per sweep 30.5 us against 42.9 as graph
+    // branches at N = 524,288, 46.5 against ~48 at 786,432, 62 against 54 at
+    // 1,048,576.
+    if (!ctx->fixed && ctx->Ctot > kTileCells64) return false;
+    const hd::TileLimits lim = hd::tile_limits(ctx->fixed);
+    int64_t total = 0;
+    ctx->tiles.clear();
+    for (const Rep& r : ctx->reps) {
+        if (r.hm < 6) return false;
+        const int least = r.hm < 12 ? 1 : 2;  // see wrap_half
+        hd::TileGrid g{int32_t(total), std::max(least, (r.m + lim.max_x - 1) / lim.max_x),
+                       std::max(least, (r.m + lim.max_y - 1) / lim.max_y)};
+        if (ctx->R == 1)
+            while (int64_t(g.ntx) * g.nty < sms && r.hm / std::max(g.ntx, g.nty) >= 8) {
+                if (r.m / g.ntx > r.m / g.nty) ++g.ntx; else ++g.nty;
+            }
+        ctx->tiles.push_back(g);
+        total += int64_t(g.ntx) * g.nty;
+    }
+    ctx->tile_cfg.total = total;
+    ctx->tile_cfg.grid0 = ctx->tiles[0];
+    return total * hd::kMaxChunk < (int64_t(1) << 31);
+}
+
 // Geometry of one chain (Sec. II.A, II.B).  Lengths in units of sigma.
 hd_status plan_replica(int64_t N, double eta, double sigma, double delta, uint64_t seed, const hd_opts& o,
                        double cell_min, Plan& pl) {
@@ -279,6 +320,12 @@ hd_status plan_replica(int64_t N, double eta, double sigma, double delta, uint64
     r.key0 = uint32_t(seed & 0xffffffffu);
     r.key1 = uint32_t(seed >> 32);
     set_f32_bounds(r);
+    if (fixed) {  // the tile sweep's bounds, in units of 2^-22 sigma
+        const double M = hd::fixed_f32_margin(r.W);
+        r.wf = float(0.25 * double(r.W));
+        r.d2_lo = std::nextafter(float(0x1p46 - M), -HUGE_VALF);
+        r.d2_hi = std::nextafter(float(0x1p46 + M), HUGE_VALF);
+    }
     pl.nlat = n;
     pl.eta_req = eta;
     return HD_OK;
@@ -622,13 +669,37 @@ cudaError_t enqueue_strips(hd_ctx* ctx, cudaStream_t s, int nc) {
 }
 
 // Enqueue n sweeps on stream s (draw tables of up to kMaxChunk sweeps, then
-// per sweep either one fused launch or a rebuild and four colour passes).
+// the table's sweeps in one tile-sweep or persistent launch, or per sweep
+// either one fused launch or a rebuild and four colour passes).
 // While a step graph is captured (not for a profiled graph, whose event nodes
 // time each kernel in order), the sweeps of a one-replica context with strips
 // run as a graph wavefront, and those of a batch with replica branches as
 // one branch per replica.
 cudaError_t enqueue_sweeps(hd_ctx* ctx, cudaStream_t s, int64_t n, bool capturing) {
     const hd::LaunchCfg c = ctx->cfg(s);
+    if (ctx->tiled && !ctx->profiling) {
+        cudaError_t e = cudaSuccess;
+        for (int64_t left = n; left > 0 && e == cudaSuccess;) {
+            const int nc = int(std::min<int64_t>(left, hd::kMaxChunk));
+            e = launch(ctx, HD_K_DRAWS, [&] { return hd::launch_draws(c, ctx->table, ctx->frame, ctx->sweep_ctr, nc); },
+                       capturing);
+            if (e == cudaSuccess)
+                e = launch(ctx, HD_K_SWEEP, [&] {
+                    if (ctx->box_spill)
+                        return hd::launch_sweeps_box(c, ctx->box_spill, ctx->table, nc, ctx->buf[ctx->cur],
+                                                     ctx->buf[ctx->cur ^ 1], ctx->counters, ctx->err);
+                    return hd::launch_sweeps_tile(c, ctx->tile_cfg, ctx->table, nc, ctx->buf[ctx->cur],
+                                                  ctx->buf[ctx->cur ^ 1], ctx->counters, ctx->err);
+                }, capturing);
+            if (nc & 1) ctx->cur ^= 1;
+            left -= nc;
+        }
+        return e;
+    }
+    if (ctx->tiled && n > 0) {  // profiled: the split kernels, whose rebuild expects the other generation cleared
+        const cudaError_t e = cudaMemsetAsync(ctx->buf[ctx->cur ^ 1].cnt, 0, size_t(ctx->Ctot) + kCellPad, s);
+        if (e != cudaSuccess) return e;
+    }
     const bool wave = capturing && !ctx->prof_capture && (ctx->strips > 1 || ctx->branches);
     if (wave) {
         const int nb = ctx->strips > 1 ? ctx->strips : ctx->R;
@@ -982,9 +1053,38 @@ hd_status hd_batch_init(hd_ctx** out, int32_t R, const int64_t* N, const double*
         }
     }
     ctx->branches = R > 1 && R <= kMaxBranches && split1 && o.replica_branches == 0;
+    // The order of the launches left to the library (strips, replica_branches
+    // 0): all sweeps of a draw table in one launch, of whole small boxes or of
+    // tiles, where the launch boundary of the split kernels costs more than
+    // their work (per sweep at N = 256 5.3 us against 11.1 as a serial graph, at
+    // 65,536 8.8 against 20.8, at 2^20 30 against 35 as 16 strips).
+    if (ok && split1 && cap == 4 && R <= kMaxTiledReplicas && (R == 1 ? o.strips == 0 : o.replica_branches == 0)) {
+        int dev = 0, sms = 0;
+        ok = cudaGetDevice(&dev) == cudaSuccess &&
+             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
+        unsigned char* spill = nullptr;
+        if (ok && std::all_of(ctx->reps.begin(), ctx->reps.end(), [](const Rep& r) { return r.hm <= hd::box_max_hm(); })) {
+            ok = dev_alloc(ctx, &spill, size_t(R) * hd::box_spill(ctx->fixed));
+            ctx->box_spill = spill;
+            ctx->tiled = true;
+        } else if (ok && plan_tiles(ctx, sms)) {
+            hd::TileCfg& t = ctx->tile_cfg;
+            hd::TileGrid* grids = nullptr;
+            ok = hd::tile_blocks(ctx->cfg(), &t.blocks) == cudaSuccess && t.blocks > 0;
+            t.blocks = int(std::min<int64_t>(t.blocks, t.total));
+            ok = ok && dev_alloc(ctx, &grids, size_t(R));
+            ok = ok && dev_alloc(ctx, &t.sync, hd::tile_sync_words(t.total));
+            ok = ok && dev_alloc(ctx, &spill, size_t(t.blocks) * hd::tile_limits(ctx->fixed).spill);
+            ok = ok && cudaMemcpy(grids, ctx->tiles.data(), sizeof(hd::TileGrid) * size_t(R), cudaMemcpyHostToDevice) == cudaSuccess;
+            t.grids = grids;
+            t.spill = spill;
+            ctx->tiled = true;
+        }
+        if (ctx->tiled) ctx->strips = 1;
+    }
     // the branches' streams and events exist before any step is captured
     // (one side stream at least: the measurement's psi_6 branch)
-    ok = ok && ensure_side(ctx, std::max(1, ctx->strips > 1 ? ctx->strips : (ctx->branches ? R : 1)),
+    ok = ok && ensure_side(ctx, std::max(1, ctx->strips > 1 ? ctx->strips : (ctx->branches && !ctx->tiled ? R : 1)),
                            ctx->strips > 1) == cudaSuccess;
     if (!ok) {
         free_ctx(ctx);

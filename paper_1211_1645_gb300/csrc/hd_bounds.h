@@ -8,6 +8,7 @@
 #pragma once
 
 #include <cmath>
+#include <cstdint>
 
 namespace hd {
 
@@ -21,6 +22,16 @@ inline double pair_f32_margin(double w, double delta) {
     const double R = 2.0 * w + delta;
     const double E = t * (2.0 * w + delta) + u * (3.0 * w + R);
     return 2.0 * (4.0 * R * E + 2.0 * E * E + 4.0 * u * (R + E) * (R + E) + 16.0 * std::ldexp(1.0, -53) * R * R);
+}
+
+// A pair of the tile sweep in the fixed form, in units of 2^-22 sigma: |q|,
+// |np| < W / 4 < 2^24 truncated to whole units (a difference errs by less than
+// 0.75), W / 4 rounded to float (0.5), the cell offset and the difference
+// below 2^25 (1 each): the difference errs by at most E = 3.25 units; the
+// square sum as above, against the exact integer.
+inline double fixed_f32_margin(int32_t W) {
+    const double u = std::ldexp(1.0, -24), R = 0.5 * double(W), E = 3.25;
+    return 2.0 * (4.0 * R * E + 2.0 * E * E + 4.0 * u * (R + E) * (R + E));
 }
 
 // A pair of a measurement H cells apart at most: both coordinates in [0, w),
