@@ -18,72 +18,121 @@ namespace hd {
 
 // Series row layout: series[(t * R + r) * 4 + {0: beta P / rho, 1: g(2 sigma+), 2: Re Psi_6, 3: Im Psi_6}].
 //
-// S[r][d] = sum_{t < T - d} Psi(t) conj(Psi(t + d)), one thread per lag d.
-__global__ void __launch_bounds__(256)
-k_acf_sums(const double* __restrict__ series, int R, int64_t T, int64_t max_lag, double2* __restrict__ S) {
+// S[r][d] = sum_{t < T - d} Psi(t) conj(Psi(t + d)).  A block takes 128 lags
+// (one per thread) and kAcfChunk times, staged with the entries the lags reach;
+// the partial sums of the chunks are added in order by k_acf_norm.  What bounds
+// it is FP64: four fused multiply-adds per term at two lanes per clock and SM.
+// One thread per lag over all T instead ran a serial chain of loads and adds
+// (T = 4000, 401 lags, four replicas: 2.31 ms, here 0.06).
+constexpr int kAcfLags = 128, kAcfChunk = 128;
+
+__global__ void __launch_bounds__(kAcfLags)
+k_acf_sums(const double* __restrict__ series, int R, int64_t T, int64_t max_lag, int64_t len, double2* __restrict__ part) {
     pdl_begin();
+    __shared__ double2 s_a[kAcfChunk], s_c[kAcfChunk + kAcfLags];
     const int r = blockIdx.y;
-    const int64_t d = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (d > max_lag) return;
-    double sr = 0.0, si = 0.0;
-    for (int64_t t = 0; t + d < T; ++t) {
-        const double a = series[(size_t(t) * R + r) * 4 + 2], b = series[(size_t(t) * R + r) * 4 + 3];
-        const double c = series[(size_t(t + d) * R + r) * 4 + 2], e = series[(size_t(t + d) * R + r) * 4 + 3];
-        // (a + i b)(c - i e) = (a c + b e) + i (b c - a e)
-        sr = __dadd_rn(sr, __dadd_rn(__dmul_rn(a, c), __dmul_rn(b, e)));
-        si = __dadd_rn(si, __dsub_rn(__dmul_rn(b, c), __dmul_rn(a, e)));
+    const int64_t d0 = int64_t(blockIdx.x) * kAcfLags, d = d0 + threadIdx.x;
+    const int64_t t1 = min(T, int64_t(blockIdx.z + 1) * len);
+    auto entry = [&](int64_t t) {
+        const double* row = series + (size_t(t) * R + r) * 4;
+        return t < T ? make_double2(row[2], row[3]) : make_double2(0.0, 0.0);
+    };
+    double sr = 0.0, si = 0.0, ur = 0.0, ui = 0.0;  // two chains per part
+    for (int64_t t0 = int64_t(blockIdx.z) * len; t0 < t1; t0 += kAcfChunk) {
+        for (int i = threadIdx.x; i < kAcfChunk + kAcfLags; i += kAcfLags) {
+            s_c[i] = entry(t0 + d0 + i);
+            if (i < kAcfChunk) s_a[i] = entry(t0 + i);
+        }
+        __syncthreads();
+        // a pair whose later entry is beyond the series is not part of the
+        // sum, also where the series holds an infinity or NaN
+        const int n = d > max_lag ? 0 : int(max(int64_t(0), min(min(int64_t(kAcfChunk), t1 - t0), T - d - t0)));
+        for (int i = 0; i < n; ++i) {
+            const double2 a = s_a[i], c = s_c[i + int(threadIdx.x)];
+            // (a.x + i a.y)(c.x - i c.y) = (a.x c.x + a.y c.y) + i (a.y c.x - a.x c.y)
+            sr = __fma_rn(a.x, c.x, sr);
+            ur = __fma_rn(a.y, c.y, ur);
+            si = __fma_rn(a.y, c.x, si);
+            ui = __fma_rn(a.x, c.y, ui);
+        }
+        __syncthreads();
     }
-    S[size_t(r) * size_t(max_lag + 1) + size_t(d)] = make_double2(sr, si);
+    if (d <= max_lag)
+        part[(size_t(blockIdx.z) * R + r) * size_t(max_lag + 1) + size_t(d)] = make_double2(__dadd_rn(sr, ur), __dsub_rn(si, ui));
 }
 
-// Eq. 9: C(d) = (S(d) / (T - d)) / (S(0) / T), in place; one block per
-// replica, so S(0) is read by every thread before any thread overwrites it.
-__global__ void __launch_bounds__(256)
-k_acf_norm(int R, int64_t T, int64_t max_lag, double2* __restrict__ S) {
+// Eq. 9: C(d) = (S(d) / (T - d)) / (S(0) / T), S from the chunks' partial sums
+// in order; blockIdx.y = replica.  Every block adds up S(0) itself.
+__global__ void __launch_bounds__(128)
+k_acf_norm(int R, int64_t T, int64_t max_lag, int chunks, const double2* __restrict__ part, double2* __restrict__ C) {
     pdl_begin();
-    double2* row = S + size_t(blockIdx.x) * size_t(max_lag + 1);
-    const double den = __ddiv_rn(row[0].x, double(T));
+    __shared__ double s_zero[128];
+    const int r = blockIdx.y;
+    const size_t row = size_t(max_lag + 1), step = size_t(R) * row;
+    const double2* p = part + size_t(r) * row;
+    double z = 0.0;
+    for (int c = threadIdx.x; c < chunks; c += 128) z = __dadd_rn(z, p[size_t(c) * step].x);
+    s_zero[threadIdx.x] = z;
     __syncthreads();
-    for (int64_t d = threadIdx.x; d <= max_lag; d += blockDim.x) {
-        const double2 s = row[d];
-        const double n = double(T - d);
-        row[d] = make_double2(__ddiv_rn(__ddiv_rn(s.x, n), den), __ddiv_rn(__ddiv_rn(s.y, n), den));
+    for (int o = 64; o > 0; o >>= 1) {
+        if (int(threadIdx.x) < o) s_zero[threadIdx.x] = __dadd_rn(s_zero[threadIdx.x], s_zero[threadIdx.x + o]);
+        __syncthreads();
     }
+    const int64_t d = int64_t(blockIdx.x) * 128 + threadIdx.x;
+    if (d > max_lag) return;
+    const double den = __ddiv_rn(s_zero[0], double(T));
+    double a = 0.0, b = 0.0;
+    for (int c = 0; c < chunks; ++c) {
+        const double2 v = p[size_t(c) * step + size_t(d)];
+        a = __dadd_rn(a, v.x);
+        b = __dadd_rn(b, v.y);
+    }
+    const double n = double(T - d);
+    // S(0) as the denominator has it, so that C(0) = 1
+    if (d == 0) a = s_zero[0];
+    C[size_t(r) * row + size_t(d)] = make_double2(__ddiv_rn(__ddiv_rn(a, n), den), __ddiv_rn(__ddiv_rn(b, n), den));
+}
+
+__device__ __forceinline__ double lane_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = __dadd_rn(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
 }
 
 // Correlation time of the exponential part: least-squares line through
 // (d, ln Re C(d)) over lag_lo <= d <= lag_hi with Re C > 0, tau = -1 / slope
-// (NaN with fewer than two such lags or a slope >= 0).  One thread per replica.
-__global__ void k_acf_tau(int R, int64_t max_lag, int64_t lag_lo, int64_t lag_hi, const double2* __restrict__ C,
-                          double* __restrict__ tau) {
+// (NaN with fewer than two such lags or a slope >= 0).  One warp per replica.
+__global__ void __launch_bounds__(32)
+k_acf_tau(int64_t max_lag, int64_t lag_lo, int64_t lag_hi, const double2* __restrict__ C, double* __restrict__ tau) {
     pdl_begin();
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R) return;
-    const double2* row = C + size_t(r) * size_t(max_lag + 1);
-    double sx = 0.0, sy = 0.0;
-    int64_t n = 0;
-    for (int64_t d = lag_lo; d <= lag_hi; ++d) {
+    const double2* row = C + size_t(blockIdx.x) * size_t(max_lag + 1);
+    const int lane = int(threadIdx.x);
+    double sx = 0.0, sy = 0.0, cnt = 0.0;
+    for (int64_t d = lag_lo + lane; d <= lag_hi; d += 32) {
         if (row[d].x > 0.0) {
             sx = __dadd_rn(sx, double(d));
             sy = __dadd_rn(sy, log(row[d].x));
-            ++n;
+            cnt += 1.0;
         }
     }
+    sx = lane_sum(sx);
+    sy = lane_sum(sy);
+    cnt = lane_sum(cnt);
     double out = CUDART_NAN;
-    if (n >= 2) {
-        const double mx = __ddiv_rn(sx, double(n)), my = __ddiv_rn(sy, double(n));
+    if (cnt >= 2.0) {
+        const double mx = __ddiv_rn(sx, cnt), my = __ddiv_rn(sy, cnt);
         double sxy = 0.0, sxx = 0.0;
-        for (int64_t d = lag_lo; d <= lag_hi; ++d) {
+        for (int64_t d = lag_lo + lane; d <= lag_hi; d += 32) {
             if (row[d].x > 0.0) {
                 const double dx = __dsub_rn(double(d), mx);
                 sxy = __dadd_rn(sxy, __dmul_rn(dx, __dsub_rn(log(row[d].x), my)));
                 sxx = __dadd_rn(sxx, __dmul_rn(dx, dx));
             }
         }
-        const double slope = __ddiv_rn(sxy, sxx);
+        const double slope = __ddiv_rn(lane_sum(sxy), lane_sum(sxx));
         if (slope < 0.0) out = __ddiv_rn(-1.0, slope);
     }
-    tau[r] = out;
+    if (lane == 0) tau[blockIdx.x] = out;
 }
 
 // Coarse field, accumulation: one thread per disk (global id order), from
@@ -371,17 +420,28 @@ k_corr_norm(int64_t n, const double* __restrict__ acc, double2* __restrict__ out
                      : make_double2(CUDART_NAN, CUDART_NAN);
 }
 
-cudaError_t launch_acf(const LaunchCfg& c, const double* series, int64_t T, int64_t max_lag, double2* C) {
-    const dim3 grid(unsigned((max_lag + 256) / 256), unsigned(c.R));
-    const cudaError_t e = launch_k(k_acf_sums, grid, dim3(256), 0, c.stream, series, c.R, T, max_lag, C);
+// Chunks of times: enough blocks to fill the GPU, no more than the series has
+// pieces of kAcfChunk entries, so that the partial sums stay small where the
+// lags and replicas are many.
+int acf_chunks(int R, int64_t T, int64_t max_lag) {
+    const int64_t tiles = int64_t(R) * ((max_lag + kAcfLags) / kAcfLags);
+    return int(std::max<int64_t>(1, std::min<int64_t>({64, (1200 + tiles - 1) / tiles, (T + kAcfChunk - 1) / kAcfChunk})));
+}
+
+cudaError_t launch_acf(const LaunchCfg& c, const double* series, int64_t T, int64_t max_lag, double2* part, double2* C) {
+    const int chunks = acf_chunks(c.R, T, max_lag);
+    const int64_t pieces = (T + kAcfChunk - 1) / kAcfChunk, len = (pieces + chunks - 1) / chunks * kAcfChunk;
+    const unsigned tiles = unsigned((max_lag + kAcfLags) / kAcfLags);
+    const cudaError_t e = launch_k(k_acf_sums, dim3(tiles, unsigned(c.R), unsigned(chunks)), dim3(kAcfLags), 0, c.stream,
+                                   series, c.R, T, max_lag, len, part);
     if (e != cudaSuccess) return e;
-    return launch_k(k_acf_norm, dim3(unsigned(c.R)), dim3(256), 0, c.stream, c.R, T, max_lag, C);
+    return launch_k(k_acf_norm, dim3(unsigned((max_lag + 128) / 128), unsigned(c.R)), dim3(128), 0, c.stream, c.R, T,
+                    max_lag, chunks, (const double2*)part, C);
 }
 
 cudaError_t launch_acf_tau(const LaunchCfg& c, int64_t max_lag, int64_t lag_lo, int64_t lag_hi, const double2* C,
                            double* tau) {
-    return launch_k(k_acf_tau, dim3(unsigned((c.R + 31) / 32)), dim3(32), 0, c.stream, c.R, max_lag, lag_lo, lag_hi,
-                    C, tau);
+    return launch_k(k_acf_tau, dim3(unsigned(c.R)), dim3(32), 0, c.stream, max_lag, lag_lo, lag_hi, C, tau);
 }
 
 cudaError_t launch_field(const LaunchCfg& c, int64_t Ntot, int bins, const double* xy, const double2* psi,

@@ -1708,7 +1708,8 @@ hd_status series_length(hd_ctx* ctx, int64_t& T) {
 
 // C[R][max_lag + 1] of the current series into ctx->acf.
 hd_status enqueue_acf(hd_ctx* ctx, int64_t T, int64_t max_lag) {
-    const size_t need = size_t(ctx->R) * size_t(max_lag + 1);
+    // the result, then the partial sums of the chunks of times
+    const size_t rows = size_t(ctx->R) * size_t(max_lag + 1), need = rows * (1 + size_t(hd::acf_chunks(ctx->R, T, max_lag)));
     if (need > ctx->acf_cap) {
         if (ctx->acf) cudaFree(ctx->acf);
         ctx->acf = nullptr;
@@ -1716,7 +1717,7 @@ hd_status enqueue_acf(hd_ctx* ctx, int64_t T, int64_t max_lag) {
         HD_CK(ctx, cudaMalloc(&ctx->acf, need * sizeof(double2)));
         ctx->acf_cap = need;
     }
-    HD_CK(ctx, launch(ctx, HD_K_ANALYSIS, [&] { return hd::launch_acf(ctx->cfg(), ctx->series, T, max_lag, ctx->acf); }));
+    HD_CK(ctx, launch(ctx, HD_K_ANALYSIS, [&] { return hd::launch_acf(ctx->cfg(), ctx->series, T, max_lag, ctx->acf + rows, ctx->acf); }));
     return HD_OK;
 }
 

@@ -99,8 +99,10 @@ cudaError_t launch_sweeps_persist(const LaunchCfg& c, const Frame* table, int ns
                                   unsigned long long* counters, int* err, uint32_t* sync, int total_bands);
 cudaError_t launch_positions(const LaunchCfg& c, const Frame* cur, CellBufs cells, double* xy);
 // Psi_6 autocorrelation of the measurement series (series[T][R][4]) for lags
-// 0..max_lag into C[R][max_lag + 1], and the correlation time from it.
-cudaError_t launch_acf(const LaunchCfg& c, const double* series, int64_t T, int64_t max_lag, double2* C);
+// 0..max_lag into C[R][max_lag + 1], and the correlation time from it.  part:
+// acf_chunks x R x (max_lag + 1) partial sums.
+int acf_chunks(int R, int64_t T, int64_t max_lag);
+cudaError_t launch_acf(const LaunchCfg& c, const double* series, int64_t T, int64_t max_lag, double2* part, double2* C);
 cudaError_t launch_acf_tau(const LaunchCfg& c, int64_t max_lag, int64_t lag_lo, int64_t lag_hi, const double2* C,
                            double* tau);
 // Coarse psi_6 field over bins x bins sampling areas per replica (acc: R bins^2 x 3 doubles of scratch).
