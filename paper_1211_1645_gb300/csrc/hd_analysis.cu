@@ -260,27 +260,205 @@ k_sq_amp(const Rep* __restrict__ reps, bool fixed, int nq, const int2* __restric
     }
 }
 
-// S_r(q) = |A_r(q)|^2 / N_r (Eq. 10); best[r] = first q of largest S.  One block per replica.
+// ---------------------------------------------------------------------------
+// The same amplitudes for wave vectors that share their components, as a map
+// or a window of them does: with U_n(h) = exp(2 pi i h x_n / L) and V_n(k)
+// likewise, A(h, k) = sum_n U_n(h) V_n(k), so a disk needs one plane wave per
+// distinct h and k (15 FP64 operations each here) and four fused
+// multiply-adds per (h, k), against ~100 FP64-pipe operations for the division
+// and the sine and cosine of every (h, k) itself.  FP64 rate is the bound:
+// N = 65,536 and 441 wave vectors of 21 x 21 components 2.88 ms before, 0.31
+// here.  The turn x / L is kept to 96 bits, so that h x / L mod 1 is exact to
+// 2^-64 for every 32-bit h (the division in double loses h 2^-53 of a turn).
+// ---------------------------------------------------------------------------
+constexpr int kPairDisks = 32;      // disks staged at a time
+constexpr int kPairThreads = 256;
+constexpr int kPairMax = 160;       // distinct h plus distinct k of a replica
+constexpr int kPairQ = 2;           // wave vectors per thread
+constexpr int kTurnTable = 128;
+
+struct Turn {
+    unsigned long long hi;  // x / L mod 1 in units of 2^-64 ...
+    uint32_t lo;            // ... and the next 32 bits
+};
+
+// X / LF for 0 <= X < LF < 2^42, digit by digit (22 bits at a time).
+__device__ __forceinline__ Turn turn_fixed(uint64_t X, uint64_t LF) {
+    uint64_t digit[5], rem = X;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {  // 110 bits
+        rem <<= 22;
+        digit[k] = rem / LF;
+        rem -= digit[k] * LF;
+    }
+    Turn t;
+    t.hi = digit[0] << 42 | digit[1] << 20 | digit[2] >> 2;
+    t.lo = uint32_t((digit[2] & 3u) << 30 | digit[3] << 8 | digit[4] >> 14);
+    return t;
+}
+
+// x / L mod 1 for finite x >= 0: the rounded quotient and the quotient of the
+// exact remainder.
+__device__ __forceinline__ Turn turn_fp64(double x, double L) {
+    const double q = __ddiv_rn(x, L), q2 = __ddiv_rn(__fma_rn(-q, L, x), L);
+    const double f = __dsub_rn(q, floor(q)), a = __dmul_rn(f, 281474976710656.0), ai = floor(a);  // 2^48
+    const uint64_t top = uint64_t(ai), mid = uint64_t(__dmul_rn(__dsub_rn(a, ai), 281474976710656.0));
+    // top 2^-48 + mid 2^-96, plus q2 (|q2| < 2^-52) in units of 2^-96
+    const int64_t low = llrint(__dmul_rn(q2, 79228162514264337593543950336.0));
+    const uint64_t m = mid + uint64_t(low);  // 48 bits, and a carry or borrow
+    const int64_t carry = int64_t(m) >> 48;
+    const uint64_t t48 = top + uint64_t(carry), m48 = m & ((uint64_t(1) << 48) - 1u);
+    return Turn{t48 << 16 | m48 >> 32, uint32_t(m48)};
+}
+
+// exp(2 pi i h t): the nearest of 128 table angles and a Taylor polynomial of
+// the remainder (|r| <= pi / 128: r^9 / 9! < 10^-20, r^8 / 8! < 10^-17).
+__device__ __forceinline__ double2 turn_wave(const Turn& t, int h, const double2* table) {
+    const uint64_t p = t.hi * uint64_t(int64_t(h)) + uint64_t((int64_t(t.lo) * int64_t(h)) >> 32);
+    const uint64_t near = p + (uint64_t(1) << 56);
+    const int64_t rem = int64_t(p - (near >> 57 << 57));  // in [-2^56, 2^56)
+    // rem / 2^5 is an integer of 52 bits: exact through the exponent trick
+    const double v = __dsub_rn(__longlong_as_double(0x4338000000000000ll + (rem >> 5)), 6755399441055744.0);  // 1.5 2^52
+    const double r = __dmul_rn(v, 1.0899589056276974e-17);  // 2 pi 2^-59
+    const double z = __dmul_rn(r, r);
+    double s = __fma_rn(z, -1.0 / 5040.0, 1.0 / 120.0);
+    s = __fma_rn(z, s, -1.0 / 6.0);
+    s = __fma_rn(__dmul_rn(z, s), r, r);
+    double c = __fma_rn(z, -1.0 / 720.0, 1.0 / 24.0);
+    c = __fma_rn(z, c, -0.5);
+    c = __dmul_rn(z, c);  // cos r - 1
+    const double2 e = table[near >> 57];
+    return make_double2(__dadd_rn(e.x, __fma_rn(e.x, c, -__dmul_rn(e.y, s))),
+                        __dadd_rn(e.y, __fma_rn(e.y, c, __dmul_rn(e.x, s))));
+}
+
+// blockIdx.x: share of the replica's disks (32 at a time), blockIdx.y: 512 of
+// its wave vectors, blockIdx.z: replica.  comp[r]: its nh distinct h, then its
+// nk distinct k; pair[r][q]: indices of q's components.  With few wave vectors
+// the threads split into groups that take every groups-th disk.
+__global__ void __launch_bounds__(kPairThreads)
+k_sq_pairs(const Rep* __restrict__ reps, bool fixed, int nq, int nh, int nk, const int* __restrict__ comp,
+           const ushort2* __restrict__ pair, const double* __restrict__ xy, double2* __restrict__ part) {
+    pdl_begin();
+    extern __shared__ double2 s_wave[];  // [kPairDisks][nh + nk], then the table
+    __shared__ Turn s_turn[kPairDisks][2];
+    const int r = blockIdx.z, nc = nh + nk, tid = int(threadIdx.x);
+    const Rep& rep = reps[r];
+    double2* table = s_wave + kPairDisks * nc;
+    for (int j = tid; j < kTurnTable; j += kPairThreads) {
+        double s, c;
+        sincospi(double(j) * (2.0 / kTurnTable), &s, &c);
+        table[j] = make_double2(c, s);
+    }
+    const int q0 = blockIdx.y * (kPairThreads * kPairQ), here = min(nq - q0, kPairThreads * kPairQ);
+    int groups = 1;
+    while (groups < 8 && 2 * groups * here <= kPairThreads) groups *= 2;
+    const int width = kPairThreads / groups, group = tid / width, lane = tid - group * width;
+    int ih[kPairQ], ik[kPairQ];
+    bool mine[kPairQ];
+    double re[kPairQ], im[kPairQ];
+#pragma unroll
+    for (int j = 0; j < kPairQ; ++j) {
+        const int q = lane + j * width;
+        mine[j] = q < here;
+        const ushort2 p = mine[j] ? pair[size_t(r) * nq + q0 + q] : make_ushort2(0, 0);
+        ih[j] = p.x;
+        ik[j] = nh + p.y;
+        re[j] = im[j] = 0.0;
+    }
+    const bool second = width < here;  // the second wave vector of a thread is in use
+    const int* cr = comp + size_t(r) * nc;
+    for (int64_t base = int64_t(blockIdx.x) * kPairDisks; base < rep.N; base += int64_t(gridDim.x) * kPairDisks) {
+        __syncthreads();
+        if (tid < 2 * kPairDisks) {
+            const int64_t i = base + (tid >> 1);
+            Turn t{0ull, 0u};
+            if (i < rep.N) {
+                double x = xy[2 * (rep.id_off + i) + (tid & 1)];
+                if (rep.sigma != 1.0) x = __ddiv_rn(x, rep.sigma);
+                t = fixed ? turn_fixed(uint64_t(llrint(__dmul_rn(x, 16777216.0))) % uint64_t(rep.LF), uint64_t(rep.LF))
+                          : turn_fp64(x, rep.Lm);
+            }
+            s_turn[tid >> 1][tid & 1] = t;
+        }
+        __syncthreads();
+        for (int e = tid; e < kPairDisks * nc; e += kPairThreads) {
+            const int n = e / nc, j = e - n * nc;
+            s_wave[e] = base + n < rep.N ? turn_wave(s_turn[n][j >= nh], cr[j], table) : make_double2(0.0, 0.0);
+        }
+        __syncthreads();
+        for (int n = group; n < kPairDisks; n += groups) {
+            const double2* w = s_wave + n * nc;
+#pragma unroll
+            for (int j = 0; j < kPairQ; ++j) {
+                if (j == 1 && !second) break;
+                const double2 u = w[ih[j]], v = w[ik[j]];
+                re[j] = __fma_rn(u.x, v.x, re[j]);
+                im[j] = __fma_rn(u.x, v.y, im[j]);
+                re[j] = __fma_rn(-u.y, v.y, re[j]);
+                im[j] = __fma_rn(u.y, v.x, im[j]);
+            }
+        }
+    }
+    // the groups' sums in order (the waves' space is free: 2 KB at least)
+    __syncthreads();
+    double2* s_sum = s_wave;
+    for (int g = 1; g < groups; ++g) {
+        if (group == g && mine[0]) s_sum[lane] = make_double2(re[0], im[0]);
+        __syncthreads();
+        if (group == 0 && mine[0]) {
+            re[0] = __dadd_rn(re[0], s_sum[lane].x);
+            im[0] = __dadd_rn(im[0], s_sum[lane].y);
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int j = 0; j < kPairQ; ++j)
+        if (group == 0 && mine[j])
+            part[(size_t(r) * gridDim.x + blockIdx.x) * nq + q0 + lane + j * width] = make_double2(re[j], im[j]);
+}
+
+// S_r(q) = |A_r(q)|^2 / N_r (Eq. 10) from the partial sums: blockIdx.y =
+// replica, 32 wave vectors per block, eight threads to each, whose sums are
+// added in order (one thread per wave vector over all partial sums ran a
+// serial chain: 134 us for 256 partial sums of 441 wave vectors, 6 here).
 __global__ void __launch_bounds__(256)
-k_sq_reduce(const Rep* __restrict__ reps, int nq, int nbx, const double2* __restrict__ part, double* __restrict__ S,
-            int* __restrict__ best) {
+k_sq_sum(const Rep* __restrict__ reps, int nq, int nbx, bool by_disks, const double2* __restrict__ part,
+         double* __restrict__ S) {
+    pdl_begin();
+    __shared__ double2 s_v[8][32];
+    const int r = blockIdx.y, lane = int(threadIdx.x & 31u), row = int(threadIdx.x >> 5);
+    const int q = blockIdx.x * 32 + lane;
+    const int nb = by_disks ? int((reps[r].N + 255) / 256) : nbx;  // blocks that hold disks of this replica
+    double a = 0.0, b = 0.0;
+    if (q < nq)
+        for (int x = row; x < nb; x += 8) {
+            const double2 p = part[(size_t(r) * nbx + x) * nq + q];
+            a = __dadd_rn(a, p.x);
+            b = __dadd_rn(b, p.y);
+        }
+    s_v[row][lane] = make_double2(a, b);
+    __syncthreads();
+    if (row == 0 && q < nq) {
+        for (int w = 1; w < 8; ++w) {
+            a = __dadd_rn(a, s_v[w][lane].x);
+            b = __dadd_rn(b, s_v[w][lane].y);
+        }
+        S[size_t(r) * nq + q] = __ddiv_rn(__dadd_rn(__dmul_rn(a, a), __dmul_rn(b, b)), double(reps[r].N));
+    }
+}
+
+// best[r] = first q of largest S_r(q).  One block per replica.
+__global__ void __launch_bounds__(256)
+k_sq_best(int nq, const double* __restrict__ S, int* __restrict__ best) {
     pdl_begin();
     const int r = blockIdx.x;
-    const Rep& rep = reps[r];
-    const int nb = int((rep.N + 255) / 256);
     __shared__ double s_v[256];
     __shared__ int s_i[256];
     double bv = -1.0;
     int bi = 0;
     for (int q = threadIdx.x; q < nq; q += blockDim.x) {
-        double a = 0.0, b = 0.0;
-        for (int x = 0; x < nb; ++x) {
-            const double2 p = part[(size_t(r) * nbx + x) * nq + q];
-            a += p.x;
-            b += p.y;
-        }
-        const double v = __ddiv_rn(__dadd_rn(__dmul_rn(a, a), __dmul_rn(b, b)), double(rep.N));
-        S[size_t(r) * nq + q] = v;
+        const double v = S[size_t(r) * nq + q];
         if (v > bv) {
             bv = v;
             bi = q;
@@ -307,11 +485,12 @@ k_sq_reduce(const Rep* __restrict__ reps, int nq, int nbx, const double2* __rest
 // around the first-shell reciprocal vector of a triangular lattice of the
 // same density (|q| = 4 pi / (a sqrt 3), area per disk sqrt(3) a^2 / 2) at
 // the angle arg(Psi_6) / 6 + 30 degrees.  psi[2r], psi[2r + 1] = Psi_6.
-__global__ void k_q0_window(const Rep* __restrict__ reps, int R, int hw, const double* __restrict__ psi,
-                            int2* __restrict__ hk) {
+// One block per replica; comp and pair as k_sq_pairs takes them (nullable).
+__global__ void __launch_bounds__(128)
+k_q0_window(const Rep* __restrict__ reps, int hw, const double* __restrict__ psi, int2* __restrict__ hk,
+            int* __restrict__ comp, ushort2* __restrict__ pair) {
     pdl_begin();
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= R) return;
+    const int r = blockIdx.x;
     const Rep& rep = reps[r];
     const double L = rep.Lm;
     const double eta = __ddiv_rn(__dmul_rn(double(rep.N), CUDART_PI), __dmul_rn(L, L));
@@ -323,8 +502,13 @@ __global__ void k_q0_window(const Rep* __restrict__ reps, int R, int hw, const d
     const int hc = int(rint(__dmul_rn(__dmul_rn(qmag, cos(th)), scale)));
     const int kc = int(rint(__dmul_rn(__dmul_rn(qmag, sin(th)), scale)));
     const int w = 2 * hw + 1;
-    for (int dh = 0; dh < w; ++dh)
-        for (int dk = 0; dk < w; ++dk) hk[size_t(r) * w * w + dh * w + dk] = make_int2(hc - hw + dh, kc - hw + dk);
+    for (int q = threadIdx.x; q < w * w; q += blockDim.x) {
+        const int dh = q / w, dk = q - dh * w;
+        hk[size_t(r) * w * w + q] = make_int2(hc - hw + dh, kc - hw + dk);
+        if (pair) pair[size_t(r) * w * w + q] = make_ushort2((unsigned short)dh, (unsigned short)dk);
+    }
+    if (comp)
+        for (int j = threadIdx.x; j < 2 * w; j += blockDim.x) comp[size_t(r) * 2 * w + j] = j < w ? hc - hw + j : kc - hw + j - w;
 }
 
 // chi_j = exp(i q_0 . x_j) (Eq. 11), by global disk id.
@@ -462,17 +646,49 @@ int sq_disk_blocks(const std::vector<int64_t>& N) {
     return int(b);
 }
 
+bool sq_pairs_fit(int nh, int nk, int nq) {
+    // fewer FP64 operations than a plane wave per wave vector and disk
+    return nh + nk <= kPairMax && nh <= 65535 && 15 * (nh + nk) + 4 * nq < 60 * nq;
+}
+
+int sq_pair_blocks(int R, int nq, const std::vector<int64_t>& N) {
+    // two blocks per SM (152) over all replicas and tiles of wave vectors
+    const int64_t tiles = int64_t(R) * ((nq + kPairThreads * kPairQ - 1) / (kPairThreads * kPairQ));
+    int64_t most = 1;
+    for (int64_t n : N) most = std::max<int64_t>(most, (n + kPairDisks - 1) / kPairDisks);
+    return int(std::max<int64_t>(1, std::min<int64_t>(most, (304 + tiles - 1) / tiles)));
+}
+
 cudaError_t launch_sq(const LaunchCfg& c, int nq, const int2* hk, const double* xy, int nbx, double2* part, double* S,
                       int* best) {
     const dim3 grid(unsigned(nbx), unsigned((nq + kSqChunk - 1) / kSqChunk), unsigned(c.R));
-    const cudaError_t e = launch_k(k_sq_amp, grid, dim3(256), 0, c.stream, c.reps, c.fixed, nq, hk, xy, nbx, part);
-    if (e != cudaSuccess) return e;
-    return launch_k(k_sq_reduce, dim3(unsigned(c.R)), dim3(256), 0, c.stream, c.reps, nq, nbx, (const double2*)part, S,
-                    best);
+    cudaError_t e = launch_k(k_sq_amp, grid, dim3(256), 0, c.stream, c.reps, c.fixed, nq, hk, xy, nbx, part);
+    if (e == cudaSuccess)
+        e = launch_k(k_sq_sum, dim3(unsigned((nq + 31) / 32), unsigned(c.R)), dim3(256), 0, c.stream, c.reps, nq, nbx, true,
+                     (const double2*)part, S);
+    if (e == cudaSuccess && best) e = launch_k(k_sq_best, dim3(unsigned(c.R)), dim3(256), 0, c.stream, nq, (const double*)S, best);
+    return e;
 }
 
-cudaError_t launch_q0_window(const LaunchCfg& c, int hw, const double* psi, int2* hk) {
-    return launch_k(k_q0_window, dim3(unsigned((c.R + 31) / 32)), dim3(32), 0, c.stream, c.reps, c.R, hw, psi, hk);
+cudaError_t launch_sq_pairs(const LaunchCfg& c, int nq, int nh, int nk, const int* comp, const ushort2* pair,
+                            const double* xy, int nbx, double2* part, double* S, int* best) {
+    static std::once_flag attr_once;
+    std::call_once(attr_once, [] {
+        cudaFuncSetAttribute(k_sq_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             int((kPairDisks * kPairMax + kTurnTable) * sizeof(double2)));
+    });
+    const dim3 grid(unsigned(nbx), unsigned((nq + kPairThreads * kPairQ - 1) / (kPairThreads * kPairQ)), unsigned(c.R));
+    cudaError_t e = launch_k(k_sq_pairs, grid, dim3(kPairThreads), size_t(kPairDisks * (nh + nk) + kTurnTable) * sizeof(double2),
+                             c.stream, c.reps, c.fixed, nq, nh, nk, comp, pair, xy, part);
+    if (e == cudaSuccess)
+        e = launch_k(k_sq_sum, dim3(unsigned((nq + 31) / 32), unsigned(c.R)), dim3(256), 0, c.stream, c.reps, nq, nbx, false,
+                     (const double2*)part, S);
+    if (e == cudaSuccess && best) e = launch_k(k_sq_best, dim3(unsigned(c.R)), dim3(256), 0, c.stream, nq, (const double*)S, best);
+    return e;
+}
+
+cudaError_t launch_q0_window(const LaunchCfg& c, int hw, const double* psi, int2* hk, int* comp, ushort2* pair) {
+    return launch_k(k_q0_window, dim3(unsigned(c.R)), dim3(128), 0, c.stream, c.reps, hw, psi, hk, comp, pair);
 }
 
 cudaError_t launch_chi(const LaunchCfg& c, int64_t Ntot, const int2* hk0, const double* xy, double2* chi) {

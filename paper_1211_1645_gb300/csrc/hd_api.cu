@@ -86,6 +86,9 @@ struct hd_ctx {
     double* sq_S = nullptr;         // [R][nq]
     int* sq_best = nullptr;         // [R]
     size_t sq_cap = 0, sq_S_cap = 0, sq_part_cap = 0;  // capacities of sq_hk, sq_S, sq_part
+    int* sq_comp = nullptr;         // [R][nh + nk] distinct components of the wave vectors
+    ushort2* sq_pair = nullptr;     // [R][nq] their indices
+    size_t sq_comp_cap = 0, sq_pair_cap = 0;
     double2* chi = nullptr;         // [Ntot] positional order by disk id
     double* corr_acc = nullptr;     // [R][nr][3]
     double2* corr = nullptr;        // [R][nr]
@@ -464,7 +467,7 @@ void free_ctx(hd_ctx* ctx) {
     if (ctx->tau) cudaFree(ctx->tau);
     if (ctx->field_acc) cudaFree(ctx->field_acc);
     if (ctx->field) cudaFree(ctx->field);
-    for (void* q : {(void*)ctx->sq_hk, (void*)ctx->sq_part, (void*)ctx->sq_S, (void*)ctx->sq_best, (void*)ctx->chi,
+    for (void* q : {(void*)ctx->sq_hk, (void*)ctx->sq_comp, (void*)ctx->sq_pair, (void*)ctx->sq_part, (void*)ctx->sq_S, (void*)ctx->sq_best, (void*)ctx->chi,
                     (void*)ctx->corr_acc, (void*)ctx->corr})
         if (q) cudaFree(q);
     if (ctx->series_len) cudaFree(ctx->series_len);
@@ -1797,14 +1800,18 @@ hd_status grow(hd_ctx* ctx, T*& p, size_t& cap, size_t need) {
     return HD_OK;
 }
 
-// S at the wave vectors already in ctx->sq_hk ([R][nq]); positions refreshed first.
-hd_status enqueue_sq(hd_ctx* ctx, int nq) {
+// S at the wave vectors already in ctx->sq_hk ([R][nq]), or with nh > 0 of the
+// components and pairs already in ctx->sq_comp and ctx->sq_pair; positions
+// refreshed first.
+hd_status enqueue_sq(hd_ctx* ctx, int nq, int nh, int nk, bool want_best) {
     std::vector<int64_t> Ns;
     for (const Rep& r : ctx->reps) Ns.push_back(r.N);
-    const int nbx = hd::sq_disk_blocks(Ns);
-    const size_t need = size_t(ctx->R) * size_t(nbx) * size_t(nq);
-    if (need > (size_t(1) << 27)) return HD_ERR_ARG;
-    hd_status st = grow(ctx, ctx->sq_part, ctx->sq_part_cap, need);
+    // (the bound on the partial sums of one plane wave per wave vector and
+    // disk, which decides what the call accepts)
+    const size_t bound = size_t(ctx->R) * size_t(hd::sq_disk_blocks(Ns)) * size_t(nq);
+    if (bound > (size_t(1) << 27)) return HD_ERR_ARG;
+    const int nbx = nh > 0 ? hd::sq_pair_blocks(ctx->R, nq, Ns) : hd::sq_disk_blocks(Ns);
+    hd_status st = grow(ctx, ctx->sq_part, ctx->sq_part_cap, size_t(ctx->R) * size_t(nbx) * size_t(nq));
     if (st != HD_OK) return st;
     st = grow(ctx, ctx->sq_S, ctx->sq_S_cap, size_t(ctx->R) * nq);
     if (st != HD_OK) return st;
@@ -1813,9 +1820,46 @@ hd_status enqueue_sq(hd_ctx* ctx, int nq) {
         return hd::launch_positions(ctx->cfg(), ctx->frame, ctx->buf[ctx->cur], ctx->xy);
     }));
     HD_CK(ctx, launch(ctx, HD_K_ANALYSIS, [&] {
-        return hd::launch_sq(ctx->cfg(), nq, ctx->sq_hk, ctx->xy, nbx, ctx->sq_part, ctx->sq_S, ctx->sq_best);
+        int* best = want_best ? ctx->sq_best : nullptr;
+        if (nh > 0)
+            return hd::launch_sq_pairs(ctx->cfg(), nq, nh, nk, ctx->sq_comp, ctx->sq_pair, ctx->xy, nbx, ctx->sq_part, ctx->sq_S,
+                                       best);
+        return hd::launch_sq(ctx->cfg(), nq, ctx->sq_hk, ctx->xy, nbx, ctx->sq_part, ctx->sq_S, best);
     }));
     return HD_OK;
+}
+
+// The distinct components of each replica's wave vectors, padded to the
+// largest count, and each wave vector's indices; false where the lists share
+// too few of them.
+bool sq_components(int R, int nq, const int32_t* hk, int& nh, int& nk, std::vector<int>& comp, std::vector<ushort2>& pair) {
+    std::vector<std::vector<int>> h(static_cast<size_t>(R)), k(static_cast<size_t>(R));
+    nh = nk = 1;
+    for (int r = 0; r < R; ++r) {
+        for (int c = 0; c < 2; ++c) {
+            std::vector<int>& v = c == 0 ? h[size_t(r)] : k[size_t(r)];
+            v.resize(size_t(nq));
+            for (int q = 0; q < nq; ++q) v[size_t(q)] = hk[2 * (size_t(r) * nq + size_t(q)) + size_t(c)];
+            std::sort(v.begin(), v.end());
+            v.erase(std::unique(v.begin(), v.end()), v.end());
+        }
+        nh = std::max(nh, int(h[size_t(r)].size()));
+        nk = std::max(nk, int(k[size_t(r)].size()));
+        if (!hd::sq_pairs_fit(nh, nk, nq)) return false;
+    }
+    comp.assign(size_t(R) * size_t(nh + nk), 0);
+    pair.resize(size_t(R) * size_t(nq));
+    for (int r = 0; r < R; ++r) {
+        const std::vector<int>&hr = h[size_t(r)], &kr = k[size_t(r)];
+        std::copy(hr.begin(), hr.end(), comp.begin() + size_t(r) * size_t(nh + nk));
+        std::copy(kr.begin(), kr.end(), comp.begin() + size_t(r) * size_t(nh + nk) + size_t(nh));
+        for (int q = 0; q < nq; ++q) {
+            const size_t at = size_t(r) * nq + size_t(q);
+            pair[at].x = (unsigned short)(std::lower_bound(hr.begin(), hr.end(), hk[2 * at]) - hr.begin());
+            pair[at].y = (unsigned short)(std::lower_bound(kr.begin(), kr.end(), hk[2 * at + 1]) - kr.begin());
+        }
+    }
+    return true;
 }
 
 }  // namespace
@@ -1824,10 +1868,23 @@ hd_status hd_structure_factor(hd_ctx* ctx, int32_t nq, const int32_t* hk, double
     const Range range("hd_structure_factor");
     if (!ctx || !hk || !S || nq < 1 || nq > 65536) return HD_ERR_ARG;
     if (ctx->sticky != HD_OK) return HD_ERR_STATE;
-    hd_status st = grow(ctx, ctx->sq_hk, ctx->sq_cap, size_t(ctx->R) * nq);
-    if (st != HD_OK) return st;
-    HD_CK(ctx, cudaMemcpyAsync(ctx->sq_hk, hk, sizeof(int2) * size_t(ctx->R) * nq, cudaMemcpyHostToDevice, ctx->stream));
-    st = enqueue_sq(ctx, nq);
+    int nh = 0, nk = 0;
+    std::vector<int> comp;
+    std::vector<ushort2> pair;
+    hd_status st;
+    if (sq_components(ctx->R, nq, hk, nh, nk, comp, pair)) {
+        st = grow(ctx, ctx->sq_comp, ctx->sq_comp_cap, comp.size());
+        if (st == HD_OK) st = grow(ctx, ctx->sq_pair, ctx->sq_pair_cap, pair.size());
+        if (st != HD_OK) return st;
+        HD_CK(ctx, cudaMemcpyAsync(ctx->sq_comp, comp.data(), comp.size() * sizeof(int), cudaMemcpyHostToDevice, ctx->stream));
+        HD_CK(ctx, cudaMemcpyAsync(ctx->sq_pair, pair.data(), pair.size() * sizeof(ushort2), cudaMemcpyHostToDevice, ctx->stream));
+    } else {
+        nh = 0;
+        st = grow(ctx, ctx->sq_hk, ctx->sq_cap, size_t(ctx->R) * nq);
+        if (st != HD_OK) return st;
+        HD_CK(ctx, cudaMemcpyAsync(ctx->sq_hk, hk, sizeof(int2) * size_t(ctx->R) * nq, cudaMemcpyHostToDevice, ctx->stream));
+    }
+    st = enqueue_sq(ctx, nq, nh, nk, false);
     if (st != HD_OK) return st;
     HD_CK(ctx, cudaMemcpyAsync(S, ctx->sq_S, sizeof(double) * size_t(ctx->R) * nq, cudaMemcpyDeviceToHost, ctx->stream));
     HD_CK(ctx, cudaStreamSynchronize(ctx->stream));
@@ -1842,8 +1899,17 @@ hd_status hd_positional_q0(hd_ctx* ctx, int32_t half_width, int32_t* hk0, double
     hd_status st = grow(ctx, ctx->sq_hk, ctx->sq_cap, size_t(ctx->R) * nq);
     if (st != HD_OK) return st;
     HD_CK(ctx, enqueue_psi6(ctx, ctx->stream, false, false));  // Psi_6 orients the window
-    HD_CK(ctx, launch(ctx, HD_K_ANALYSIS, [&] { return hd::launch_q0_window(ctx->cfg(), half_width, ctx->psi_res, ctx->sq_hk); }));
-    st = enqueue_sq(ctx, nq);
+    const bool pairs = hd::sq_pairs_fit(w, w, nq);
+    if (pairs) {
+        st = grow(ctx, ctx->sq_comp, ctx->sq_comp_cap, size_t(ctx->R) * size_t(2 * w));
+        if (st == HD_OK) st = grow(ctx, ctx->sq_pair, ctx->sq_pair_cap, size_t(ctx->R) * nq);
+        if (st != HD_OK) return st;
+    }
+    HD_CK(ctx, launch(ctx, HD_K_ANALYSIS, [&] {
+        return hd::launch_q0_window(ctx->cfg(), half_width, ctx->psi_res, ctx->sq_hk, pairs ? ctx->sq_comp : nullptr,
+                                    pairs ? ctx->sq_pair : nullptr);
+    }));
+    st = enqueue_sq(ctx, nq, pairs ? w : 0, w, true);
     if (st != HD_OK) return st;
     std::vector<int2> win(size_t(ctx->R) * nq);
     std::vector<int> best(size_t(ctx->R));
