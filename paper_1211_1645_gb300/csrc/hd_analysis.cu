@@ -13,6 +13,7 @@
 
 #include "hd_kernels.h"
 #include "hd_analysis.h"
+#include "hd_cell.cuh"
 
 namespace hd {
 
@@ -594,6 +595,216 @@ k_poscorr(const Rep* __restrict__ reps, int R, const uint8_t* __restrict__ cnt, 
         if (s_acc[k] != 0.0) atomicAdd(&acc[size_t(r) * 3 * nr + k], s_acc[k]);
 }
 
+// ---------------------------------------------------------------------------
+// The same correlation from unordered pairs, one disk per thread.  A pair is in
+// the windows k with b <= k < a, where a counts the windows whose lower bound
+// is at most d^2 and b those whose upper bound is below it, so one addition to
+// the elementary interval a + b stands for all its windows; the imaginary
+// parts of a pair's two orders cancel exactly.  Every thread keeps its own sums
+// per interval in shared memory (interval-major: no two lanes share a bank), so
+// nothing is atomic until a block's sums are added up.  a and b come from a
+// float estimate of the distance in the cell frame; a pair whose estimate lies
+// within its error bound of a window's edge takes the FP64 comparisons of
+// k_poscorr on the global positions.  Three FP64 operations per pair remain.
+// N = 16,384, 40 windows of 0.5 out to 20 sigma: 13.3 ms with a division, two
+// square roots' worth of FP64 and a dozen shared FP64 atomics per ordered pair,
+// 0.25 here.
+// ---------------------------------------------------------------------------
+constexpr size_t kCorrSmem = 112 * 1024;  // two blocks per SM at least
+constexpr size_t kCorrBytes = 12;         // a thread's sum and count of one interval
+
+// Threads per block whose interval sums fit, 0 if not even a warp's do.
+__host__ __device__ constexpr int corr_threads(int nr) {
+    return size_t(2 * nr + 1) * kCorrBytes * 128 <= kCorrSmem ? 128
+           : size_t(2 * nr + 1) * kCorrBytes * 64 <= kCorrSmem ? 64
+           : size_t(2 * nr + 1) * kCorrBytes * 32 <= kCorrSmem ? 32 : 0;
+}
+
+// Per slot and cell: the disk's global position (as k_poscorr reads it), its
+// float offset in the cell, and chi.
+template <bool FIX, int CAP>
+__global__ void __launch_bounds__(256)
+k_corr_stage(const Rep* __restrict__ reps, const Frame* __restrict__ cur, const uint8_t* __restrict__ cnt,
+             const P2<FIX>* __restrict__ pos, const int2* __restrict__ hk0, double2* __restrict__ gpos,
+             double2* __restrict__ chi, float2* __restrict__ off) {
+    pdl_begin();
+    const int r = blockIdx.y;
+    const Rep& rep = reps[r];
+    const int m = rep.m;
+    const uint32_t a = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a >= uint32_t(m) * uint32_t(m)) return;
+    int cx, cy;
+    cell_coords(rep, a, cx, cy);
+    const Frame f = cur[r];
+    const uint32_t cell = rep.coff + a;
+    const int n = min(int(cnt[cell]), CAP);
+    for (int k = 0; k < n; ++k) {
+        const size_t at = size_t(k) * rep.stride32 + cell;
+        const P2<FIX> q = pos[at];
+        double X, Y;
+        global_position<FIX>(rep, f, cx, cy, q, X, Y);
+        if (rep.sigma != 1.0) {
+            X = __ddiv_rn(__dmul_rn(X, rep.sigma), rep.sigma);
+            Y = __ddiv_rn(__dmul_rn(Y, rep.sigma), rep.sigma);
+        }
+        gpos[at] = make_double2(X, Y);
+        chi[at] = plane_wave(rep, FIX, hk0[r].x, hk0[r].y, X, Y);
+        if constexpr (FIX) off[at] = make_float2(__fmul_rn(__int2float_rn(q.x), 0x1p-24f), __fmul_rn(__int2float_rn(q.y), 0x1p-24f));
+        else off[at] = make_float2(__double2float_rn(q.x), __double2float_rn(q.y));
+    }
+}
+
+// Bounds of window k squared, as k_poscorr compares them.
+__device__ __forceinline__ double corr_lo2(int k, double dr) {
+    const double rk = __dmul_rn(double(k + 1), dr), lo = rk > 1.0 ? __dsub_rn(rk, 1.0) : 0.0;
+    return __dmul_rn(lo, lo);
+}
+__device__ __forceinline__ double corr_hi2(int k, double dr) {
+    const double hi = __dadd_rn(__dmul_rn(double(k + 1), dr), 1.0);
+    return __dmul_rn(hi, hi);
+}
+
+// a and b of a pair by the FP64 comparisons, from a guess.
+static __device__ __noinline__ int2 corr_exact(double2 pn, double2 pm, double L, int nr, double dr, int a, int b) {
+    double dx = __dsub_rn(pm.x, pn.x), dy = __dsub_rn(pm.y, pn.y);
+    dx = __dsub_rn(dx, __dmul_rn(L, rint(__ddiv_rn(dx, L))));
+    dy = __dsub_rn(dy, __dmul_rn(L, rint(__ddiv_rn(dy, L))));
+    const double d2 = __dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy));
+    while (a < nr && corr_lo2(a, dr) <= d2) ++a;
+    while (a > 0 && corr_lo2(a - 1, dr) > d2) --a;
+    while (b < nr && corr_hi2(b, dr) < d2) ++b;
+    while (b > 0 && corr_hi2(b - 1, dr) >= d2) --b;
+    return make_int2(a, b);
+}
+
+// blockIdx.y: replica, blockIdx.x: cells_per_block of its cells (planar order).
+// acc[r][interval] = (sum of Re, pairs).
+template <int CAP, int NT>
+__global__ void __launch_bounds__(NT)
+k_corr_pairs(const Rep* __restrict__ reps, const uint8_t* __restrict__ cnt, const double2* __restrict__ gpos,
+             const double2* __restrict__ chi, const float2* __restrict__ off, int nr, double dr, int reach,
+             int cells_per_block, double2* __restrict__ acc) {
+    extern __shared__ double s_sum[];  // [2 nr + 1][NT], then the counts
+    const int bins = 2 * nr + 1;
+    uint32_t* s_cnt = reinterpret_cast<uint32_t*>(s_sum + size_t(bins) * NT);
+    __shared__ uint16_t s_list[NT * CAP];
+    __shared__ int s_n;
+    pdl_begin();
+    const int r = blockIdx.y, tid = int(threadIdx.x);
+    const Rep& rep = reps[r];
+    const int m = rep.m;
+    const uint32_t mm = uint32_t(m) * uint32_t(m), a0 = blockIdx.x * uint32_t(cells_per_block);
+    if (a0 >= mm) return;
+    for (int k = tid; k < bins * NT; k += NT) {
+        s_sum[k] = 0.0;
+        s_cnt[k] = 0;
+    }
+    if (tid == 0) s_n = 0;
+    __syncthreads();
+    // the block's disks, a warp's cells in order
+    for (int c0 = 0; c0 < cells_per_block; c0 += NT) {
+        const uint32_t a = a0 + uint32_t(c0 + tid);
+        const int n = (c0 + tid < cells_per_block && a < mm) ? min(int(cnt[rep.coff + a]), CAP) : 0;
+        int v = n;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, v, o);
+            if ((tid & 31) >= o) v += u;
+        }
+        int base = 0;
+        if ((tid & 31) == 31) base = atomicAdd(&s_n, v);
+        base = __shfl_sync(0xffffffffu, base, 31) + v - n;
+        for (int k = 0; k < n; ++k) s_list[base + k] = uint16_t((c0 + tid) << 4 | k);
+    }
+    __syncthreads();
+    const int disks = s_n;
+    const float wf = float(rep.w), inv = __fdiv_rn(1.0f, float(dr)), rmax = float(nr) * float(dr) + 1.0f;
+    // error of the float distance: the offsets, the cell offset and the
+    // difference each round by at most 2^-24 of the reach, in both components;
+    // four times that, and the roundings of the scaled distance
+    const float eps = (float(reach + 2) * wf * 0x1p-20f + (rmax + 1.0f) * 0x1p-20f) * inv;
+    const double L = rep.Lm;
+    for (int d = tid; d < disks; d += NT) {
+        const uint32_t a = a0 + (s_list[d] >> 4);
+        const int slot = int(s_list[d] & 15u);
+        int cx, cy;
+        cell_coords(rep, a, cx, cy);
+        const size_t me = size_t(slot) * rep.stride32 + rep.coff + a;
+        const float2 un = off[me];
+        const double2 cn = chi[me];
+        for (int dcy = 0; dcy <= reach; ++dcy) {
+            const int y = cy + dcy >= m ? cy + dcy - m : cy + dcy;
+            const uint32_t row = rep.coff + row_part(rep, y);
+            const float gy = fmaxf(float(dcy - 1), 0.0f) * wf;
+            const float by = __fsub_rn(__fmul_rn(float(dcy), wf), un.y);
+            for (int dcx = dcy == 0 ? 0 : -reach; dcx <= reach; ++dcx) {
+                const float gx = fmaxf(fabsf(float(dcx)) - 1.0f, 0.0f) * wf;
+                if (gx * gx + gy * gy > (rmax + 0.01f) * (rmax + 0.01f)) continue;  // no point of the cell is in reach
+                const uint32_t c = row + col_part(rep, wrap_cell(cx + dcx, m));
+                const int n = min(int(cnt[c]), CAP);
+                const float bx = __fsub_rn(__fmul_rn(float(dcx), wf), un.x);
+                for (int q = (dcx == 0 && dcy == 0) ? slot + 1 : 0; q < n; ++q) {
+                    const size_t at = size_t(q) * rep.stride32 + c;
+                    const float2 um = off[at];
+                    const float sx = __fadd_rn(um.x, bx), sy = __fadd_rn(um.y, by);
+                    const float dist = sqrtf(__fadd_rn(__fmul_rn(sx, sx), __fmul_rn(sy, sy)));
+                    const float fu = __fmul_rn(__fadd_rn(dist, 1.0f), inv), fv = __fmul_rn(__fsub_rn(dist, 1.0f), inv);
+                    int wa = int(fminf(floorf(fu), float(nr))), wb = int(fminf(fmaxf(ceilf(fv) - 1.0f, 0.0f), float(nr)));
+                    // (false also where a window width out of float's range made the estimate infinite)
+                    const bool sure = eps < 0.25f && fabsf(fu - rintf(fu)) >= eps && fabsf(fv - rintf(fv)) >= eps;
+                    if (!sure) {
+                        const int2 e = corr_exact(gpos[me], gpos[at], L, nr, dr, wa, wb);
+                        wa = e.x;
+                        wb = e.y;
+                    }
+                    if (wa <= wb) continue;
+                    const double2 cm = chi[at];
+                    const int s = (wa + wb) * NT + tid;
+                    s_sum[s] = __dadd_rn(s_sum[s], __fma_rn(cn.x, cm.x, __dmul_rn(cn.y, cm.y)));
+                    s_cnt[s] += 1u;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    for (int b = tid >> 5; b < bins; b += NT / 32) {
+        double v = 0.0;
+        uint32_t c = 0u;
+        for (int t = tid & 31; t < NT; t += 32) {
+            v = __dadd_rn(v, s_sum[b * NT + t]);
+            c += s_cnt[b * NT + t];
+        }
+        c = __reduce_add_sync(0xffffffffu, c);
+        v = lane_sum(v);
+        if ((tid & 31) == 0 && c > 0u) {
+            double2* o = acc + size_t(r) * bins + b;
+            atomicAdd(&o->x, v);
+            atomicAdd(&o->y, double(c));
+        }
+    }
+}
+
+// C(r_k): the intervals with b <= k < a.  The pair (a, b) of interval s follows
+// from merging the windows' lower and upper bounds (at a tie the lower one
+// first: d^2 on both is above the lower and not above the upper).
+__global__ void __launch_bounds__(128)
+k_corr_windows(int nr, double dr, const double2* __restrict__ acc, double2* __restrict__ out) {
+    pdl_begin();
+    const int r = blockIdx.y, k = int(blockIdx.x * blockDim.x + threadIdx.x);
+    if (k >= nr) return;
+    const double2* p = acc + size_t(r) * (2 * nr + 1);
+    double s = 0.0, c = 0.0;
+    int a = 0, b = 0;
+    for (int i = 0; i <= 2 * nr; ++i) {
+        if (b <= k && k < a) {
+            s = __dadd_rn(s, p[i].x);
+            c = __dadd_rn(c, p[i].y);
+        }
+        if (a < nr && (b >= nr || corr_lo2(a, dr) <= corr_hi2(b, dr))) ++a; else ++b;
+    }
+    out[size_t(r) * nr + k] = c > 0.0 ? make_double2(__ddiv_rn(s, c), 0.0) : make_double2(CUDART_NAN, CUDART_NAN);
+}
+
 __global__ void __launch_bounds__(256)
 k_corr_norm(int64_t n, const double* __restrict__ acc, double2* __restrict__ out) {
     pdl_begin();
@@ -706,6 +917,61 @@ static cudaError_t poscorr_t(const LaunchCfg& c, CellBufs cells, const double* x
     });
     return launch_k(k_poscorr<CAP>, dim3(c.blocks_cell), dim3(c.threads), size_t(3 * nr) * sizeof(double), c.stream,
                     c.reps, c.R, (const uint8_t*)cells.cnt, (const int32_t*)cells.pid, xy, chi, nr, dr, reach, acc);
+}
+
+bool corr_pairs_fit(int nr) { return corr_threads(nr) > 0; }
+size_t corr_pairs_acc(int R, int nr) { return size_t(R) * size_t(2 * nr + 1) * 2; }
+
+template <bool FIX, int CAP>
+static cudaError_t corr_stage_t(const LaunchCfg& c, unsigned cells, const Frame* cur, CellBufs b, const int2* hk0, double2* gpos,
+                                double2* chi, float2* off) {
+    return launch_k(k_corr_stage<FIX, CAP>, dim3((cells + 255) / 256, unsigned(c.R)), dim3(256), 0, c.stream, c.reps, cur,
+                    (const uint8_t*)b.cnt, (const P2<FIX>*)b.pos, hk0, gpos, chi, off);
+}
+
+template <int CAP, int NT>
+static cudaError_t corr_pairs_t(const LaunchCfg& c, unsigned cells, CellBufs b, const double2* gpos, const double2* chi,
+                                const float2* off, int nr, double dr, int reach, double2* acc) {
+    static std::once_flag attr_once;
+    std::call_once(attr_once, [] {
+        cudaFuncSetAttribute(k_corr_pairs<CAP, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCorrSmem));
+    });
+    // a little under one cell per thread: at liquid densities a block's disks
+    // are then a single round of its threads
+    const int cells_per_block = NT * 7 / 8;
+    return launch_k(k_corr_pairs<CAP, NT>, dim3((cells + cells_per_block - 1) / cells_per_block, unsigned(c.R)), dim3(NT),
+                    size_t(2 * nr + 1) * kCorrBytes * NT, c.stream, c.reps, (const uint8_t*)b.cnt, gpos, chi, off, nr, dr, reach,
+                    cells_per_block, acc);
+}
+
+template <int CAP>
+static cudaError_t corr_pairs_nt(const LaunchCfg& c, unsigned cells, CellBufs b, const double2* gpos, const double2* chi,
+                                 const float2* off, int nr, double dr, int reach, double2* acc) {
+    switch (corr_threads(nr)) {
+        case 128: return corr_pairs_t<CAP, 128>(c, cells, b, gpos, chi, off, nr, dr, reach, acc);
+        case 64: return corr_pairs_t<CAP, 64>(c, cells, b, gpos, chi, off, nr, dr, reach, acc);
+        case 32: return corr_pairs_t<CAP, 32>(c, cells, b, gpos, chi, off, nr, dr, reach, acc);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t launch_corr_pairs(const LaunchCfg& c, int64_t most_cells, const Frame* cur, CellBufs cells, const int2* hk0,
+                              double2* gpos, double2* chi, float2* off, int nr, double dr, int reach, double* acc,
+                              double2* out) {
+    const unsigned n = unsigned(most_cells);
+    double2* sums = reinterpret_cast<double2*>(acc);
+    cudaError_t e = cudaMemsetAsync(acc, 0, corr_pairs_acc(c.R, nr) * sizeof(double), c.stream);
+    if (e == cudaSuccess)
+        e = c.fixed ? (c.cap == 4 ? corr_stage_t<true, 4>(c, n, cur, cells, hk0, gpos, chi, off)
+                                  : corr_stage_t<true, 9>(c, n, cur, cells, hk0, gpos, chi, off))
+                    : (c.cap == 4 ? corr_stage_t<false, 4>(c, n, cur, cells, hk0, gpos, chi, off)
+                                  : corr_stage_t<false, 9>(c, n, cur, cells, hk0, gpos, chi, off));
+    if (e == cudaSuccess)
+        e = c.cap == 4 ? corr_pairs_nt<4>(c, n, cells, gpos, chi, off, nr, dr, reach, sums)
+                       : corr_pairs_nt<9>(c, n, cells, gpos, chi, off, nr, dr, reach, sums);
+    if (e != cudaSuccess) return e;
+    return launch_k(k_corr_windows, dim3(unsigned((nr + 127) / 128), unsigned(c.R)), dim3(128), 0, c.stream, nr, dr,
+                    (const double2*)sums, out);
 }
 
 cudaError_t launch_poscorr(const LaunchCfg& c, CellBufs cells, const double* xy, const double2* chi, int nr, double dr,

@@ -28,4 +28,15 @@ cudaError_t launch_chi(const LaunchCfg& c, int64_t Ntot, const int2* hk0, const 
 cudaError_t launch_poscorr(const LaunchCfg& c, CellBufs cells, const double* xy, const double2* chi, int nr, double dr,
                            int reach, double* acc, double2* out);
 
+// The same from unordered pairs, for the windows whose sums fit shared memory
+// (corr_pairs_fit) and a reach that holds the largest window with a cell to
+// spare.  most_cells: of one
+// replica; gpos, chi, off: one entry per slot of the cell arrays; acc:
+// corr_pairs_acc doubles.
+bool corr_pairs_fit(int nr);
+size_t corr_pairs_acc(int R, int nr);
+cudaError_t launch_corr_pairs(const LaunchCfg& c, int64_t most_cells, const Frame* cur, CellBufs cells, const int2* hk0,
+                              double2* gpos, double2* chi, float2* off, int nr, double dr, int reach, double* acc,
+                              double2* out);
+
 }  // namespace hd

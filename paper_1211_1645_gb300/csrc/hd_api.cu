@@ -93,6 +93,8 @@ struct hd_ctx {
     double* corr_acc = nullptr;     // [R][nr][3]
     double2* corr = nullptr;        // [R][nr]
     size_t corr_cap = 0;
+    double2* corr_stage = nullptr;  // per slot: global positions, chi, then float offsets
+    size_t corr_stage_cap = 0;
     int tile = 48;
     double sigma = 1.0;
     std::vector<Rep> reps;
@@ -468,7 +470,7 @@ void free_ctx(hd_ctx* ctx) {
     if (ctx->field_acc) cudaFree(ctx->field_acc);
     if (ctx->field) cudaFree(ctx->field);
     for (void* q : {(void*)ctx->sq_hk, (void*)ctx->sq_comp, (void*)ctx->sq_pair, (void*)ctx->sq_part, (void*)ctx->sq_S, (void*)ctx->sq_best, (void*)ctx->chi,
-                    (void*)ctx->corr_acc, (void*)ctx->corr})
+                    (void*)ctx->corr_acc, (void*)ctx->corr, (void*)ctx->corr_stage})
         if (q) cudaFree(q);
     if (ctx->series_len) cudaFree(ctx->series_len);
     for (cudaEvent_t e : ctx->ev) cudaEventDestroy(e);
@@ -1982,8 +1984,16 @@ hd_status hd_positional_corr(hd_ctx* ctx, const int32_t* hk0, int32_t nr, double
     for (const Rep& r : ctx->reps) reach = std::max(reach, int(std::ceil(rmax / r.w)) + 1);
     for (const Rep& r : ctx->reps)
         if (2 * reach + 1 > r.m) return HD_ERR_REACH;
-    hd_status st = enqueue_chi(ctx, hk0);
-    if (st != HD_OK) return st;
+    // the pair kernel takes distances in the cell frame, which are the minimum
+    // image's up to half the box: the windows (r in units of sigma) end a cell
+    // short of the reach
+    bool pairs = hd::corr_pairs_fit(nr);
+    for (const Rep& r : ctx->reps) pairs = pairs && double(nr) * (dr / ctx->sigma) + 1.0 <= double(reach - 1) * r.w;
+    hd_status st;
+    if (!pairs) {
+        st = enqueue_chi(ctx, hk0);
+        if (st != HD_OK) return st;
+    }
     const size_t need = size_t(ctx->R) * size_t(nr);
     if (need > ctx->corr_cap) {
         if (ctx->corr_acc) cudaFree(ctx->corr_acc);
@@ -1991,14 +2001,29 @@ hd_status hd_positional_corr(hd_ctx* ctx, const int32_t* hk0, int32_t nr, double
         ctx->corr_acc = nullptr;
         ctx->corr = nullptr;
         ctx->corr_cap = 0;
-        HD_CK(ctx, cudaMalloc(&ctx->corr_acc, need * 3 * sizeof(double)));
+        HD_CK(ctx, cudaMalloc(&ctx->corr_acc, need * 6 * sizeof(double)));  // (2 nr + 1) x 2, or nr x 3, per replica
         HD_CK(ctx, cudaMalloc(&ctx->corr, need * sizeof(double2)));
         ctx->corr_cap = need;
     }
-    HD_CK(ctx, launch(ctx, HD_K_ANALYSIS, [&] {
-        return hd::launch_poscorr(ctx->cfg(), ctx->buf[ctx->cur], ctx->xy, ctx->chi, nr, dr / ctx->sigma, reach,
-                                  ctx->corr_acc, ctx->corr);
-    }));
+    if (pairs) {
+        const size_t slots = size_t(ctx->Ctot) * ctx->cap;
+        st = grow(ctx, ctx->sq_hk, ctx->sq_cap, size_t(ctx->R));
+        if (st == HD_OK) st = grow(ctx, ctx->corr_stage, ctx->corr_stage_cap, 2 * slots + (slots + 1) / 2);
+        if (st != HD_OK) return st;
+        HD_CK(ctx, cudaMemcpyAsync(ctx->sq_hk, hk0, sizeof(int2) * size_t(ctx->R), cudaMemcpyHostToDevice, ctx->stream));
+        int64_t most = 0;
+        for (const Rep& r : ctx->reps) most = std::max(most, int64_t(r.m) * r.m);
+        HD_CK(ctx, launch(ctx, HD_K_ANALYSIS, [&] {
+            return hd::launch_corr_pairs(ctx->cfg(), most, ctx->frame, ctx->buf[ctx->cur], ctx->sq_hk, ctx->corr_stage,
+                                         ctx->corr_stage + slots, reinterpret_cast<float2*>(ctx->corr_stage + 2 * slots), nr,
+                                         dr / ctx->sigma, reach, ctx->corr_acc, ctx->corr);
+        }));
+    } else {
+        HD_CK(ctx, launch(ctx, HD_K_ANALYSIS, [&] {
+            return hd::launch_poscorr(ctx->cfg(), ctx->buf[ctx->cur], ctx->xy, ctx->chi, nr, dr / ctx->sigma, reach,
+                                      ctx->corr_acc, ctx->corr);
+        }));
+    }
     HD_CK(ctx, cudaMemcpyAsync(C, ctx->corr, need * sizeof(double2), cudaMemcpyDeviceToHost, ctx->stream));
     HD_CK(ctx, cudaStreamSynchronize(ctx->stream));
     return HD_OK;

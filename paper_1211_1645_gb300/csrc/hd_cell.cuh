@@ -79,6 +79,26 @@ __device__ __forceinline__ void load_cell(const uint8_t* __restrict__ cnt, const
     }
 }
 
+// Global position (sigma units) of offset q in cell (cx, cy) of frame f:
+// X = (cx w + u) + shift, wrapped once.
+template <bool FIX>
+__device__ __forceinline__ void global_position(const Rep& rep, const Frame& f, int cx, int cy, const P2<FIX>& q, double& X,
+                                                double& Y) {
+    if constexpr (FIX) {
+        int64_t IX = int64_t(cx) * rep.W + q.x + f.Sx;
+        int64_t IY = int64_t(cy) * rep.W + q.y + f.Sy;
+        if (IX >= rep.LF) IX -= rep.LF;
+        if (IY >= rep.LF) IY -= rep.LF;
+        X = double(IX) * 0x1p-24;
+        Y = double(IY) * 0x1p-24;
+    } else {
+        X = __dadd_rn(__dadd_rn(__dmul_rn(double(cx), rep.w), q.x), f.sx);
+        Y = __dadd_rn(__dadd_rn(__dmul_rn(double(cy), rep.w), q.y), f.sy);
+        if (X >= rep.L) X = __dsub_rn(X, rep.L);
+        if (Y >= rep.L) Y = __dsub_rn(Y, rep.L);
+    }
+}
+
 // Shift difference between two frames (old minus new) and the direction of
 // the second feeding cell per axis (-1: old c-1 also feeds c; +1: old c+1).
 template <bool FIX>

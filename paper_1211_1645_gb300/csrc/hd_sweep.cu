@@ -172,19 +172,7 @@ k_positions(const Rep* __restrict__ reps, int R, const Frame* __restrict__ cur, 
         const P2<FIX> q = pos[size_t(k) * rep.stride32 + cell];
         const int64_t id = rep.id_off + pid[size_t(k) * rep.stride32 + cell];
         double X, Y;
-        if constexpr (FIX) {
-            int64_t IX = int64_t(cx) * rep.W + q.x + f.Sx;
-            int64_t IY = int64_t(cy) * rep.W + q.y + f.Sy;
-            if (IX >= rep.LF) IX -= rep.LF;
-            if (IY >= rep.LF) IY -= rep.LF;
-            X = double(IX) * 0x1p-24;
-            Y = double(IY) * 0x1p-24;
-        } else {
-            X = __dadd_rn(__dadd_rn(__dmul_rn(double(cx), rep.w), q.x), f.sx);
-            Y = __dadd_rn(__dadd_rn(__dmul_rn(double(cy), rep.w), q.y), f.sy);
-            if (X >= rep.L) X = __dsub_rn(X, rep.L);
-            if (Y >= rep.L) Y = __dsub_rn(Y, rep.L);
-        }
+        global_position<FIX>(rep, f, cx, cy, q, X, Y);
         xy[2 * id] = __dmul_rn(X, rep.sigma);
         xy[2 * id + 1] = __dmul_rn(Y, rep.sigma);
     }
