@@ -230,6 +230,11 @@ def _ntot(h) -> int:
     return sum(hd_get_geometry(h, r)["N"] for r in range(hd_replicas(h)))
 
 
+def _complex(a):
+    """The (Re, Im) pairs of an array [..., 2] as complex numbers, without a copy."""
+    return a.view(np.complex128)[..., 0]
+
+
 def hd_pressure(h, want_hist: bool = True):
     R = hd_replicas(h)
     bp = np.zeros(R, np.float64)
@@ -244,9 +249,9 @@ def hd_psi6(h, want_local: bool = True):
     R = hd_replicas(h)
     re = np.zeros(R, np.float64)
     im = np.zeros(R, np.float64)
-    loc = np.zeros((_ntot(h), 2), np.float64) if want_local else None
+    loc = np.empty((_ntot(h), 2), np.float64) if want_local else None  # written in full, or the call raises
     _check(load().hd_psi6(h, _ptr(re), _ptr(im), _ptr(loc)), "hd_psi6")
-    return re + 1j * im, (None if loc is None else loc[:, 0] + 1j * loc[:, 1])
+    return re + 1j * im, (None if loc is None else _complex(loc))
 
 
 def hd_positions(h) -> np.ndarray:
@@ -338,9 +343,9 @@ def hd_profile(h, enable: bool):
 def hd_psi6_acf(h, max_lag: int):
     """Eq. 9 autocorrelation of the recorded Psi_6 series: complex [R, max_lag + 1]."""
     R = hd_replicas(h)
-    out = np.zeros((R, int(max_lag) + 1, 2), np.float64)
+    out = np.empty((R, int(max_lag) + 1, 2), np.float64)
     _check(load().hd_psi6_acf(h, int(max_lag), _ptr(out)), "hd_psi6_acf")
-    return out[..., 0] + 1j * out[..., 1]
+    return _complex(out)
 
 
 def hd_psi6_tau(h, lag_lo: int, lag_hi: int):
@@ -356,7 +361,7 @@ def hd_psi6_field(h, bins: int):
     R = hd_replicas(h)
     out = np.zeros((R, int(bins), int(bins), 2), np.float64)
     _check(load().hd_psi6_field(h, int(bins), _ptr(out)), "hd_psi6_field")
-    return out[..., 0] + 1j * out[..., 1]
+    return _complex(out)
 
 
 def hd_structure_factor(h, hk):
@@ -386,7 +391,7 @@ def hd_positional_field(h, hk0, bins: int):
     hk0 = np.ascontiguousarray(np.broadcast_to(np.asarray(hk0, np.int32), (R, 2)), np.int32)
     out = np.zeros((R, int(bins), int(bins), 2), np.float64)
     _check(load().hd_positional_field(h, _ptr(hk0), int(bins), _ptr(out)), "hd_positional_field")
-    return out[..., 0] + 1j * out[..., 1]
+    return _complex(out)
 
 
 def hd_positional_corr(h, hk0, nr: int, dr: float):
@@ -395,7 +400,7 @@ def hd_positional_corr(h, hk0, nr: int, dr: float):
     hk0 = np.ascontiguousarray(np.broadcast_to(np.asarray(hk0, np.int32), (R, 2)), np.int32)
     out = np.zeros((R, int(nr), 2), np.float64)
     _check(load().hd_positional_corr(h, _ptr(hk0), int(nr), float(dr), _ptr(out)), "hd_positional_corr")
-    return out[..., 0] + 1j * out[..., 1]
+    return _complex(out)
 
 
 def hd_kernel_times(h):
