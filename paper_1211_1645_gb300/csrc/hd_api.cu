@@ -115,7 +115,7 @@ struct hd_ctx {
     double* fit = nullptr;
     double* fit_qr = nullptr;  // Householder factor of the fit's design matrix
     double2* psi_local = nullptr;
-    hd::ExactPair* psi_part = nullptr;  // [blocks_t32] exact block sums of psi_j
+    unsigned long long* psi_total = nullptr;  // exact sums of psi_j while psi_6 runs, zero between
     double* psi_res = nullptr;
     double* xy = nullptr;
     uint16_t* rep_of_act = nullptr;   // replica of each active-cell-grid block
@@ -774,10 +774,10 @@ cudaError_t enqueue_pressure(hd_ctx* ctx, cudaStream_t s, bool capturing) {
 cudaError_t enqueue_psi6(hd_ctx* ctx, cudaStream_t s, bool local, bool capturing) {
     const hd::LaunchCfg c = ctx->cfg(s);
     cudaError_t e = launch(ctx, HD_K_PSI6, [&] {
-        return hd::launch_psi6(c, ctx->buf[ctx->cur], local ? ctx->psi_local : nullptr, ctx->psi_part, ctx->err);
+        return hd::launch_psi6(c, ctx->buf[ctx->cur], local ? ctx->psi_local : nullptr, ctx->psi_total, ctx->err);
     }, capturing);
     if (e != cudaSuccess) return e;
-    return launch(ctx, HD_K_PSI6_REDUCE, [&] { return hd::launch_psi6_reduce(c, ctx->psi_part, ctx->psi_res); },
+    return launch(ctx, HD_K_PSI6_REDUCE, [&] { return hd::launch_psi6_reduce(c, ctx->psi_total, ctx->psi_res); },
                   capturing);
 }
 
@@ -928,7 +928,7 @@ hd_status hd_batch_init(hd_ctx** out, int32_t R, const int64_t* N, const double*
             rep.tx_mul = uint32_t((((uint64_t(1) << l) - uint64_t(rep.tiles_x)) << 32) / uint64_t(rep.tiles_x) + 1u);
             rep.tx_sh = l - 1;
         }
-        blk_t32 += int(int64_t(rep.tiles_x) * ((rep.m + ctx->threads / 32 - 1) / (ctx->threads / 32)));
+        blk_t32 += int(int64_t(rep.tiles_x) * ((rep.m + hd::psi6_rows() - 1) / hd::psi6_rows()));
         rep.blk_seg = blk_seg;
         rep.nseg = (rep.hm + ctx->threads - 1) / ctx->threads;
         rep.segw = (rep.hm + rep.nseg - 1) / rep.nseg;
@@ -1020,7 +1020,7 @@ hd_status hd_batch_init(hd_ctx** out, int32_t R, const int64_t* N, const double*
     ok = ok && dev_alloc(ctx, &ctx->fit, size_t(4 * R));
     ok = ok && dev_alloc(ctx, &ctx->fit_qr, hd::fit_factor_len(ctx->K));
     ok = ok && dev_alloc(ctx, &ctx->psi_local, size_t(ctx->Ntot));
-    ok = ok && dev_alloc(ctx, &ctx->psi_part, size_t(ctx->blocks_t32));
+    ok = ok && dev_alloc(ctx, &ctx->psi_total, hd::psi6_total_words(R));
     ok = ok && dev_alloc(ctx, &ctx->psi_res, size_t(2 * R));
     ok = ok && dev_alloc(ctx, &ctx->rep_of_act, size_t(ctx->blocks_act));
     ok = ok && dev_alloc(ctx, &ctx->rep_of_cell, size_t(ctx->blocks_cell));
@@ -1121,6 +1121,7 @@ hd_status hd_batch_init(hd_ctx** out, int32_t R, const int64_t* N, const double*
     cu = cu && cudaMemset(ctx->sweep_ctr, 0, sizeof(uint64_t) * size_t(R)) == cudaSuccess;
     cu = cu && cudaMemset(ctx->counters, 0, sizeof(unsigned long long) * size_t(2 * R)) == cudaSuccess;
     cu = cu && cudaMemset(ctx->err, 0, sizeof(int)) == cudaSuccess;
+    cu = cu && cudaMemset(ctx->psi_total, 0, hd::psi6_total_words(R) * sizeof(unsigned long long)) == cudaSuccess;
     cu = cu && cudaMemset(ctx->buf[0].cnt, 0, size_t(ctx->Ctot) + kCellPad) == cudaSuccess;
     cu = cu && cudaMemset(ctx->buf[1].cnt, 0, size_t(ctx->Ctot) + kCellPad) == cudaSuccess;
     cu = cu && hd::launch_fit_factor(nullptr, ctx->K, ctx->fit_qr) == cudaSuccess;

@@ -33,7 +33,7 @@ struct LaunchCfg {
     int blocks_cell;   // whole-cell grid size (all replicas)
     int blocks_act;    // active-cell grid size (all replicas)
     int blocks_tile;   // fused-sweep tile grid size (all replicas)
-    int blocks_t32;    // 32 x (threads / 32) cell-tile grid size (all replicas)
+    int blocks_t32;    // 32 x psi6_rows() cell-tile grid size (all replicas)
     int blocks_seg;    // half-row segment grid size of one colour pass (all replicas)
     int persist_blocks;  // grid of the persistent sweep (resident blocks), from persist_grid
     bool persist_stall;  // test hook: the persistent sweep withholds one item and gives up waiting early
@@ -123,10 +123,14 @@ cudaError_t launch_hist(const LaunchCfg& c, const HistCfg& h, CellBufs cells, un
 size_t fit_factor_len(int K);
 cudaError_t launch_fit_factor(cudaStream_t s, int K, double* qr);
 cudaError_t launch_fit(const LaunchCfg& c, int K, const double* qr, const unsigned long long* hist, double* res);
-// Local psi_6 into local (nullable) and each block's exact sum into partial
-// [blocks_t32]; the reduction rounds each replica's total once and divides by N.
-cudaError_t launch_psi6(const LaunchCfg& c, CellBufs cells, double2* local, ExactPair* partial, int* err);
-cudaError_t launch_psi6_reduce(const LaunchCfg& c, const ExactPair* partial, double* res);
+// Local psi_6 into local (nullable) and its exact sums added to total
+// (psi6_total_words(R) words, zero before); the reduction rounds each
+// replica's once, divides by N and leaves total zero.  psi6_rows: rows of cells
+// of the 32-column tile grid (blk_t32, blocks_t32).
+size_t psi6_total_words(int R);
+int psi6_rows();
+cudaError_t launch_psi6(const LaunchCfg& c, CellBufs cells, double2* local, unsigned long long* total, int* err);
+cudaError_t launch_psi6_reduce(const LaunchCfg& c, unsigned long long* total, double* res);
 // Append (beta P / rho, g(2 sigma+), Re Psi_6, Im Psi_6) of every replica to
 // series[len] and advance len (bounded by cap; a full series sets err bit 4).
 cudaError_t launch_record(const LaunchCfg& c, const double* fit, const double* psi, double* series,

@@ -466,197 +466,353 @@ __device__ __forceinline__ bool ring_covers(const Rep& rep, const Nbr<FIX>& nb, 
 // cells plus a halo of two cells (the 5 x 5 stencil of every tile cell).
 constexpr int kPsiHalo = 2;
 constexpr int kPsiSX = 32 + 2 * kPsiHalo;
+constexpr int kPsiThreads = 256;  // a tile of eight rows: 1.7 staged cells per cell
 
 template <bool FIX, int CAP>
 __host__ __device__ constexpr size_t psi6_stage_bytes(int rows) {
-    return size_t(kPsiSX) * size_t(rows + 2 * kPsiHalo) * (CAP * (sizeof(P2<FIX>) + sizeof(int32_t)) + 1);
+    return size_t(kPsiSX) * size_t(rows + 2 * kPsiHalo) * (2 * sizeof(float2) + CAP * (sizeof(P2<FIX>) + sizeof(int32_t)) + 1);
 }
 
-// psi_6 of every disk.  A block stages its tile and halo in shared memory in
-// one cooperative round of loads; each disk then scans its 5 x 5 stencil
-// there, nearest cells first (so the six-neighbour list fills early and most
-// later candidates are rejected by one comparison).  The rare disk whose six
-// neighbours are not certified by the 5 x 5 stencil (low density) continues
-// the ring search in global memory.
-// Registers per thread: the fixed form runs at four blocks of 256 per SM
-// (64 registers, a few spilled, 0.238 -> 0.211 ms at N = 1M: more resident
-// warps hide the insertion's dependency chains); the FP64 form at 118
-// registers (no spill).
+// What a disk of a tile sees.
+template <bool FIX>
+struct PsiStage {
+    const float2* img;   // [2][nS] float offsets of slots 0 and 1, infinite where unoccupied
+    const P2<FIX>* pos;  // [CAP][nS]
+    const int32_t* id;   // [CAP][nS]
+    const uint8_t* n;    // [nS]
+    int nS;
+};
+
+// The general search of a disk's six nearest: ordered insertion of every
+// candidate by (r^2, id) from the staged rings 0, 1, 2, then rings in global
+// memory until the sixth is certified.  Out of line: the float search below
+// leaves it about one disk in a thousand.
 template <bool FIX, int CAP>
-__global__ void __launch_bounds__(256, FIX ? 4 : 1)
+static __device__ __noinline__ bool nearest_general(const Rep& rep, const PsiStage<FIX>& st, const uint8_t* cnt,
+                                                    const P2<FIX>* pos, const int32_t* pid, int own, int cx, int cy,
+                                                    P2<FIX> me, int32_t idme, int rmax, typename Nbr<FIX>::Off* ox,
+                                                    typename Nbr<FIX>::Off* oy) {
+    Nbr<FIX> nb;
+    nb.n = 0;
+    bool ok = false;
+    if (rmax >= 2) {
+#pragma unroll 1
+        for (int ring = 0; ring <= 2; ++ring) {
+            for (int dcy = -ring; dcy <= ring; ++dcy) {
+                for (int dcx = -ring; dcx <= ring; ++dcx) {
+                    if (max(abs(dcx), abs(dcy)) != ring) continue;
+                    const int sc = own + dcy * kPsiSX + dcx;
+                    const int nn = st.n[sc];
+                    for (int q = 0; q < nn; ++q) {
+                        const int32_t idq = st.id[q * st.nS + sc];
+                        if (idq == idme) continue;
+                        const P2<FIX> o = st.pos[q * st.nS + sc];
+                        if constexpr (FIX) {
+                            const int32_t rx = (o.x + dcx * rep.W) - me.x;
+                            const int32_t ry = (o.y + dcy * rep.W) - me.y;
+                            nb.insert(int64_t(rx) * rx + int64_t(ry) * ry, idq, rx, ry);
+                        } else {
+                            const double rx = __dsub_rn(__dadd_rn(o.x, __dmul_rn(double(dcx), rep.w)), me.x);
+                            const double ry = __dsub_rn(__dadd_rn(o.y, __dmul_rn(double(dcy), rep.w)), me.y);
+                            nb.insert(__double_as_longlong(__dadd_rn(__dmul_rn(rx, rx), __dmul_rn(ry, ry))), idq, rx, ry);
+                        }
+                    }
+                }
+            }
+        }
+        ok = ring_covers<FIX>(rep, nb, me, 2);
+    }
+    for (int RR = 3; RR <= rmax && !ok; ++RR) {
+        for (int e = -RR; e <= RR; ++e) {
+            scan_cell<FIX, CAP>(rep, cnt, pos, pid, cx, cy, e, -RR, me, idme, nb);
+            scan_cell<FIX, CAP>(rep, cnt, pos, pid, cx, cy, e, RR, me, idme, nb);
+        }
+        for (int e = -RR + 1; e <= RR - 1; ++e) {
+            scan_cell<FIX, CAP>(rep, cnt, pos, pid, cx, cy, -RR, e, me, idme, nb);
+            scan_cell<FIX, CAP>(rep, cnt, pos, pid, cx, cy, RR, e, me, idme, nb);
+        }
+        ok = ring_covers<FIX>(rep, nb, me, RR);
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        ox[q] = nb.rx[q];
+        oy[q] = nb.ry[q];
+    }
+    return ok;
+}
+
+// The six nearest of a disk (slot k of staged cell own) from its 5 x 5 stencil
+// by float distances: every candidate's d^2 + 64 has its 23 mantissa bits as a
+// fixed-point d^2 (quantum 2^-17) above seven bits of candidate number, and
+// the seven smallest of these words are kept by min / max (fourteen
+// instructions per candidate, no branch).  For d^2 < 64 the float value errs by
+// less than 5.2 quanta: offsets and cell side rounded to 2^-23, two sums below
+// 16, the square sum and the addition of 64.  So words 16 quanta apart are in
+// the order of the exact distances: a sixth and seventh closer than that, or a
+// sixth at 64 or beyond, go to nearest_general (returns 0); closer words among
+// the six are put in order by their exact (r^2, id).  Returns 1 when the six
+// are certified by the stencil, else 0.
+constexpr uint32_t kPsiMargin = 16u << 7;
+
+template <bool FIX, int CAP>
+__device__ __forceinline__ bool nearest_float(const Rep& rep, const PsiStage<FIX>& st, int own, int k, const P2<FIX>& me,
+                                              typename Nbr<FIX>::Off (&ox)[6], typename Nbr<FIX>::Off (&oy)[6]) {
+    const float wf = FIX ? __fmul_rn(__int2float_rn(rep.W), 0x1p-24f) : float(rep.w);
+    float2 um;
+    if constexpr (FIX) um = make_float2(__fmul_rn(__int2float_rn(me.x), 0x1p-24f), __fmul_rn(__int2float_rn(me.y), 0x1p-24f));
+    else um = make_float2(__double2float_rn(me.x), __double2float_rn(me.y));
+    uint32_t key[7];
+#pragma unroll
+    for (int s = 0; s < 7; ++s) key[s] = ~0u;
+    auto take = [&](const float2& f, float bx, float by, uint32_t number, bool self) {
+        const float sx = __fadd_rn(f.x, bx), sy = __fadd_rn(f.y, by);
+        const float d = __fadd_rn(__fmaf_rn(sx, sx, __fmul_rn(sy, sy)), 64.0f);
+        uint32_t x = (__float_as_uint(d) << 7) + number;
+        if (self) x = ~0u;
+#pragma unroll
+        for (int s = 0; s < 7; ++s) {
+            const uint32_t lo = min(key[s], x);
+            x = max(key[s], x);
+            key[s] = lo;
+        }
+    };
+#pragma unroll 1
+    for (int dcy = -2; dcy <= 2; ++dcy) {
+        const float by = __fsub_rn(__fmul_rn(float(dcy), wf), um.y);
+        const int row = own + dcy * kPsiSX;
+        const uint32_t number = uint32_t(dcy + 2) * 20u;
+#pragma unroll
+        for (int dcx = -2; dcx <= 2; ++dcx) {
+            const float bx = __fsub_rn(__fmul_rn(float(dcx), wf), um.x);
+            const bool here = dcx == 0 && dcy == 0;
+            take(st.img[row + dcx], bx, by, number + uint32_t(dcx + 2) * 4u, here && k == 0);
+            take(st.img[st.nS + row + dcx], bx, by, number + uint32_t(dcx + 2) * 4u + 1u, here && k == 1);
+            const int n = st.n[row + dcx];
+            for (int q = 2; q < n; ++q) {  // rare
+                const P2<FIX> o = st.pos[q * st.nS + row + dcx];
+                float2 f;
+                if constexpr (FIX) f = make_float2(__fmul_rn(__int2float_rn(o.x), 0x1p-24f), __fmul_rn(__int2float_rn(o.y), 0x1p-24f));
+                else f = make_float2(__double2float_rn(o.x), __double2float_rn(o.y));
+                take(f, bx, by, number + uint32_t(dcx + 2) * 4u + uint32_t(q), here && k == q);
+            }
+        }
+    }
+    if (key[5] >= 0x80000000u || key[6] - key[5] < kPsiMargin) return false;
+    Nbr<FIX> nb;
+    bool close = false;
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+        if (s > 0) close |= key[s] - key[s - 1] < kPsiMargin;
+        const uint32_t number = key[s] & 127u, c = number >> 2, dy = (c * 13u) >> 6;  // c / 5 for c < 25
+        const int dcx = int(c - dy * 5u) - 2, dcy = int(dy) - 2;
+        const int at = int(number & 3u) * st.nS + own + dcy * kPsiSX + dcx;
+        const P2<FIX> o = st.pos[at];
+        if constexpr (FIX) {
+            nb.rx[s] = (o.x + dcx * rep.W) - me.x;
+            nb.ry[s] = (o.y + dcy * rep.W) - me.y;
+        } else {
+            nb.rx[s] = __dsub_rn(__dadd_rn(o.x, __dmul_rn(double(dcx), rep.w)), me.x);
+            nb.ry[s] = __dsub_rn(__dadd_rn(o.y, __dmul_rn(double(dcy), rep.w)), me.y);
+        }
+    }
+    auto square = [&](int s) -> long long {
+        if constexpr (FIX) return int64_t(nb.rx[s]) * nb.rx[s] + int64_t(nb.ry[s]) * nb.ry[s];
+        else return __double_as_longlong(__dadd_rn(__dmul_rn(nb.rx[s], nb.rx[s]), __dmul_rn(nb.ry[s], nb.ry[s])));
+    };
+    if (close) {  // rare: the exact order of the six
+        Nbr<FIX> in;
+        in.n = 0;
+#pragma unroll
+        for (int s = 0; s < 6; ++s) {
+            const uint32_t number = key[s] & 127u, c = number >> 2, dy = (c * 13u) >> 6;
+            const int at = int(number & 3u) * st.nS + own + (int(dy) - 2) * kPsiSX + int(c - dy * 5u) - 2;
+            in.insert(square(s), st.id[at], nb.rx[s], nb.ry[s]);
+        }
+#pragma unroll
+        for (int s = 0; s < 6; ++s) {
+            nb.rx[s] = in.rx[s];
+            nb.ry[s] = in.ry[s];
+        }
+    }
+    nb.n = 6;
+    nb.key[5] = square(5);
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+        ox[s] = nb.rx[s];
+        oy[s] = nb.ry[s];
+    }
+    return ring_covers<FIX>(rep, nb, me, 2);
+}
+
+// Global sums of psi_j of each replica while k_psi6 runs: the 192-bit sums of
+// its blocks added as 32-bit limbs in 64-bit words (Re six, Im six), so that
+// blocks add atomically without carries; word 12 is set by a sum marked bad.
+// k_psi6_reduce reads them and leaves them zero (one block over a partial sum
+// per tile took 27 us at N = 2^20 after the last block; this takes 6).
+constexpr int kPsiWords = 16;
+
+// psi_6 of every disk.  A block stages its tile and halo in shared memory in
+// one cooperative round of loads; each disk then finds its six nearest there
+// (nearest_float, or nearest_general: a stencil that does not certify them, as
+// at low density, continues in global memory).
+// Instruction-bound in the fixed form (ordered insertion of 25 candidates by
+// 64-bit keys took ~4800 instructions per disk, this ~3050): 182 -> 138 us at N
+// = 2^20, 58 -> 47 at 262,144.  The FP64 form is bound by the FP64 pipe (84%
+// busy, mostly the fourteen correctly rounded divisions per disk): 952 -> 668.
+template <bool FIX, int CAP>
+__global__ void __launch_bounds__(kPsiThreads, FIX ? 4 : 2)
 k_psi6(const Rep* __restrict__ reps, int R, const uint8_t* __restrict__ cnt, const P2<FIX>* __restrict__ pos,
-       const int32_t* __restrict__ pid, double2* __restrict__ local, ExactPair* __restrict__ partial,
+       const int32_t* __restrict__ pid, double2* __restrict__ local, unsigned long long* __restrict__ total,
        int* __restrict__ err) {
     extern __shared__ __align__(16) unsigned char s_raw[];
     pdl_begin();
     const int r = find_rep<kGridT32>(reps, R, blockIdx.x);
     const Rep& rep = reps[r];
     const int m = rep.m;
-    const int rows = int(blockDim.x >> 5);
+    constexpr int rows = kPsiThreads / 32;
     int X0, Y0;
     tile32_origin(rep, uint32_t(blockIdx.x - rep.blk_t32), rows, X0, Y0);
-    const int nS = kPsiSX * (rows + 2 * kPsiHalo);
-    P2<FIX>* s_pos = reinterpret_cast<P2<FIX>*>(s_raw);                  // [CAP][nS]
-    int32_t* s_id = reinterpret_cast<int32_t*>(s_pos + size_t(CAP) * nS);  // [CAP][nS]
+    constexpr int nS = kPsiSX * (rows + 2 * kPsiHalo);
+    P2<FIX>* s_pos = reinterpret_cast<P2<FIX>*>(s_raw);                    // [CAP][nS]
+    float2* s_img = reinterpret_cast<float2*>(s_pos + size_t(CAP) * nS);   // [2][nS]
+    int32_t* s_id = reinterpret_cast<int32_t*>(s_img + size_t(2) * nS);    // [CAP][nS]
     uint8_t* s_n = reinterpret_cast<uint8_t*>(s_id + size_t(CAP) * nS);    // [nS]
-    for (int t = threadIdx.x; t < nS; t += blockDim.x) {
+    for (int t = threadIdx.x; t < nS; t += kPsiThreads) {
         const int sy = t / kPsiSX, sx = t - sy * kPsiSX;
         const uint32_t c = uint32_t(rep.coff) + row_part(rep, wrap_cell(Y0 - kPsiHalo + sy, m)) +
                            col_part(rep, wrap_cell(X0 - kPsiHalo + sx, m));
         const int n = min(int(cnt[c]), CAP);
         s_n[t] = uint8_t(n);
+        float2 f[2];
+        f[0] = f[1] = make_float2(__uint_as_float(0x7F800000u), __uint_as_float(0x7F800000u));
         for (int q = 0; q < n; ++q) {
-            s_pos[q * nS + t] = pos[size_t(q) * rep.stride32 + c];
+            const P2<FIX> o = pos[size_t(q) * rep.stride32 + c];
+            s_pos[q * nS + t] = o;
             s_id[q * nS + t] = pid[size_t(q) * rep.stride32 + c];
+            if (q < 2) {
+                if constexpr (FIX) f[q] = make_float2(__fmul_rn(__int2float_rn(o.x), 0x1p-24f), __fmul_rn(__int2float_rn(o.y), 0x1p-24f));
+                else f[q] = make_float2(__double2float_rn(o.x), __double2float_rn(o.y));
+            }
         }
+        s_img[t] = f[0];
+        s_img[nS + t] = f[1];
     }
     __syncthreads();
 
-    __shared__ uint16_t s_list[256 * CAP];
+    __shared__ uint16_t s_list[kPsiThreads * CAP];
     __shared__ int s_warp[8];
     const int D = tile_disk_list(s_n, kPsiSX, kPsiHalo, X0, Y0, m, s_list, s_warp);
+    const PsiStage<FIX> st{s_img, s_pos, s_id, s_n, nS};
     Exact192 sr = exact_zero(), si = exact_zero();  // exact sums of this thread's psi_j
     int rmax = (m - 1) / 2;
     if constexpr (FIX) {
         const int lim = int((int64_t(1) << 31) / rep.W) - 1;
         if (lim < rmax) rmax = lim;
     }
-    {
-        for (int d = threadIdx.x; d < D; d += blockDim.x) {
-            const int own = int(s_list[d] >> 4), k = int(s_list[d] & 15u);
+    for (int d = threadIdx.x; d < D; d += kPsiThreads) {
+        const int own = int(s_list[d] >> 4), k = int(s_list[d] & 15u);
+        const P2<FIX> me = s_pos[k * nS + own];
+        const int32_t idme = s_id[k * nS + own];
+        typename Nbr<FIX>::Off rx[6], ry[6];
+        bool ok = false;
+        if (CAP == 4 && rmax >= 2) ok = nearest_float<FIX, CAP>(rep, st, own, k, me, rx, ry);
+        if (!ok) {
             const int sy = own / kPsiSX;
             const int cx = X0 + (own - sy * kPsiSX) - kPsiHalo, cy = Y0 + sy - kPsiHalo;
-            const P2<FIX> me = s_pos[k * nS + own];
-            const int32_t idme = s_id[k * nS + own];
-            float mfx = 0.0f, mfy = 0.0f;  // FP64 form: float images of the disk's offsets
-            if constexpr (!FIX) {
-                mfx = approx_f32(me.x);
-                mfy = approx_f32(me.y);
-            }
-            Nbr<FIX> nb;
-            nb.n = 0;
-            bool ok = false;
-            if (rmax >= 2) {
-                // rings 0, 1, 2 of the staged stencil, nearest first
-#pragma unroll 1
-                for (int ring = 0; ring <= 2; ++ring) {
-                    for (int dcy = -ring; dcy <= ring; ++dcy) {
-                        for (int dcx = -ring; dcx <= ring; ++dcx) {
-                            if (max(abs(dcx), abs(dcy)) != ring) continue;
-                            const int sc = own + dcy * kPsiSX + dcx;
-                            const int nn = s_n[sc];
-                            for (int q = 0; q < nn; ++q) {
-                                const int32_t idq = s_id[q * nS + sc];
-                                if (idq == idme) continue;
-                                const P2<FIX> o = s_pos[q * nS + sc];
-                                if constexpr (FIX) {
-                                    const int32_t rx = (o.x + dcx * rep.W) - me.x;
-                                    const int32_t ry = (o.y + dcy * rep.W) - me.y;
-                                    nb.insert(int64_t(rx) * rx + int64_t(ry) * ry, idq, rx, ry);
-                                } else {
-                                    if (nb.n == 6) {
-                                        // float pre-test: a candidate whose float estimate
-                                        // of r^2 exceeds the sixth key by more than the
-                                        // estimate's error bound is farther in FP64 too
-                                        // (approx_f32 truncates; the product rounds up
-                                        // past the key itself)
-                                        const float sx = __fsub_rn(__fadd_rn(approx_f32(o.x), __fmul_rn(float(dcx), rep.wf)), mfx);
-                                        const float sy = __fsub_rn(__fadd_rn(approx_f32(o.y), __fmul_rn(float(dcy), rep.wf)), mfy);
-                                        const float d2f = __fadd_rn(__fmul_rn(sx, sx), __fmul_rn(sy, sy));
-                                        const float k5 = __fmul_ru(approx_f32(__longlong_as_double(nb.key[5])), 1.0f + 0x1p-19f);
-                                        if (d2f > __fadd_ru(k5, rep.psi_m)) continue;
-                                    }
-                                    const double rx = __dsub_rn(__dadd_rn(o.x, __dmul_rn(double(dcx), rep.w)), me.x);
-                                    const double ry = __dsub_rn(__dadd_rn(o.y, __dmul_rn(double(dcy), rep.w)), me.y);
-                                    nb.insert(__double_as_longlong(__dadd_rn(__dmul_rn(rx, rx), __dmul_rn(ry, ry))), idq, rx, ry);
-                                }
-                            }
-                        }
-                    }
-                }
-                ok = ring_covers<FIX>(rep, nb, me, 2);
-            }
-            for (int RR = 3; RR <= rmax && !ok; ++RR) {
-                for (int e = -RR; e <= RR; ++e) {
-                    scan_cell<FIX, CAP>(rep, cnt, pos, pid, cx, cy, e, -RR, me, idme, nb);
-                    scan_cell<FIX, CAP>(rep, cnt, pos, pid, cx, cy, e, RR, me, idme, nb);
-                }
-                for (int e = -RR + 1; e <= RR - 1; ++e) {
-                    scan_cell<FIX, CAP>(rep, cnt, pos, pid, cx, cy, -RR, e, me, idme, nb);
-                    scan_cell<FIX, CAP>(rep, cnt, pos, pid, cx, cy, RR, e, me, idme, nb);
-                }
-                ok = ring_covers<FIX>(rep, nb, me, RR);
-            }
-            double pre, pim;
-            if (!ok) {
-                atomicOr(err, 2);
-                pre = pim = 0.0;
-            } else if constexpr (FIX) {
-                float fr = 0.0f, fi = 0.0f;
+            typename Nbr<FIX>::Off gx[6], gy[6];
+            ok = nearest_general<FIX, CAP>(rep, st, cnt, pos, pid, own, cx, cy, me, idme, rmax, gx, gy);
 #pragma unroll
-                for (int q = 0; q < 6; ++q) {
-                    const float x = __fmul_rn(__int2float_rn(nb.rx[q]), 0x1p-24f);
-                    const float y = __fmul_rn(__int2float_rn(nb.ry[q]), 0x1p-24f);
-                    const float xx = __fmul_rn(x, x), yy = __fmul_rn(y, y);
-                    const float r2 = __fadd_rn(xx, yy);
-                    const float c2 = __fsub_rn(xx, yy), s2 = __fmul_rn(__fmul_rn(x, y), 2.0f);
-                    const float c4 = __fsub_rn(__fmul_rn(c2, c2), __fmul_rn(s2, s2));
-                    const float s4 = __fmul_rn(__fmul_rn(c2, s2), 2.0f);
-                    const float c6 = __fsub_rn(__fmul_rn(c4, c2), __fmul_rn(s4, s2));
-                    const float s6 = __fadd_rn(__fmul_rn(c4, s2), __fmul_rn(s4, c2));
-                    const float r6 = __fmul_rn(__fmul_rn(r2, r2), r2);
-                    fr = __fadd_rn(fr, __fdiv_rn(c6, r6));
-                    fi = __fadd_rn(fi, __fdiv_rn(s6, r6));
-                }
-                pre = double(__fdiv_rn(fr, 6.0f));
-                pim = double(__fdiv_rn(fi, 6.0f));
-            } else {
-                double dr_ = 0.0, di = 0.0;
-#pragma unroll
-                for (int q = 0; q < 6; ++q) {
-                    const double x = nb.rx[q], y = nb.ry[q];
-                    const double xx = __dmul_rn(x, x), yy = __dmul_rn(y, y);
-                    const double r2 = __dadd_rn(xx, yy);
-                    const double c2 = __dsub_rn(xx, yy), s2 = __dmul_rn(__dmul_rn(x, y), 2.0);
-                    const double c4 = __dsub_rn(__dmul_rn(c2, c2), __dmul_rn(s2, s2));
-                    const double s4 = __dmul_rn(__dmul_rn(c2, s2), 2.0);
-                    const double c6 = __dsub_rn(__dmul_rn(c4, c2), __dmul_rn(s4, s2));
-                    const double s6 = __dadd_rn(__dmul_rn(c4, s2), __dmul_rn(s4, c2));
-                    const double r6 = __dmul_rn(__dmul_rn(r2, r2), r2);
-                    dr_ = __dadd_rn(dr_, __ddiv_rn(c6, r6));
-                    di = __dadd_rn(di, __ddiv_rn(s6, r6));
-                }
-                pre = __ddiv_rn(dr_, 6.0);
-                pim = __ddiv_rn(di, 6.0);
+            for (int q = 0; q < 6; ++q) {
+                rx[q] = gx[q];
+                ry[q] = gy[q];
             }
-            if (local) local[rep.id_off + idme] = make_double2(pre, pim);
-            exact_add(sr, pre);
-            exact_add(si, pim);
         }
+        double pre, pim;
+        if (!ok) {
+            atomicOr(err, 2);
+            pre = pim = 0.0;
+        } else if constexpr (FIX) {
+            float fr = 0.0f, fi = 0.0f;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                const float x = __fmul_rn(__int2float_rn(rx[q]), 0x1p-24f);
+                const float y = __fmul_rn(__int2float_rn(ry[q]), 0x1p-24f);
+                const float xx = __fmul_rn(x, x), yy = __fmul_rn(y, y);
+                const float r2 = __fadd_rn(xx, yy);
+                const float c2 = __fsub_rn(xx, yy), s2 = __fmul_rn(__fmul_rn(x, y), 2.0f);
+                const float c4 = __fsub_rn(__fmul_rn(c2, c2), __fmul_rn(s2, s2));
+                const float s4 = __fmul_rn(__fmul_rn(c2, s2), 2.0f);
+                const float c6 = __fsub_rn(__fmul_rn(c4, c2), __fmul_rn(s4, s2));
+                const float s6 = __fadd_rn(__fmul_rn(c4, s2), __fmul_rn(s4, c2));
+                const float r6 = __fmul_rn(__fmul_rn(r2, r2), r2);
+                fr = __fadd_rn(fr, __fdiv_rn(c6, r6));
+                fi = __fadd_rn(fi, __fdiv_rn(s6, r6));
+            }
+            pre = double(__fdiv_rn(fr, 6.0f));
+            pim = double(__fdiv_rn(fi, 6.0f));
+        } else {
+            double dr_ = 0.0, di = 0.0;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                const double x = rx[q], y = ry[q];
+                const double xx = __dmul_rn(x, x), yy = __dmul_rn(y, y);
+                const double r2 = __dadd_rn(xx, yy);
+                const double c2 = __dsub_rn(xx, yy), s2 = __dmul_rn(__dmul_rn(x, y), 2.0);
+                const double c4 = __dsub_rn(__dmul_rn(c2, c2), __dmul_rn(s2, s2));
+                const double s4 = __dmul_rn(__dmul_rn(c2, s2), 2.0);
+                const double c6 = __dsub_rn(__dmul_rn(c4, c2), __dmul_rn(s4, s2));
+                const double s6 = __dadd_rn(__dmul_rn(c4, s2), __dmul_rn(s4, c2));
+                const double r6 = __dmul_rn(__dmul_rn(r2, r2), r2);
+                dr_ = __dadd_rn(dr_, __ddiv_rn(c6, r6));
+                di = __dadd_rn(di, __ddiv_rn(s6, r6));
+            }
+            pre = __ddiv_rn(dr_, 6.0);
+            pim = __ddiv_rn(di, 6.0);
+        }
+        if (local) local[rep.id_off + idme] = make_double2(pre, pim);
+        exact_add(sr, pre);
+        exact_add(si, pim);
     }
     // block sum: exact, so its value does not depend on the order of the disks
     const ExactPair t = exact_block_sum(sr, si);
-    if (threadIdx.x == 0) partial[blockIdx.x] = t;
+    if (threadIdx.x == 0) {
+        unsigned long long* w = total + size_t(r) * kPsiWords;
+        const unsigned long long v[6] = {t.re.w0, t.re.w1, t.re.w2, t.im.w0, t.im.w1, t.im.w2};
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {
+            atomicAdd(&w[2 * q], v[q] & 0xFFFFFFFFull);
+            atomicAdd(&w[2 * q + 1], v[q] >> 32);
+        }
+        if (t.re.bad) atomicOr(&w[12], 1ull);
+        if (t.im.bad) atomicOr(&w[12], 2ull);
+    }
 }
 
-// Psi_6 of each replica: the exact sum of its block partials rounded once to
-// double, then divided by N (the oracle's order of operations).
-__global__ void k_psi6_reduce(const Rep* __restrict__ reps, int R, int blocks_total,
-                              const ExactPair* __restrict__ partial, double* __restrict__ res) {
+// Psi_6 of each replica: its exact sum rounded once to double, then divided by
+// N (the oracle's order of operations).  One block of one warp per replica.
+__global__ void __launch_bounds__(32)
+k_psi6_reduce(const Rep* __restrict__ reps, unsigned long long* __restrict__ total, double* __restrict__ res) {
     pdl_begin();
-    const int r = blockIdx.x;
-    const Rep& rep = reps[r];
-    const int b0 = rep.blk_t32;
-    const int b1 = (r + 1 < R) ? reps[r + 1].blk_t32 : blocks_total;
-    Exact192 sr = exact_zero(), si = exact_zero();
-    for (int b = b0 + int(threadIdx.x); b < b1; b += blockDim.x) {
-        exact_merge(sr, partial[b].re);
-        exact_merge(si, partial[b].im);
+    const int r = blockIdx.x, lane = int(threadIdx.x);
+    unsigned long long* w = total + size_t(r) * kPsiWords;
+    __shared__ unsigned long long s_w[kPsiWords];
+    if (lane < 13) {
+        s_w[lane] = w[lane];
+        w[lane] = 0ull;
     }
-    const ExactPair t = exact_block_sum(sr, si);
-    if (threadIdx.x == 0) {
-        res[2 * r] = __ddiv_rn(exact_round(t.re), double(rep.N));
-        res[2 * r + 1] = __ddiv_rn(exact_round(t.im), double(rep.N));
+    __syncwarp();
+    if (lane < 2) {
+        const unsigned long long* p = s_w + 6 * lane;
+        unsigned long long limb[6], carry = 0ull;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) {  // fewer than 2^31 blocks: no overflow
+            const unsigned long long v = p[q] + carry;
+            limb[q] = v & 0xFFFFFFFFull;
+            carry = v >> 32;
+        }
+        const Exact192 sum{limb[0] | limb[1] << 32, limb[2] | limb[3] << 32, limb[4] | limb[5] << 32,
+                           (unsigned int)(s_w[12] >> lane) & 1u};
+        res[2 * r + lane] = __ddiv_rn(exact_round(sum), double(reps[r].N));
     }
 }
 
@@ -671,8 +827,8 @@ static cudaError_t hist_t(const LaunchCfg& c, const HistCfg& h, CellBufs cells, 
             cudaFuncSetAttribute(k_hist_tile<FIX, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  int(hist_stage_bytes<FIX, CAP>(8, kHistMaxHalo, kMaxFitBins)));
         });
-        return launch_k(k_hist_tile<FIX, CAP>, dim3(c.blocks_t32), dim3(c.threads),
-                        hist_stage_bytes<FIX, CAP>(c.threads / 32, h.halo, h.K), c.stream, c.reps, c.R, h.K, h.edges,
+        return launch_k(k_hist_tile<FIX, CAP>, dim3(c.blocks_t32), dim3(kPsiThreads),
+                        hist_stage_bytes<FIX, CAP>(kPsiThreads / 32, h.halo, h.K), c.stream, c.reps, c.R, h.K, h.edges,
                         h.edgesF, (const uint8_t*)cells.cnt, (const P2<FIX>*)cells.pos, (const int32_t*)cells.pid,
                         hist, h.halo);
     }
@@ -699,22 +855,24 @@ cudaError_t launch_fit(const LaunchCfg& c, int K, const double* qr, const unsign
     return launch_k(k_fit, dim3(c.R), dim3(32), 0, c.stream, c.reps, K, qr, hist, res);
 }
 
+size_t psi6_total_words(int R) { return size_t(R) * kPsiWords; }
+int psi6_rows() { return kPsiThreads / 32; }
+
 template <bool FIX, int CAP>
-static cudaError_t psi6_t(const LaunchCfg& c, CellBufs cells, double2* local, ExactPair* partial, int* err) {
-    const size_t smem = psi6_stage_bytes<FIX, CAP>(c.threads / 32);
+static cudaError_t psi6_t(const LaunchCfg& c, CellBufs cells, double2* local, unsigned long long* total, int* err) {
+    constexpr size_t smem = psi6_stage_bytes<FIX, CAP>(kPsiThreads / 32);
     static std::once_flag attr_once;
     std::call_once(attr_once, [] {
-        cudaFuncSetAttribute(k_psi6<FIX, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(psi6_stage_bytes<FIX, CAP>(8)));
+        cudaFuncSetAttribute(k_psi6<FIX, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     });
-    return launch_k(k_psi6<FIX, CAP>, dim3(c.blocks_t32), dim3(c.threads), smem, c.stream, c.reps, c.R,
-                    (const uint8_t*)cells.cnt, (const P2<FIX>*)cells.pos, (const int32_t*)cells.pid, local, partial,
+    return launch_k(k_psi6<FIX, CAP>, dim3(c.blocks_t32), dim3(kPsiThreads), smem, c.stream, c.reps, c.R,
+                    (const uint8_t*)cells.cnt, (const P2<FIX>*)cells.pos, (const int32_t*)cells.pid, local, total,
                     err);
 }
 
-cudaError_t launch_psi6(const LaunchCfg& c, CellBufs cells, double2* local, ExactPair* partial, int* err) {
-    if (c.fixed) return c.cap == 4 ? psi6_t<true, 4>(c, cells, local, partial, err) : psi6_t<true, 9>(c, cells, local, partial, err);
-    return c.cap == 4 ? psi6_t<false, 4>(c, cells, local, partial, err) : psi6_t<false, 9>(c, cells, local, partial, err);
+cudaError_t launch_psi6(const LaunchCfg& c, CellBufs cells, double2* local, unsigned long long* total, int* err) {
+    if (c.fixed) return c.cap == 4 ? psi6_t<true, 4>(c, cells, local, total, err) : psi6_t<true, 9>(c, cells, local, total, err);
+    return c.cap == 4 ? psi6_t<false, 4>(c, cells, local, total, err) : psi6_t<false, 9>(c, cells, local, total, err);
 }
 
 __global__ void k_record(int R, const double* __restrict__ fit, const double* __restrict__ psi,
@@ -741,8 +899,8 @@ cudaError_t launch_record(const LaunchCfg& c, const double* fit, const double* p
     return launch_k(k_record, dim3(1), dim3(((c.R + 31) / 32) * 32), 0, c.stream, c.R, fit, psi, series, len, cap, err);
 }
 
-cudaError_t launch_psi6_reduce(const LaunchCfg& c, const ExactPair* partial, double* res) {
-    return launch_k(k_psi6_reduce, dim3(c.R), dim3(1024), 0, c.stream, c.reps, c.R, c.blocks_t32, partial, res);
+cudaError_t launch_psi6_reduce(const LaunchCfg& c, unsigned long long* total, double* res) {
+    return launch_k(k_psi6_reduce, dim3(c.R), dim3(32), 0, c.stream, c.reps, total, res);
 }
 
 }  // namespace hd
