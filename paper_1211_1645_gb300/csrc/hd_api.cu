@@ -230,13 +230,12 @@ void set_f32_bounds(Rep& r) {
     r.d2_hi = std::nextafter(float(4.0 + M), HUGE_VALF);
 }
 
-// The histogram's range [e0, eK) widened by the margin of pairs hist_R cells
-// apart, and the psi_6 margin (candidates two cells apart).
+// The histogram's range [e0, eK) (sigma units) widened by the margin of pairs
+// hist_R cells apart.
 void set_hist_f32_bounds(Rep& r, double e0, double eK) {
     const double M = hd::cells_f32_margin(r.w, r.hist_R);
     r.h_lo = std::nextafter(float(e0 - M), -HUGE_VALF);
     r.h_hi = std::nextafter(float(eK + M), HUGE_VALF);
-    r.psi_m = std::nextafter(float(hd::cells_f32_margin(r.w, 2)), HUGE_VALF);
 }
 
 // Tiles of every replica for the tile sweep (see hd_tile.h); false where it
@@ -318,6 +317,8 @@ hd_status plan_replica(int64_t N, double eta, double sigma, double delta, uint64
     r.LF = int64_t(m) * W;
     r.w = w;
     r.w_below = std::nextafter(w, 0.0);
+    r.w_inv = 1.0 / w;
+    r.wf_sigma = float(fixed ? double(W) / kFx : w);
     r.L = L;
     r.Lm = fixed ? double(r.LF) / kFx : L;
     r.delta = dhat;

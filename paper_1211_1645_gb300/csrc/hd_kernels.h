@@ -117,9 +117,9 @@ struct HistCfg {
     int halo;                 // largest histogram reach (cells) over the replicas
 };
 cudaError_t launch_hist(const LaunchCfg& c, const HistCfg& h, CellBufs cells, unsigned long long* hist);
-// The quartic fit's design matrix depends on K alone: launch_fit_factor
-// writes its Householder factor (fit_factor_len(K) doubles) once per context,
-// launch_fit applies it to each measurement.
+// The quartic fit's value at contact is linear in g(r), with weights that
+// depend on K alone: launch_fit_factor writes them (fit_factor_len(K) doubles)
+// once per context, launch_fit applies them to each measurement.
 size_t fit_factor_len(int K);
 cudaError_t launch_fit_factor(cudaStream_t s, int K, double* qr);
 cudaError_t launch_fit(const LaunchCfg& c, int K, const double* qr, const unsigned long long* hist, double* res);

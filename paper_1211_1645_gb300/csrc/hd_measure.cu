@@ -27,7 +27,7 @@ constexpr int kMaxFitBins = 512;
 // One thread per cell scans the (2R+1)^2 stencil; counts gather in a shared
 // histogram and are flushed with one atomic per non-empty bin and block.
 // k_hist_global reads the stencil from global memory (any reach R);
-// k_hist_tile (reach up to kHistMaxHalo) first stages the block's 32 x rows
+// k_hist_tile (reach up to kHistMaxHalo) first stages the block's 32 x 8
 // tile of cells and a halo of R cells in shared memory, like k_psi6.
 // ---------------------------------------------------------------------------
 template <bool FIX, int CAP>
@@ -131,21 +131,23 @@ __device__ __forceinline__ int tile_disk_list(const uint8_t* s_n, int SX, int ha
     return total;
 }
 
+constexpr int kTileThreads = 256;  // a 32 x 8 tile of cells, one thread per cell
+
 template <bool FIX, int CAP>
-__host__ __device__ constexpr size_t hist_stage_bytes(int rows, int halo, int K) {
-    return size_t(32 + 2 * halo) * size_t(rows + 2 * halo) * (CAP * (sizeof(P2<FIX>) + sizeof(int32_t)) + 1) + 16 +
-           size_t(K + 1) * 8 + size_t(K) * 4;
+__host__ __device__ constexpr size_t hist_stage_bytes(int halo, int K) {
+    return size_t(32 + 2 * halo) * size_t(kTileThreads / 32 + 2 * halo) *
+               (CAP * (sizeof(P2<FIX>) + (FIX ? 0 : sizeof(float2) + sizeof(int32_t))) + 1) +
+           16 + size_t(K + 1) * 8 + size_t(K) * 4;
 }
 
 // FP64 bin of a pair (o at cell offset (dcx, dcy) from me) among the K bins
-// of squared edges edge[0..K], or -1 outside [edge_0, edge_K).  Out of line,
-// so that its FP64 instructions issue only for the pairs the float pre-test
-// leaves; the non-negative squared distance is compared through its bit
-// pattern, which orders as the value does.
-static __device__ __noinline__ int hist_bin_fp64(double ox, double oy, double mx, double my, int dcx, int dcy,
-                                                 double w, const double* edge, int K) {
-    const double rx = __dsub_rn(__dadd_rn(ox, __dmul_rn(double(dcx), w)), mx);
-    const double ry = __dsub_rn(__dadd_rn(oy, __dmul_rn(double(dcy), w)), my);
+// of squared edges edge[0..K], or -1 outside [edge_0, edge_K); the non-negative
+// squared distance is compared through its bit pattern, which orders as the
+// value does.
+__device__ __forceinline__ int hist_bin_fp64(const double2& o, const double2& me, int dcx, int dcy, double w, const double* edge,
+                                             int K) {
+    const double rx = __dsub_rn(__dadd_rn(o.x, __dmul_rn(double(dcx), w)), me.x);
+    const double ry = __dsub_rn(__dadd_rn(o.y, __dmul_rn(double(dcy), w)), me.y);
     const long long b = __double_as_longlong(__dadd_rn(__dmul_rn(rx, rx), __dmul_rn(ry, ry)));
     if (b < __double_as_longlong(edge[0]) || b >= __double_as_longlong(edge[K])) return -1;
     int lo = 0, hi = K - 1;  // largest k with edge[k] <= r^2
@@ -156,8 +158,18 @@ static __device__ __noinline__ int hist_bin_fp64(double ox, double oy, double mx
     return lo;
 }
 
+// Each unordered pair is seen once, from the cell whose offset to the other is
+// in the upper half of the stencil, or within a cell from the lower slot.
+// Fixed form: binned where it is found, by its exact integer distance.
+// FP64 form: a pair whose float estimate of r^2 lies within the binned range
+// widened by its error bound (set_hist_f32_bounds) is queued, and a warp bins
+// its queue 32 pairs at a time by their exact squared distances in the lower
+// id's view, whose rounding the oracle follows: about one candidate in forty is
+// in the contact shell, so binning each where it was found ran its FP64
+// arithmetic once per such pair with one lane in it (57% of the FP64 pipe).
+// N = 2^20: FP64 133 -> 78 us; the fixed form 52, with the queue 59.
 template <bool FIX, int CAP>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kTileThreads)
 k_hist_tile(const Rep* __restrict__ reps, int R, int K, const double* __restrict__ edges,
             const long long* __restrict__ edgesF, const uint8_t* __restrict__ cnt, const P2<FIX>* __restrict__ pos,
             const int32_t* __restrict__ pid, unsigned long long* __restrict__ hist, int H) {
@@ -166,109 +178,142 @@ k_hist_tile(const Rep* __restrict__ reps, int R, int K, const double* __restrict
     const int r = find_rep<kGridT32>(reps, R, blockIdx.x);
     const Rep& rep = reps[r];
     const int m = rep.m;
-    const int rows = int(blockDim.x >> 5);
+    constexpr int rows = kTileThreads / 32;
     int X0, Y0;
     tile32_origin(rep, uint32_t(blockIdx.x - rep.blk_t32), rows, X0, Y0);
     const int SX = 32 + 2 * H, nS = SX * (rows + 2 * H);
-    P2<FIX>* s_pos = reinterpret_cast<P2<FIX>*>(s_raw);                  // [CAP][nS]
-    int32_t* s_id = reinterpret_cast<int32_t*>(s_pos + size_t(CAP) * nS);  // [CAP][nS]
-    uint8_t* s_n = reinterpret_cast<uint8_t*>(s_id + size_t(CAP) * nS);    // [nS]
+    P2<FIX>* s_pos = reinterpret_cast<P2<FIX>*>(s_raw);                      // [CAP][nS]
+    // FP64 form: float offsets and ids
+    float2* s_img = reinterpret_cast<float2*>(s_pos + size_t(CAP) * nS);                // [CAP][nS]
+    int32_t* s_id = reinterpret_cast<int32_t*>(s_img + (FIX ? 0 : size_t(CAP) * nS));   // [CAP][nS]
+    uint8_t* s_n = reinterpret_cast<uint8_t*>(s_id + (FIX ? 0 : size_t(CAP) * nS));     // [nS]
     using E = std::conditional_t<FIX, long long, double>;
-    E* s_edge = reinterpret_cast<E*>(s_raw + ((size_t(CAP) * nS * (sizeof(P2<FIX>) + 4) + nS + 15) & ~size_t(15)));
+    E* s_edge = reinterpret_cast<E*>(s_raw + ((size_t(CAP) * nS * (sizeof(P2<FIX>) + (FIX ? 0 : sizeof(float2) + 4)) + nS + 15) & ~size_t(15)));
     unsigned int* s_bins = reinterpret_cast<unsigned int*>(s_edge + (K + 1));
-    for (int b = threadIdx.x; b <= K; b += blockDim.x) {
+    for (int b = threadIdx.x; b <= K; b += kTileThreads) {
         if constexpr (FIX) s_edge[b] = edgesF[b];
         else s_edge[b] = edges[b];
         if (b < K) s_bins[b] = 0u;
     }
-    for (int t = threadIdx.x; t < nS; t += blockDim.x) {
+    for (int t = threadIdx.x; t < nS; t += kTileThreads) {
         const int sy = t / SX, sx = t - sy * SX;
         const uint32_t c = uint32_t(rep.coff) + row_part(rep, wrap_cell(Y0 - H + sy, m)) +
                            col_part(rep, wrap_cell(X0 - H + sx, m));
         const int n = min(int(cnt[c]), CAP);
         s_n[t] = uint8_t(n);
         for (int q = 0; q < n; ++q) {
-            s_pos[q * nS + t] = pos[size_t(q) * rep.stride32 + c];
-            s_id[q * nS + t] = pid[size_t(q) * rep.stride32 + c];
+            const P2<FIX> o = pos[size_t(q) * rep.stride32 + c];
+            s_pos[q * nS + t] = o;
+            if constexpr (!FIX) {
+                s_img[q * nS + t] = make_float2(approx_f32(o.x), approx_f32(o.y));
+                s_id[q * nS + t] = pid[size_t(q) * rep.stride32 + c];
+            }
         }
+        if (!FIX && n == 0) s_img[t] = make_float2(__uint_as_float(0x7F800000u), 0.0f);  // slot 0 is tested in any case
     }
     __syncthreads();
-    __shared__ uint16_t s_list[256 * CAP];
+    __shared__ uint16_t s_list[kTileThreads * CAP];
     __shared__ int s_warp[8];
     const int D = tile_disk_list(s_n, SX, H, X0, Y0, m, s_list, s_warp);
     const int RR = rep.hist_R;
-    const E lo_edge = s_edge[0], hi_edge = s_edge[K];
-    for (int d = threadIdx.x; d < D; d += blockDim.x) {
-        const int own = int(s_list[d] >> 4), k = int(s_list[d] & 15u);
-        const P2<FIX> me = s_pos[k * nS + own];
-        const int32_t idme = FIX ? 0 : s_id[k * nS + own];  // the FP64 form's pair rule
-        float mfx = 0.0f, mfy = 0.0f;  // FP64 form: float images of the disk's offsets
-        if constexpr (!FIX) {
-            mfx = approx_f32(me.x);
-            mfy = approx_f32(me.y);
-        }
-        // Each unordered pair once.  Fixed form: from the cell whose offset to
-        // the other is in the upper half of the stencil (dcy > 0, or dcy = 0
-        // and dcx > 0), or within a cell from the lower slot -- the squared
-        // distance is the same exact integer seen from either side, so the
-        // counts equal those of a lower-id rule.  FP64: from the lower id,
-        // whose rounding the oracle follows.
-        for (int dcy = FIX ? 0 : -RR; dcy <= RR; ++dcy) {
-            for (int dcx = (FIX && dcy == 0) ? 0 : -RR; dcx <= RR; ++dcx) {
-                const int sc = own + dcy * SX + dcx;
-                const int nn = s_n[sc];
-                for (int q = (FIX && dcy == 0 && dcx == 0) ? k + 1 : 0; q < nn; ++q) {
-                    if constexpr (!FIX) {
-                        if (s_id[q * nS + sc] <= idme) continue;
-                    }
-                    const P2<FIX> o = s_pos[q * nS + sc];
-                    E r2 = E(0);
-                    if constexpr (FIX) {
+    if constexpr (FIX) {
+        const long long lo_edge = s_edge[0], hi_edge = s_edge[K];
+        for (int d = threadIdx.x; d < D; d += kTileThreads) {
+            const int own = int(s_list[d] >> 4), k = int(s_list[d] & 15u);
+            const int2 me = s_pos[k * nS + own];
+            for (int dcy = 0; dcy <= RR; ++dcy) {
+                for (int dcx = dcy == 0 ? 0 : -RR; dcx <= RR; ++dcx) {
+                    const int sc = own + dcy * SX + dcx;
+                    const int nn = s_n[sc];
+                    for (int q = (dcy == 0 && dcx == 0) ? k + 1 : 0; q < nn; ++q) {
+                        const int2 o = s_pos[q * nS + sc];
                         // |offset| < (RR + 1) W <= 5 W < 2^31
-                        const int32_t rx = (o.x + dcx * rep.W) - me.x;
-                        const int32_t ry = (o.y + dcy * rep.W) - me.y;
-                        r2 = int64_t(rx) * rx + int64_t(ry) * ry;
-                    } else {
-                        // float pre-test (as pair_clear's): a pair whose float
-                        // estimate of r^2 lies outside the range widened by its
-                        // error bound is outside it in FP64 too
-                        const float sx = __fsub_rn(__fadd_rn(approx_f32(o.x), __fmul_rn(float(dcx), rep.wf)), mfx);
-                        const float sy = __fsub_rn(__fadd_rn(approx_f32(o.y), __fmul_rn(float(dcy), rep.wf)), mfy);
-                        const float d2f = __fadd_rn(__fmul_rn(sx, sx), __fmul_rn(sy, sy));
-                        if (d2f < rep.h_lo || d2f >= rep.h_hi) continue;
-                        const int bin = hist_bin_fp64(o.x, o.y, me.x, me.y, dcx, dcy, rep.w, s_edge, K);
-                        if (bin >= 0) atomicAdd(&s_bins[bin], 1u);
-                        continue;
+                        const int32_t rx = (o.x + dcx * rep.W) - me.x, ry = (o.y + dcy * rep.W) - me.y;
+                        const long long r2 = int64_t(rx) * rx + int64_t(ry) * ry;
+                        if (r2 < lo_edge || r2 >= hi_edge) continue;
+                        int lo = 0, hi = K - 1;  // largest k with edge[k] <= r2
+                        while (lo < hi) {
+                            const int mid = (lo + hi + 1) >> 1;
+                            if (s_edge[mid] <= r2) lo = mid; else hi = mid - 1;
+                        }
+                        atomicAdd(&s_bins[lo], 1u);
                     }
-                    if (r2 < lo_edge || r2 >= hi_edge) continue;
-                    int lo = 0, hi = K - 1;  // largest k with edge[k] <= r2
-                    while (lo < hi) {
-                        const int mid = (lo + hi + 1) >> 1;
-                        if (s_edge[mid] <= r2) lo = mid; else hi = mid - 1;
-                    }
-                    atomicAdd(&s_bins[lo], 1u);
                 }
             }
         }
+    } else {
+        __shared__ uint32_t s_queue[kTileThreads / 32][64];  // own entry | other entry << 16
+        const int lane = int(threadIdx.x & 31u), warp = int(threadIdx.x >> 5);
+        uint32_t* queue = s_queue[warp];
+        int queued = 0;  // the same in every lane
+        auto bin_queued = [&](int count) {
+            if (lane < count) {
+                const uint32_t v = queue[lane];
+                const int a = int(v & 0xFFFFu), b = int(v >> 16);  // entries slot * nS + cell
+                const int ca = a % nS, cb = b % nS;
+                const int dcy = cb / SX - ca / SX, dcx = cb % SX - ca % SX;
+                const double2 pa = s_pos[a], pb = s_pos[b];
+                const int bin = s_id[a] < s_id[b] ? hist_bin_fp64(pb, pa, dcx, dcy, rep.w, s_edge, K)
+                                                  : hist_bin_fp64(pa, pb, -dcx, -dcy, rep.w, s_edge, K);
+                if (bin >= 0) atomicAdd(&s_bins[bin], 1u);
+            }
+        };
+        for (int base = warp * 32; base < D; base += kTileThreads) {
+            const int d = base + lane;
+            const bool live = d < D;
+            const int own = live ? int(s_list[d] >> 4) : 0, k = live ? int(s_list[d] & 15u) : 0;
+            const int mine = k * nS + own;
+            const float2 me = s_img[mine];
+            for (int dcy = 0; dcy <= RR; ++dcy) {
+                const float by = __fmul_rn(float(dcy), rep.wf_sigma);
+                for (int dcx = dcy == 0 ? 0 : -RR; dcx <= RR; ++dcx) {
+                    const float bx = __fmul_rn(float(dcx), rep.wf_sigma);
+                    const bool same = dcx == 0 && dcy == 0;
+                    const int sc = live ? own + dcy * SX + dcx : 0;
+                    const int nn = s_n[sc];
+                    // slot 0 without a look at the occupancy, the others while any lane has one
+                    for (int q = 0;; ++q) {
+                        const float2 f = s_img[q * nS + sc];
+                        const float sx = __fsub_rn(__fadd_rn(f.x, bx), me.x), sy = __fsub_rn(__fadd_rn(f.y, by), me.y);
+                        const float d2f = __fadd_rn(__fmul_rn(sx, sx), __fmul_rn(sy, sy));
+                        const bool in = live && (q == 0 || q < nn) && (!same || q > k) && d2f >= rep.h_lo && d2f < rep.h_hi;
+                        const uint32_t who = __ballot_sync(0xffffffffu, in);
+                        if (who) {
+                            if (in) queue[queued + __popc(who & ((1u << lane) - 1u))] = uint32_t(mine) | uint32_t(q * nS + sc) << 16;
+                            queued += __popc(who);
+                            __syncwarp();
+                            if (queued >= 32) {
+                                bin_queued(32);
+                                __syncwarp();
+                                const uint32_t v = lane < queued - 32 ? queue[32 + lane] : 0u;
+                                __syncwarp();
+                                if (lane < queued - 32) queue[lane] = v;
+                                queued -= 32;
+                            }
+                        }
+                        if (q + 1 == CAP || !__any_sync(0xffffffffu, q + 1 < nn)) break;
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        bin_queued(queued);
     }
     __syncthreads();
-    for (int b = threadIdx.x; b < K; b += blockDim.x)
+    for (int b = threadIdx.x; b < K; b += kTileThreads)
         if (s_bins[b]) atomicAdd(&hist[size_t(r) * K + b], (unsigned long long)s_bins[b]);
 }
 
 // ---------------------------------------------------------------------------
 // g(r) normalisation (Eq. 2, p = N^2 / 2), least-squares quartic in
 // t = (r - 2 sigma) / (K dr) by Householder QR, value at contact, and the
-// contact-value pressure (Eq. 4).  The design matrix depends on K alone, so
-// k_fit_factor triangularises it once per context and k_fit applies the
-// stored reflectors to each measurement's g(r): the same operations, in the
-// same order, as a factorisation of [A | b] at every measurement.  One warp
-// per replica: the K rows are spread over the lanes and every column norm
-// and dot product is a warp sum.
-// Factor layout: [0, 5K) the K x 5 matrix row-major after triangularisation
-// (R on and above the diagonal, reflector j's tail below it); [5K, 5K + 5)
-// v0_j, the first element of reflector j; [5K + 5, 5K + 10) v_j^T v_j, 0 for a
-// column with zero norm (no reflector).
+// contact-value pressure (Eq. 4).  The design matrix A = Q R depends on K
+// alone, and the value at contact is linear in g(r): g(2 sigma+) = sum_k c_k
+// g(r_k) with c = Q (R^-T e_0).  k_fit_factor works c out once per context;
+// k_fit then takes one product sum per measurement, where applying the
+// reflectors and solving took a chain of five dot products (18 -> 5 us).
+// One warp: the K rows are spread over the lanes and every column norm and dot
+// product is a warp sum.
 // res[4r + 0..3] = beta P / rho, g(2 sigma+), P* = beta P (2 sigma)^2, eta.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double warp_sum(double v) {
@@ -277,8 +322,9 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-__global__ void __launch_bounds__(32) k_fit_factor(int K, double* __restrict__ qr) {
-    __shared__ double A[kMaxFitBins * 5];
+__global__ void __launch_bounds__(32) k_fit_factor(int K, double* __restrict__ weight) {
+    __shared__ double A[kMaxFitBins * 5], c[kMaxFitBins];
+    __shared__ double v0s[5], vtvs[5];
     const int lane = threadIdx.x;
     for (int k = lane; k < K; k += 32) {
         const double t = __ddiv_rn(__dadd_rn(double(k), 0.5), double(K));
@@ -293,14 +339,7 @@ __global__ void __launch_bounds__(32) k_fit_factor(int K, double* __restrict__ q
         double part = 0.0;
         for (int i = j + lane; i < K; i += 32) part = __dadd_rn(part, __dmul_rn(A[i * 5 + j], A[i * 5 + j]));
         const double nrm2 = warp_sum(part);
-        const double nrm = sqrt(nrm2);
-        if (nrm == 0.0) {
-            if (lane == 0) {
-                qr[5 * K + j] = 0.0;
-                qr[5 * K + 5 + j] = 0.0;
-            }
-            continue;
-        }
+        const double nrm = sqrt(nrm2);  // positive: the columns are independent for K >= 5
         const double ajj = A[j * 5 + j];
         const double alpha = ajj > 0.0 ? -nrm : nrm;
         const double v0 = __dsub_rn(ajj, alpha);
@@ -317,49 +356,49 @@ __global__ void __launch_bounds__(32) k_fit_factor(int K, double* __restrict__ q
         }
         if (lane == 0) {
             A[j * 5 + j] = alpha;  // R diagonal
-            qr[5 * K + j] = v0;
-            qr[5 * K + 5 + j] = vtv;
+            v0s[j] = v0;
+            vtvs[j] = vtv;
         }
         __syncwarp();
     }
-    for (int i = lane; i < 5 * K; i += 32) qr[i] = A[i];
+    // y = R^-T e_0, then c = H_0 H_1 .. H_4 (y, 0)
+    for (int k = lane; k < K; k += 32) c[k] = 0.0;
+    __syncwarp();
+    if (lane == 0)
+        for (int i = 0; i < 5; ++i) {
+            double acc = i == 0 ? 1.0 : 0.0;
+            for (int q = 0; q < i; ++q) acc = __dsub_rn(acc, __dmul_rn(A[q * 5 + i], c[q]));
+            c[i] = __ddiv_rn(acc, A[i * 5 + i]);
+        }
+    __syncwarp();
+    for (int j = 4; j >= 0; --j) {
+        double dp = 0.0;
+        for (int i = j + lane; i < K; i += 32) dp = __dadd_rn(dp, __dmul_rn(i == j ? v0s[j] : A[i * 5 + j], c[i]));
+        const double sc = __ddiv_rn(__dmul_rn(2.0, warp_sum(dp)), vtvs[j]);
+        for (int i = j + lane; i < K; i += 32) c[i] = __dsub_rn(c[i], __dmul_rn(sc, i == j ? v0s[j] : A[i * 5 + j]));
+        __syncwarp();
+    }
+    for (int k = lane; k < K; k += 32) weight[k] = c[k];
 }
 
-__global__ void __launch_bounds__(32) k_fit(const Rep* __restrict__ reps, int K, const double* __restrict__ qr,
+__global__ void __launch_bounds__(32) k_fit(const Rep* __restrict__ reps, int K, const double* __restrict__ weight,
                                             const unsigned long long* __restrict__ hist, double* __restrict__ res) {
     pdl_begin();
-    __shared__ double b[kMaxFitBins];
     const int r = blockIdx.x, lane = threadIdx.x;
     const Rep& rep = reps[r];
     const double PI = 3.14159265358979323846;
     const double V = __dmul_rn(rep.Lm, rep.Lm);
     const double p = __dmul_rn(__dmul_rn(double(rep.N), double(rep.N)), 0.5);
     const double dr = rep.dr;
+    double part = 0.0;
     for (int k = lane; k < K; k += 32) {
         const double rk = __dadd_rn(2.0, __dmul_rn(__dadd_rn(double(k), 0.5), dr));
         const double shell = __ddiv_rn(__dmul_rn(__dmul_rn(__dmul_rn(2.0, PI), rk), dr), V);
-        b[k] = __ddiv_rn(__ddiv_rn(double(hist[size_t(r) * K + k]), p), shell);
+        const double g = __ddiv_rn(__ddiv_rn(double(hist[size_t(r) * K + k]), p), shell);
+        part = __dadd_rn(part, __dmul_rn(weight[k], g));
     }
-    __syncwarp();
-    // b <- Q^T b, reflector by reflector
-    for (int j = 0; j < 5; ++j) {
-        const double vtv = qr[5 * K + 5 + j];
-        if (vtv == 0.0) continue;
-        const double v0 = qr[5 * K + j];
-        double dp = 0.0;
-        for (int i = j + lane; i < K; i += 32) dp = __dadd_rn(dp, __dmul_rn(i == j ? v0 : qr[i * 5 + j], b[i]));
-        const double sc = __ddiv_rn(__dmul_rn(2.0, warp_sum(dp)), vtv);
-        for (int i = j + lane; i < K; i += 32) b[i] = __dsub_rn(b[i], __dmul_rn(sc, i == j ? v0 : qr[i * 5 + j]));
-        __syncwarp();
-    }
+    const double g0 = warp_sum(part);
     if (lane != 0) return;
-    double coef[5];
-    for (int j = 4; j >= 0; --j) {
-        double acc = b[j];
-        for (int q = j + 1; q < 5; ++q) acc = __dsub_rn(acc, __dmul_rn(qr[j * 5 + q], coef[q]));
-        coef[j] = __ddiv_rn(acc, qr[j * 5 + j]);
-    }
-    const double g0 = coef[0];
     const double eta = __ddiv_rn(__dmul_rn(double(rep.N), PI), V);
     const double bp = __dadd_rn(1.0, __dmul_rn(__dmul_rn(2.0, eta), g0));
     res[4 * r + 0] = bp;
@@ -466,7 +505,7 @@ __device__ __forceinline__ bool ring_covers(const Rep& rep, const Nbr<FIX>& nb, 
 // cells plus a halo of two cells (the 5 x 5 stencil of every tile cell).
 constexpr int kPsiHalo = 2;
 constexpr int kPsiSX = 32 + 2 * kPsiHalo;
-constexpr int kPsiThreads = 256;  // a tile of eight rows: 1.7 staged cells per cell
+constexpr int kPsiThreads = kTileThreads;  // eight rows: 1.7 staged cells per cell
 
 template <bool FIX, int CAP>
 __host__ __device__ constexpr size_t psi6_stage_bytes(int rows) {
@@ -825,10 +864,10 @@ static cudaError_t hist_t(const LaunchCfg& c, const HistCfg& h, CellBufs cells, 
         static std::once_flag attr_once;
         std::call_once(attr_once, [] {
             cudaFuncSetAttribute(k_hist_tile<FIX, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 int(hist_stage_bytes<FIX, CAP>(8, kHistMaxHalo, kMaxFitBins)));
+                                 int(hist_stage_bytes<FIX, CAP>(kHistMaxHalo, kMaxFitBins)));
         });
-        return launch_k(k_hist_tile<FIX, CAP>, dim3(c.blocks_t32), dim3(kPsiThreads),
-                        hist_stage_bytes<FIX, CAP>(kPsiThreads / 32, h.halo, h.K), c.stream, c.reps, c.R, h.K, h.edges,
+        return launch_k(k_hist_tile<FIX, CAP>, dim3(c.blocks_t32), dim3(kTileThreads),
+                        hist_stage_bytes<FIX, CAP>(h.halo, h.K), c.stream, c.reps, c.R, h.K, h.edges,
                         h.edgesF, (const uint8_t*)cells.cnt, (const P2<FIX>*)cells.pos, (const int32_t*)cells.pid,
                         hist, h.halo);
     }
@@ -842,7 +881,7 @@ cudaError_t launch_hist(const LaunchCfg& c, const HistCfg& h, CellBufs cells, un
     return c.cap == 4 ? hist_t<false, 4>(c, h, cells, hist) : hist_t<false, 9>(c, h, cells, hist);
 }
 
-size_t fit_factor_len(int K) { return size_t(5 * K + 10); }
+size_t fit_factor_len(int K) { return size_t(K); }
 
 cudaError_t launch_fit_factor(cudaStream_t s, int K, double* qr) {
     if (K < 5 || K > kMaxFitBins) return cudaErrorInvalidValue;
