@@ -234,7 +234,7 @@ __device__ __forceinline__ void visit_cell(const S& st, const TileRep<FIX>& rep,
     if ((w & 15u) == 0u) return;
     const uint32_t cl = (2u * gy + uint32_t(py)) * (2u * hm) + 2u * gx + uint32_t(px);
     P2<FIX>* pos = static_cast<P2<FIX>*>(it.to.pos);
-    const uint32_t got = tile_cell<FIX, NTC, HARD, S>(st, rep, it.sweep, px, py, hx, hy, w, cl,
+    const uint32_t got = tile_cell<FIX, NTC, HARD, false, S>(st, rep, it.sweep, px, py, hx, hy, w, cl,
                                                       [&](int k, const P2<FIX>& q, int32_t id) {
                                                           if (own) {
                                                               pos[size_t(k) * it.stride + cell] = q;
@@ -496,7 +496,10 @@ k_sweep_tile(const Rep* __restrict__ reps, const TileGrid* __restrict__ grids, i
 // opposite sides, filled after a rebuild and kept up by the thread that moves
 // a disk of an edge cell, so that the passes are those of the tiles.  A
 // launch boundary between phases costs 2 to 4 us, here a phase is one block
-// barrier: what bounds a sweep is the latency of five dependent phases.
+// barrier: what bounds a sweep is the latency of five dependent phases.  The
+// draws of the next sweep's trials (generator, step, swap word: a third of a
+// pass's chain) are therefore made by warps of their own while the others
+// sweep.
 // ---------------------------------------------------------------------------
 template <bool FIX, int HB>
 using BoxStage = Stage<FIX, HB, HB, 64>;
@@ -518,8 +521,14 @@ __device__ __forceinline__ void copy_cell(const S& st, int from, int to) {
             if (((w >> (k == 2 ? 12 : 22)) & 0x3FFu) == kFar) *st.extra(w, to, k) = *st.extra(w, from, k);
 }
 
+template <bool FIX, int HB>
+constexpr size_t box_smem() {
+    return 2 * BoxStage<FIX, HB>::kBytes + size_t(2) * BoxStage<FIX, HB>::NC * (sizeof(P2<FIX>) + 4);
+}
+constexpr int kBoxDrawThreads = 128;
+
 template <bool FIX, int NTC, int HB, int NT>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(NT + kBoxDrawThreads)
 k_sweep_box(const Rep* __restrict__ reps, const Frame* __restrict__ table, int nsweeps, CellBufs g0, CellBufs g1,
             unsigned long long* __restrict__ counters, int* __restrict__ err, void* spill) {
     using S = BoxStage<FIX, HB>;
@@ -544,10 +553,46 @@ k_sweep_box(const Rep* __restrict__ reps, const Frame* __restrict__ table, int n
         ly = 2 * int(row) + int(pl >> 1) + 2;
     };
     auto wrap_local = [m](int v) { return v < 2 ? v + m : (v >= m + 2 ? v - m : v); };
+    // [2][NC] steps, then swap words, by entry of the stage
+    P2<FIX>* s_step = reinterpret_cast<P2<FIX>*>(s_raw + 2 * S::kBytes);
+    uint32_t* s_swap = reinterpret_cast<uint32_t*>(s_step + 2 * S::NC);
+    // frame changes of two sweeps, read ahead
+    struct Change {
+        double dx, dy;
+        int32_t fx, fy;
+        uint32_t sweep, perm;
+    };
+    __shared__ Change s_change[2];
+    auto read_change = [&](int i) {
+        const Frame fn = tab[i + 1];
+        const ShiftDelta<FIX> sd(tab[i], fn);
+        s_change[i & 1] = Change{sd.dx, sd.dy, sd.fx, sd.fy, fn.sweep, fn.perm};
+    };
+    if (tid >= NT) {  // the draws of sweep i and the frame change of sweep i + 1 are ready at barrier i
+        if (tid == NT) read_change(0);
+        __syncthreads();
+        for (int i = 0; i < nsweeps; ++i) {
+            const uint32_t sweep = s_change[i & 1].sweep;
+            if (tid == NT && i + 1 < nsweeps) read_change(i + 1);
+            for (uint32_t e = uint32_t(tid - NT); e < 4u * hh; e += kBoxDrawThreads) {
+                int lx, ly;
+                local(e, lx, ly);
+                const uint32_t cl = uint32_t(ly - 2) * uint32_t(m) + uint32_t(lx - 2);
+                const int at = (i & 1) * S::NC + S::index(lx, ly);
+                const uint4 u = philox(sweep, 0u, cl, kTagTrial, rep.key0, rep.key1);
+                s_step[at] = trial_step<FIX>(rep, u);
+                s_swap[at] = FIX ? u.z : philox(sweep, 0u, cl, kTagShuffle, rep.key0, rep.key1).x;
+            }
+            __syncthreads();
+        }
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        return;
+    }
+    auto sync_sweepers = [] { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); };
     {
         const S st(s_raw, far);
         clear_stage(st, hm + 2, tid, NT);
-        __syncthreads();
+        sync_sweepers();
         for (uint32_t e = uint32_t(tid); e < 4u * hh; e += NT) {
             int lx, ly;
             local(e, lx, ly);
@@ -558,14 +603,13 @@ k_sweep_box(const Rep* __restrict__ reps, const Frame* __restrict__ table, int n
                          g0.pid[size_t(k) * stride + c]);
         }
     }
-    Frame fo = tab[0], fn = tab[1];
+    __syncthreads();
     for (int i = 0; i < nsweeps; ++i) {
         const S old(s_raw + (i & 1 ? S::kBytes : 0), far + (i & 1 ? 2 * S::NC : 0));
         const S st(s_raw + (i & 1 ? 0 : S::kBytes), far + (i & 1 ? 0 : 2 * S::NC));
-        const ShiftDelta<FIX> sd(fo, fn);
-        const Frame ahead = tab[min(i + 2, nsweeps)];  // in flight during the sweep
+        const Change sd = s_change[i & 1];
         clear_stage(st, hm + 2, tid, NT);
-        __syncthreads();
+        sync_sweepers();
         // ---- move every disk into the new frame -------------------------------
         for (uint32_t e = uint32_t(tid); e < 4u * hh; e += NT) {
             int lx, ly;
@@ -596,7 +640,7 @@ k_sweep_box(const Rep* __restrict__ reps, const Frame* __restrict__ table, int n
                 over |= !st.place(x, y, S::index(x, y), p, id);
             }
         }
-        __syncthreads();
+        sync_sweepers();
         // ---- the neighbours of crowded cells, and the hard cells ---------------
         const uint32_t pooled = *st.pool_n;
         if (pooled != 0u) {
@@ -611,7 +655,7 @@ k_sweep_box(const Rep* __restrict__ reps, const Frame* __restrict__ table, int n
             }
             // a pool that overflowed: every cell looks at its neighbours itself
             if (pooled > uint32_t(S::POOL)) {
-                __syncthreads();
+                sync_sweepers();
                 for (uint32_t e = uint32_t(tid); e < 4u * hh; e += NT) {
                     int lx, ly;
                     local(e, lx, ly);
@@ -624,7 +668,7 @@ k_sweep_box(const Rep* __restrict__ reps, const Frame* __restrict__ table, int n
                     if (bits) atomicOr(&st.word[S::index(lx, ly)], bits);
                 }
             }
-            __syncthreads();
+            sync_sweepers();
         }
         // ---- the ring around the box -------------------------------------------
         for (int t = tid; t < 4 * (m + 1); t += NT) {
@@ -635,37 +679,47 @@ k_sweep_box(const Rep* __restrict__ reps, const Frame* __restrict__ table, int n
             st.word[to] = st.word[from];
             copy_cell<FIX, S>(st, from, to);
         }
-        __syncthreads();
+        __syncthreads();  // and this sweep's draws are made
         // ---- the four colour passes --------------------------------------------
         const bool every = st.hard_n[4] != 0u;
 #pragma unroll 1
         for (int p = 0; p < 4; ++p) {
-            const int col = int(fn.perm >> (2 * p)) & 3, px = col & 1, py = col >> 1;
+            const int col = int(sd.perm >> (2 * p)) & 3, px = col & 1, py = col >> 1;
             auto visit = [&](auto hard, int hx, int hy) {
                 const int e = col * S::NP + hy * S::HP + hx;
                 const uint32_t w = st.word[e];
                 if (is_hard(w) != hard.value || (w & 15u) == 0u) return;
                 const uint32_t cx = uint32_t(2 * hx + px - 2), cy = uint32_t(2 * hy + py - 2);
-                const uint32_t got = tile_cell<FIX, NTC, hard.value, S>(
-                    st, rep, fn.sweep, px, py, hx, hy, w, cy * uint32_t(m) + cx, [&](int k, const P2<FIX>& q, int32_t id) {
-                        // in id order, ids and positions together
-                        if (k < 2) {
-                            st.set(e, k, q);
-                            reinterpret_cast<int32_t*>(st.id)[2 * e + k] = id;
-                        } else {
-                            st.extra(w, e, k)->p = q;
-                            st.extra(w, e, k)->id = id;
-                        }
-                    });
-                att += uint32_t(rep.nt);
-                acc += got;
                 // an edge cell's copies in the ring
                 const int gx = cx == 0u ? m + 2 : (cx == uint32_t(m - 1) ? 1 : 0);
                 const int gy = cy == 0u ? m + 2 : (cy == uint32_t(m - 1) ? 1 : 0);
                 const int lx = int(cx) + 2, ly = int(cy) + 2;
-                if (gx) copy_cell<FIX, S>(st, e, S::index(gx, ly));
-                if (gy) copy_cell<FIX, S>(st, e, S::index(lx, gy));
-                if (gx && gy) copy_cell<FIX, S>(st, e, S::index(gx, gy));
+                const int at = (i & 1) * S::NC + e;
+                const uint32_t got = tile_cell<FIX, NTC, hard.value, true, S>(
+                    st, rep, sd.sweep, px, py, hx, hy, w, cy * uint32_t(m) + cx,
+                    [&](int k, const P2<FIX>& q, int32_t id) {
+                        // in id order, ids and positions together
+                        if (k < 2) {
+                            const typename S::Stored v = st.stored(q);
+                            st.set(e, k, v);
+                            reinterpret_cast<int32_t*>(st.id)[2 * e + k] = id;
+                            if (gx) st.set(S::index(gx, ly), k, v);
+                            if (gy) st.set(S::index(lx, gy), k, v);
+                            if (gx && gy) st.set(S::index(gx, gy), k, v);
+                        } else {
+                            PoolEntry<FIX>* x = st.extra(w, e, k);
+                            x->p = q;
+                            x->id = id;
+                            if (x >= st.spill && x < st.spill + 2 * S::NC) {  // the copies share a pool entry, not the spill area's
+                                if (gx) st.extra(w, S::index(gx, ly), k)->p = q;
+                                if (gy) st.extra(w, S::index(lx, gy), k)->p = q;
+                                if (gx && gy) st.extra(w, S::index(gx, gy), k)->p = q;
+                            }
+                        }
+                    },
+                    Drawn<FIX>{s_step[at], s_swap[at]});
+                att += uint32_t(rep.nt);
+                acc += got;
             };
             const uint32_t nhard = every ? hh : st.hard_n[col];
             for (uint32_t h = uint32_t(tid); h < nhard; h += NT) {
@@ -683,10 +737,8 @@ k_sweep_box(const Rep* __restrict__ reps, const Frame* __restrict__ table, int n
                 const uint32_t row = div_by(h, hm_mul, hm_sh);
                 visit(std::false_type{}, int(h - row * uhm) + 1, int(row) + 1);
             }
-            __syncthreads();
+            sync_sweepers();
         }
-        fo = fn;
-        fn = ahead;
     }
     // ---- the final state into the generation of the last sweep ------------------
     {
@@ -751,12 +803,12 @@ cudaError_t tile_t(const LaunchCfg& c, const TileCfg& t, const Frame* table, int
 template <bool FIX, int NTC, int HB, int NT>
 cudaError_t box_t(const LaunchCfg& c, void* spill, const Frame* table, int nsweeps, CellBufs a, CellBufs b,
                   unsigned long long* counters, int* err) {
-    constexpr size_t smem = 2 * BoxStage<FIX, HB>::kBytes;
+    constexpr size_t smem = box_smem<FIX, HB>();
     static std::once_flag attr_once;
     std::call_once(attr_once, [] {
         cudaFuncSetAttribute(k_sweep_box<FIX, NTC, HB, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     });
-    return launch_k(k_sweep_box<FIX, NTC, HB, NT>, dim3(c.R), dim3(NT), smem, c.stream, c.reps, table, nsweeps, a, b,
+    return launch_k(k_sweep_box<FIX, NTC, HB, NT>, dim3(c.R), dim3(NT + kBoxDrawThreads), smem, c.stream, c.reps, table, nsweeps, a, b,
                     counters, err, spill);
 }
 

@@ -121,6 +121,19 @@ struct Stage {
         if constexpr (FIX) low[2 * e + k] = uint8_t((p.x & 3) | (p.y & 3) << 2);
         else p0[k * NC + e] = p;
     }
+    // The same in several entries: what is stored of a position, made once.
+    struct Stored {
+        float2 f;
+        P2<FIX> p;
+    };
+    __device__ __forceinline__ Stored stored(const P2<FIX>& p) const {
+        return Stored{make_float2(image<FIX>(p.x), image<FIX>(p.y)), p};
+    }
+    __device__ __forceinline__ void set(int e, int k, const Stored& v) const {
+        reinterpret_cast<float2*>(quad)[2 * e + k] = v.f;
+        if constexpr (FIX) low[2 * e + k] = uint8_t((v.p.x & 3) | (v.p.y & 3) << 2);
+        else p0[k * NC + e] = v.p;
+    }
     // Claim a slot of local cell (lx, ly), entry e, for disk (p, i); false if the cell is full.
     __device__ __forceinline__ bool place(int lx, int ly, int e, const P2<FIX>& p, int32_t i) const {
         const uint32_t s = atomicAdd(&word[e], 1u) & 0xFu;
@@ -337,15 +350,35 @@ static __device__ __noinline__ void put_many(const S& st, int e, uint32_t w, int
     }
 }
 
+// The draws of a cell's first trial, made ahead: the step, and the word that
+// decides the shuffle of two occupants.
+template <bool FIX>
+__device__ __forceinline__ P2<FIX> trial_step(const TileRep<FIX>& rep, const uint4& u) {
+    if constexpr (FIX) {
+        const uint32_t span = uint32_t(2 * rep.D + 1);
+        return make_int2(int32_t(bounded(u.x, span)) - rep.D, int32_t(bounded(u.y, span)) - rep.D);
+    } else {
+        return make_double2(step_fp64(u.x, u.y, rep.delta), step_fp64(u.z, u.w, rep.delta));
+    }
+}
+template <bool FIX>
+struct Drawn {
+    P2<FIX> step;
+    uint32_t swap;
+};
+
 // One active cell: plane (px, py), half-row hy, half-column hx, word w, Philox
 // cell counter cl.  Its occupants are ordered by id, shuffled and make rep.nt
 // serial trial moves, as try_cell_in defines.  Cells of one or two disks keep
 // them in registers; the few with more take their moving disk from per-thread
-// memory.  HARD = false: the cell is known not to be hard.  emit(k, position, id) is called for every occupant
+// memory.  HARD = false: the cell is known not to be hard.  PRE: the first
+// trial's draws are given; the caller's emit stores the positions of slots 0
+// and 1 in the stage.  emit(k, position, id) is called for every occupant
 // afterwards.  Returns the accepted moves.
-template <bool FIX, int NTC, bool HARD, class S, class Emit>
+template <bool FIX, int NTC, bool HARD, bool PRE, class S, class Emit>
 __device__ __forceinline__ uint32_t tile_cell(const S& st, const TileRep<FIX>& rep, uint32_t sweep, int px, int py, int hx,
-                                              int hy, uint32_t w, uint32_t cl, Emit&& emit) {
+                                              int hy, uint32_t w, uint32_t cl, Emit&& emit,
+                                              const Drawn<FIX>& pre = Drawn<FIX>{}) {
     const int e = ((py << 1) | px) * S::NP + hy * S::HP + hx;
     const int n = min(int(w & 15u), 4);
     const bool two = n == 2, many = HARD && n > 2;
@@ -371,7 +404,10 @@ __device__ __forceinline__ uint32_t tile_cell(const S& st, const TileRep<FIX>& r
     // Fisher-Yates of two: position 0 takes slot 1 when the swap word's bound is 0
     uint4 u0 = make_uint4(0u, 0u, 0u, 0u);
     bool flip = false;
-    if constexpr (FIX) {
+    if constexpr (PRE) {
+        flip = two && (pre.swap >> 31) == 0u;
+        if (FIX && many) u0 = philox(sweep, 0u, cl, kTagTrial, rep.key0, rep.key1);
+    } else if constexpr (FIX) {
         u0 = philox(sweep, 0u, cl, kTagTrial, rep.key0, rep.key1);
         flip = two && (u0.z >> 31) == 0u;
     } else if (two) {
@@ -387,7 +423,9 @@ __device__ __forceinline__ uint32_t tile_cell(const S& st, const TileRep<FIX>& r
     uint32_t acc = 0;
     const int nt = NTC > 0 ? NTC : rep.nt;
     for (int t = 0; t < nt; ++t) {
-        const uint4 u = (FIX && t == 0) ? u0 : philox(sweep, uint32_t(t), cl, kTagTrial, rep.key0, rep.key1);
+        P2<FIX> step;
+        if (PRE && t == 0) step = pre.step;
+        else step = trial_step<FIX>(rep, (FIX && !PRE && t == 0) ? u0 : philox(sweep, uint32_t(t), cl, kTagTrial, rep.key0, rep.key1));
         const bool second = two && (((t & 1) != 0) != flip);
         P2<FIX> me = second ? q1 : q0, other = second ? q0 : q1;
         int slot = 0;
@@ -398,13 +436,12 @@ __device__ __forceinline__ uint32_t tile_cell(const S& st, const TileRep<FIX>& r
         P2<FIX> np;
         bool ok;
         if constexpr (FIX) {
-            const uint32_t span = uint32_t(2 * rep.D + 1);
-            np.x = me.x + (int32_t(bounded(u.x, span)) - rep.D);
-            np.y = me.y + (int32_t(bounded(u.y, span)) - rep.D);
+            np.x = me.x + step.x;
+            np.y = me.y + step.y;
             ok = uint32_t(np.x) < uint32_t(rep.W) && uint32_t(np.y) < uint32_t(rep.W);
         } else {
-            np.x = __dadd_rn(me.x, step_fp64(u.x, u.y, rep.delta));
-            np.y = __dadd_rn(me.y, step_fp64(u.z, u.w, rep.delta));
+            np.x = __dadd_rn(me.x, step.x);
+            np.y = __dadd_rn(me.y, step.y);
             ok = nonneg_bits(np.x) && below_pos_bits(np.x, rep.w) && nonneg_bits(np.y) && below_pos_bits(np.y, rep.w);
         }
         if (ok) ok = tile_clear<FIX, S>(st, rep, nb, np, other, two, crowd, 2 * hx + px, 2 * hy + py);
@@ -422,7 +459,7 @@ __device__ __forceinline__ uint32_t tile_cell(const S& st, const TileRep<FIX>& r
         for (int k = 0; k < n; ++k) emit(k, P[k], I[k]);
         return acc;
     }
-    if (acc) {
+    if (!PRE && acc) {
         st.set(e, 0, q0);
         if (two) st.set(e, 1, q1);
     }
