@@ -677,8 +677,11 @@ static __device__ __noinline__ int2 corr_exact(double2 pn, double2 pm, double L,
     return make_int2(a, b);
 }
 
-// blockIdx.y: replica, blockIdx.x: cells_per_block of its cells (planar order).
-// acc[r][interval] = (sum of Re, pairs).
+// blockIdx.y: replica, blockIdx.x: cells_per_block of its cells (planar order),
+// blockIdx.z: every gridDim.z-th row of the stencil (a small system's blocks
+// alone leave the GPU idle).  acc[r][interval] = (sum of Re, pairs).  What
+// bounds it is the latency of a neighbour cell's loads, so four cells' are in
+// flight at a time.
 template <int CAP, int NT>
 __global__ void __launch_bounds__(NT)
 k_corr_pairs(const Rep* __restrict__ reps, const uint8_t* __restrict__ cnt, const double2* __restrict__ gpos,
@@ -732,36 +735,55 @@ k_corr_pairs(const Rep* __restrict__ reps, const uint8_t* __restrict__ cnt, cons
         const size_t me = size_t(slot) * rep.stride32 + rep.coff + a;
         const float2 un = off[me];
         const double2 cn = chi[me];
-        for (int dcy = 0; dcy <= reach; ++dcy) {
+        auto pair = [&](size_t at, const float2& um, const double2& cm, float bx, float by) {
+            const float sx = __fadd_rn(um.x, bx), sy = __fadd_rn(um.y, by);
+            const float dist = sqrtf(__fadd_rn(__fmul_rn(sx, sx), __fmul_rn(sy, sy)));
+            const float fu = __fmul_rn(__fadd_rn(dist, 1.0f), inv), fv = __fmul_rn(__fsub_rn(dist, 1.0f), inv);
+            int wa = int(fminf(floorf(fu), float(nr))), wb = int(fminf(fmaxf(ceilf(fv) - 1.0f, 0.0f), float(nr)));
+            // (false also where a window width out of float's range made the estimate infinite)
+            const bool sure = eps < 0.25f && fabsf(fu - rintf(fu)) >= eps && fabsf(fv - rintf(fv)) >= eps;
+            if (!sure) {
+                const int2 e = corr_exact(gpos[me], gpos[at], L, nr, dr, wa, wb);
+                wa = e.x;
+                wb = e.y;
+            }
+            if (wa <= wb) return;
+            const int s = (wa + wb) * NT + tid;
+            s_sum[s] = __dadd_rn(s_sum[s], __fma_rn(cn.x, cm.x, __dmul_rn(cn.y, cm.y)));
+            s_cnt[s] += 1u;
+        };
+        for (int dcy = int(blockIdx.z); dcy <= reach; dcy += int(gridDim.z)) {
             const int y = cy + dcy >= m ? cy + dcy - m : cy + dcy;
             const uint32_t row = rep.coff + row_part(rep, y);
             const float gy = fmaxf(float(dcy - 1), 0.0f) * wf;
             const float by = __fsub_rn(__fmul_rn(float(dcy), wf), un.y);
-            for (int dcx = dcy == 0 ? 0 : -reach; dcx <= reach; ++dcx) {
-                const float gx = fmaxf(fabsf(float(dcx)) - 1.0f, 0.0f) * wf;
-                if (gx * gx + gy * gy > (rmax + 0.01f) * (rmax + 0.01f)) continue;  // no point of the cell is in reach
-                const uint32_t c = row + col_part(rep, wrap_cell(cx + dcx, m));
-                const int n = min(int(cnt[c]), CAP);
-                const float bx = __fsub_rn(__fmul_rn(float(dcx), wf), un.x);
-                for (int q = (dcx == 0 && dcy == 0) ? slot + 1 : 0; q < n; ++q) {
-                    const size_t at = size_t(q) * rep.stride32 + c;
-                    const float2 um = off[at];
-                    const float sx = __fadd_rn(um.x, bx), sy = __fadd_rn(um.y, by);
-                    const float dist = sqrtf(__fadd_rn(__fmul_rn(sx, sx), __fmul_rn(sy, sy)));
-                    const float fu = __fmul_rn(__fadd_rn(dist, 1.0f), inv), fv = __fmul_rn(__fsub_rn(dist, 1.0f), inv);
-                    int wa = int(fminf(floorf(fu), float(nr))), wb = int(fminf(fmaxf(ceilf(fv) - 1.0f, 0.0f), float(nr)));
-                    // (false also where a window width out of float's range made the estimate infinite)
-                    const bool sure = eps < 0.25f && fabsf(fu - rintf(fu)) >= eps && fabsf(fv - rintf(fv)) >= eps;
-                    if (!sure) {
-                        const int2 e = corr_exact(gpos[me], gpos[at], L, nr, dr, wa, wb);
-                        wa = e.x;
-                        wb = e.y;
+            // cells of the row with a point in reach
+            const float gx2 = (rmax + 0.01f) * (rmax + 0.01f) - gy * gy;
+            const int half = gx2 < 0.0f ? -1 : min(reach, int(sqrtf(gx2) / wf) + 2);
+            for (int x0 = dcy == 0 ? 0 : -half; x0 <= half; x0 += 4) {
+                uint32_t c[4];
+                int n[4];
+                float2 um[4];
+                double2 cm[4];
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    n[h] = 0;
+                    if (x0 + h <= half) {
+                        c[h] = row + col_part(rep, wrap_cell(cx + x0 + h, m));
+                        n[h] = min(int(cnt[c[h]]), CAP);
+                        um[h] = off[c[h]];
+                        cm[h] = chi[c[h]];
                     }
-                    if (wa <= wb) continue;
-                    const double2 cm = chi[at];
-                    const int s = (wa + wb) * NT + tid;
-                    s_sum[s] = __dadd_rn(s_sum[s], __fma_rn(cn.x, cm.x, __dmul_rn(cn.y, cm.y)));
-                    s_cnt[s] += 1u;
+                }
+#pragma unroll
+                for (int h = 0; h < 4; ++h) {
+                    const bool same = dcy == 0 && x0 + h == 0;
+                    const float bx = __fsub_rn(__fmul_rn(float(x0 + h), wf), un.x);
+                    if (n[h] > 0 && !same) pair(c[h], um[h], cm[h], bx, by);
+                    for (int q = same ? slot + 1 : 1; q < n[h]; ++q) {
+                        const size_t at = size_t(q) * rep.stride32 + c[h];
+                        pair(at, off[at], chi[at], bx, by);
+                    }
                 }
             }
         }
@@ -789,18 +811,38 @@ k_corr_pairs(const Rep* __restrict__ reps, const uint8_t* __restrict__ cnt, cons
 // first: d^2 on both is above the lower and not above the upper).
 __global__ void __launch_bounds__(128)
 k_corr_windows(int nr, double dr, const double2* __restrict__ acc, double2* __restrict__ out) {
+    extern __shared__ double2 s_acc2[];  // [2 nr + 1] sums, then [2 nr] bounds
     pdl_begin();
-    const int r = blockIdx.y, k = int(blockIdx.x * blockDim.x + threadIdx.x);
-    if (k >= nr) return;
-    const double2* p = acc + size_t(r) * (2 * nr + 1);
-    double s = 0.0, c = 0.0;
-    int a = 0, b = 0;
-    for (int i = 0; i <= 2 * nr; ++i) {
-        if (b <= k && k < a) {
-            s = __dadd_rn(s, p[i].x);
-            c = __dadd_rn(c, p[i].y);
+    const int r = blockIdx.y, bins = 2 * nr + 1, k = int(blockIdx.x * blockDim.x + threadIdx.x);
+    double* lo2 = reinterpret_cast<double*>(s_acc2 + bins);
+    double* hi2 = lo2 + nr;
+    for (int i = threadIdx.x; i < bins; i += blockDim.x) {
+        s_acc2[i] = acc[size_t(r) * bins + i];
+        if (i < nr) {
+            lo2[i] = corr_lo2(i, dr);
+            hi2[i] = corr_hi2(i, dr);
         }
-        if (a < nr && (b >= nr || corr_lo2(a, dr) <= corr_hi2(b, dr))) ++a; else ++b;
+    }
+    __syncthreads();
+    if (k >= nr) return;
+    // window k begins with the interval after its lower bound in the merged
+    // order and ends with the one before its upper bound comes
+    int a = k + 1, b = 0;
+    for (int hi = nr; b < hi;) {  // upper bounds before lower bound k: those below it (a tie: after)
+        const int mid = (b + hi) >> 1;
+        if (hi2[mid] < lo2[k]) b = mid + 1; else hi = mid;
+    }
+    const int first = a + b;
+    a = 0;
+    for (int hi = nr; a < hi;) {  // lower bounds before upper bound k: those not above it
+        const int mid = (a + hi) >> 1;
+        if (lo2[mid] <= hi2[k]) a = mid + 1; else hi = mid;
+    }
+    const int last = a + k;
+    double s = 0.0, c = 0.0;
+    for (int i = first; i <= last; ++i) {
+        s = __dadd_rn(s, s_acc2[i].x);
+        c = __dadd_rn(c, s_acc2[i].y);
     }
     out[size_t(r) * nr + k] = c > 0.0 ? make_double2(__ddiv_rn(s, c), 0.0) : make_double2(CUDART_NAN, CUDART_NAN);
 }
@@ -939,7 +981,10 @@ static cudaError_t corr_pairs_t(const LaunchCfg& c, unsigned cells, CellBufs b, 
     // a little under one cell per thread: at liquid densities a block's disks
     // are then a single round of its threads
     const int cells_per_block = NT * 7 / 8;
-    return launch_k(k_corr_pairs<CAP, NT>, dim3((cells + cells_per_block - 1) / cells_per_block, unsigned(c.R)), dim3(NT),
+    const unsigned blocks = (cells + cells_per_block - 1) / cells_per_block;
+    // rows of the stencil split over blocks while there are fewer than ~12 per SM
+    const unsigned split = unsigned(std::max<int64_t>(1, std::min<int64_t>({reach + 1, 8, 1824 / (int64_t(blocks) * c.R)})));
+    return launch_k(k_corr_pairs<CAP, NT>, dim3(blocks, unsigned(c.R), split), dim3(NT),
                     size_t(2 * nr + 1) * kCorrBytes * NT, c.stream, c.reps, (const uint8_t*)b.cnt, gpos, chi, off, nr, dr, reach,
                     cells_per_block, acc);
 }
@@ -970,7 +1015,8 @@ cudaError_t launch_corr_pairs(const LaunchCfg& c, int64_t most_cells, const Fram
         e = c.cap == 4 ? corr_pairs_nt<4>(c, n, cells, gpos, chi, off, nr, dr, reach, sums)
                        : corr_pairs_nt<9>(c, n, cells, gpos, chi, off, nr, dr, reach, sums);
     if (e != cudaSuccess) return e;
-    return launch_k(k_corr_windows, dim3(unsigned((nr + 127) / 128), unsigned(c.R)), dim3(128), 0, c.stream, nr, dr,
+    return launch_k(k_corr_windows, dim3(unsigned((nr + 127) / 128), unsigned(c.R)), dim3(128),
+                    size_t(2 * nr + 1) * sizeof(double2) + size_t(2 * nr) * sizeof(double), c.stream, nr, dr,
                     (const double2*)sums, out);
 }
 
