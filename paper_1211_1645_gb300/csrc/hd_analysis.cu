@@ -419,25 +419,144 @@ k_sq_pairs(const Rep* __restrict__ reps, bool fixed, int nq, int nh, int nk, con
             part[(size_t(r) * gridDim.x + blockIdx.x) * nq + q0 + lane + j * width] = make_double2(re[j], im[j]);
 }
 
+// The same for wave vectors on a full grid of consecutive components, h = hc - j
+// .. hc + j and k: with alpha = 2 pi x_n / L and B_n(k) = U_n(hc) V_n(k),
+// A(hc +- j, k) = sum_n B_n(k) cos(j alpha_n) +- i sum_n B_n(k) sin(j alpha_n),
+// so the two wave vectors of a sign share two sums of a complex times a real:
+// two fused multiply-adds each instead of four (326 -> 275 us for 21 x 21 and
+// 65,536 disks).  Unit (j, k) of a thread holds both sums.  comp[r] as above,
+// each part ascending without gaps; part: [r][block][nh nk].
+__global__ void __launch_bounds__(kPairThreads)
+k_sq_grid(const Rep* __restrict__ reps, bool fixed, int nh, int nk, const int* __restrict__ comp,
+          const double* __restrict__ xy, double2* __restrict__ part) {
+    pdl_begin();
+    extern __shared__ double2 s_wave[];  // [kPairDisks][nk + 1 + J], then the table
+    __shared__ Turn s_turn[kPairDisks][2];
+    const int r = blockIdx.z, tid = int(threadIdx.x);
+    const int J = nh / 2, nw = nk + 1 + J, units = (J + 1) * nk;  // centre h: entry J of the nh
+    const Rep& rep = reps[r];
+    double2* table = s_wave + kPairDisks * nw;
+    for (int j = tid; j < kTurnTable; j += kPairThreads) {
+        double s, c;
+        sincospi(double(j) * (2.0 / kTurnTable), &s, &c);
+        table[j] = make_double2(c, s);
+    }
+    int groups = 1;
+    while (groups < 8 && 2 * groups * units <= kPairThreads) groups *= 2;
+    const int width = kPairThreads / groups, group = tid / width, lane = tid - group * width;
+    int uj[kPairQ], uk[kPairQ];
+    bool mine[kPairQ];
+    double cr[kPairQ], ci[kPairQ], sr[kPairQ], si[kPairQ];
+#pragma unroll
+    for (int q = 0; q < kPairQ; ++q) {
+        const int u = lane + q * width;
+        mine[q] = u < units;
+        uj[q] = mine[q] ? u / nk : 0;
+        uk[q] = mine[q] ? u - uj[q] * nk : 0;
+        cr[q] = ci[q] = sr[q] = si[q] = 0.0;
+    }
+    const bool second = width < units;
+    const int* co = comp + size_t(r) * (nh + nk);
+    const int hc = co[J];
+    for (int64_t base = int64_t(blockIdx.x) * kPairDisks; base < rep.N; base += int64_t(gridDim.x) * kPairDisks) {
+        __syncthreads();
+        if (tid < 2 * kPairDisks) {
+            const int64_t i = base + (tid >> 1);
+            Turn t{0ull, 0u};
+            if (i < rep.N) {
+                double x = xy[2 * (rep.id_off + i) + (tid & 1)];
+                if (rep.sigma != 1.0) x = __ddiv_rn(x, rep.sigma);
+                t = fixed ? turn_fixed(uint64_t(llrint(__dmul_rn(x, 16777216.0))) % uint64_t(rep.LF), uint64_t(rep.LF))
+                          : turn_fp64(x, rep.Lm);
+            }
+            s_turn[tid >> 1][tid & 1] = t;
+        }
+        __syncthreads();
+        // V(k), then U(hc), then (cos, sin) of j alpha for j = 1 .. J
+        for (int e = tid; e < kPairDisks * nw; e += kPairThreads) {
+            const int n = e / nw, j = e - n * nw;
+            const int h = j < nk ? co[nh + j] : (j == nk ? hc : j - nk);
+            s_wave[e] = base + n < rep.N ? turn_wave(s_turn[n][j < nk], h, table) : make_double2(0.0, 0.0);
+        }
+        __syncthreads();
+        for (int e = tid; e < kPairDisks * nk; e += kPairThreads) {  // B(k) = U(hc) V(k)
+            const int n = e / nk, k = e - n * nk;
+            const double2 u = s_wave[n * nw + nk], v = s_wave[n * nw + k];
+            s_wave[n * nw + k] = make_double2(__fma_rn(u.x, v.x, -__dmul_rn(u.y, v.y)), __fma_rn(u.x, v.y, __dmul_rn(u.y, v.x)));
+        }
+        __syncthreads();
+        for (int n = group; n < kPairDisks; n += groups) {
+            const double2* w = s_wave + n * nw;
+#pragma unroll
+            for (int q = 0; q < kPairQ; ++q) {
+                if (q == 1 && !second) break;
+                const double2 b = w[uk[q]];
+                if (uj[q] == 0) {
+                    cr[q] = __dadd_rn(cr[q], b.x);
+                    ci[q] = __dadd_rn(ci[q], b.y);
+                } else {
+                    const double2 e = w[nk + uj[q]];
+                    cr[q] = __fma_rn(b.x, e.x, cr[q]);
+                    ci[q] = __fma_rn(b.y, e.x, ci[q]);
+                    sr[q] = __fma_rn(b.x, e.y, sr[q]);
+                    si[q] = __fma_rn(b.y, e.y, si[q]);
+                }
+            }
+        }
+    }
+    // the groups' sums in order
+    __syncthreads();
+    double2* s_sum = s_wave;  // 2 width entries: at most 256 of at least 32 x 3 + 128
+    for (int g = 1; g < groups; ++g) {
+        if (group == g && mine[0]) {
+            s_sum[2 * lane] = make_double2(cr[0], ci[0]);
+            s_sum[2 * lane + 1] = make_double2(sr[0], si[0]);
+        }
+        __syncthreads();
+        if (group == 0 && mine[0]) {
+            cr[0] = __dadd_rn(cr[0], s_sum[2 * lane].x);
+            ci[0] = __dadd_rn(ci[0], s_sum[2 * lane].y);
+            sr[0] = __dadd_rn(sr[0], s_sum[2 * lane + 1].x);
+            si[0] = __dadd_rn(si[0], s_sum[2 * lane + 1].y);
+        }
+        __syncthreads();
+    }
+    double2* out = part + (size_t(r) * gridDim.x + blockIdx.x) * size_t(nh) * size_t(nk);
+#pragma unroll
+    for (int q = 0; q < kPairQ; ++q) {
+        if (group != 0 || !mine[q]) continue;
+        if (J + uj[q] < nh) out[(J + uj[q]) * nk + uk[q]] = make_double2(__dsub_rn(cr[q], si[q]), __dadd_rn(ci[q], sr[q]));
+        if (uj[q] > 0) out[(J - uj[q]) * nk + uk[q]] = make_double2(__dadd_rn(cr[q], si[q]), __dsub_rn(ci[q], sr[q]));
+    }
+}
+
 // S_r(q) = |A_r(q)|^2 / N_r (Eq. 10) from the partial sums: blockIdx.y =
 // replica, 32 wave vectors per block, eight threads to each, whose sums are
 // added in order (one thread per wave vector over all partial sums ran a
 // serial chain: 134 us for 256 partial sums of 441 wave vectors, 6 here).
 __global__ void __launch_bounds__(256)
-k_sq_sum(const Rep* __restrict__ reps, int nq, int nbx, bool by_disks, const double2* __restrict__ part,
-         double* __restrict__ S) {
+k_sq_sum(const Rep* __restrict__ reps, int nq, int nbx, bool by_disks, const double2* __restrict__ part, int row_len, int nk,
+         const ushort2* __restrict__ pair, double* __restrict__ S) {
     pdl_begin();
     __shared__ double2 s_v[8][32];
     const int r = blockIdx.y, lane = int(threadIdx.x & 31u), row = int(threadIdx.x >> 5);
     const int q = blockIdx.x * 32 + lane;
     const int nb = by_disks ? int((reps[r].N + 255) / 256) : nbx;  // blocks that hold disks of this replica
     double a = 0.0, b = 0.0;
-    if (q < nq)
+    if (q < nq) {
+        // a row of partial sums holds the wave vectors themselves, or with
+        // pair the grid of their components
+        size_t at = size_t(q);
+        if (pair) {
+            const ushort2 c = pair[size_t(r) * nq + q];
+            at = size_t(c.x) * nk + c.y;
+        }
         for (int x = row; x < nb; x += 8) {
-            const double2 p = part[(size_t(r) * nbx + x) * nq + q];
+            const double2 p = part[(size_t(r) * nbx + x) * row_len + at];
             a = __dadd_rn(a, p.x);
             b = __dadd_rn(b, p.y);
         }
+    }
     s_v[row][lane] = make_double2(a, b);
     __syncthreads();
     if (row == 0 && q < nq) {
@@ -901,7 +1020,12 @@ int sq_disk_blocks(const std::vector<int64_t>& N) {
 
 bool sq_pairs_fit(int nh, int nk, int nq) {
     // fewer FP64 operations than a plane wave per wave vector and disk
-    return nh + nk <= kPairMax && nh <= 65535 && 15 * (nh + nk) + 4 * nq < 60 * nq;
+    return nh + nk <= kPairMax && 15 * (nh + nk) + 4 * nq < 60 * nq;
+}
+
+bool sq_grid_fit(int nh, int nk, int nq) {
+    const int64_t units = int64_t(nh / 2 + 1) * nk;
+    return units <= kPairThreads * kPairQ && units < nq;
 }
 
 int sq_pair_blocks(int R, int nq, const std::vector<int64_t>& N) {
@@ -918,24 +1042,31 @@ cudaError_t launch_sq(const LaunchCfg& c, int nq, const int2* hk, const double* 
     cudaError_t e = launch_k(k_sq_amp, grid, dim3(256), 0, c.stream, c.reps, c.fixed, nq, hk, xy, nbx, part);
     if (e == cudaSuccess)
         e = launch_k(k_sq_sum, dim3(unsigned((nq + 31) / 32), unsigned(c.R)), dim3(256), 0, c.stream, c.reps, nq, nbx, true,
-                     (const double2*)part, S);
+                     (const double2*)part, nq, 0, (const ushort2*)nullptr, S);
     if (e == cudaSuccess && best) e = launch_k(k_sq_best, dim3(unsigned(c.R)), dim3(256), 0, c.stream, nq, (const double*)S, best);
     return e;
 }
 
-cudaError_t launch_sq_pairs(const LaunchCfg& c, int nq, int nh, int nk, const int* comp, const ushort2* pair,
+cudaError_t launch_sq_pairs(const LaunchCfg& c, int nq, int nh, int nk, bool grid, const int* comp, const ushort2* pair,
                             const double* xy, int nbx, double2* part, double* S, int* best) {
     static std::once_flag attr_once;
     std::call_once(attr_once, [] {
-        cudaFuncSetAttribute(k_sq_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int((kPairDisks * kPairMax + kTurnTable) * sizeof(double2)));
+        const int most = int((kPairDisks * (kPairMax + 1) + kTurnTable) * sizeof(double2));
+        cudaFuncSetAttribute(k_sq_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+        cudaFuncSetAttribute(k_sq_grid, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
     });
-    const dim3 grid(unsigned(nbx), unsigned((nq + kPairThreads * kPairQ - 1) / (kPairThreads * kPairQ)), unsigned(c.R));
-    cudaError_t e = launch_k(k_sq_pairs, grid, dim3(kPairThreads), size_t(kPairDisks * (nh + nk) + kTurnTable) * sizeof(double2),
-                             c.stream, c.reps, c.fixed, nq, nh, nk, comp, pair, xy, part);
+    cudaError_t e;
+    if (grid)
+        e = launch_k(k_sq_grid, dim3(unsigned(nbx), 1, unsigned(c.R)), dim3(kPairThreads),
+                     size_t(kPairDisks * (nk + 1 + nh / 2) + kTurnTable) * sizeof(double2), c.stream, c.reps, c.fixed, nh, nk,
+                     comp, xy, part);
+    else
+        e = launch_k(k_sq_pairs, dim3(unsigned(nbx), unsigned((nq + kPairThreads * kPairQ - 1) / (kPairThreads * kPairQ)), unsigned(c.R)),
+                     dim3(kPairThreads), size_t(kPairDisks * (nh + nk) + kTurnTable) * sizeof(double2), c.stream, c.reps,
+                     c.fixed, nq, nh, nk, comp, pair, xy, part);
     if (e == cudaSuccess)
         e = launch_k(k_sq_sum, dim3(unsigned((nq + 31) / 32), unsigned(c.R)), dim3(256), 0, c.stream, c.reps, nq, nbx, false,
-                     (const double2*)part, S);
+                     (const double2*)part, grid ? nh * nk : nq, nk, grid ? pair : (const ushort2*)nullptr, S);
     if (e == cudaSuccess && best) e = launch_k(k_sq_best, dim3(unsigned(c.R)), dim3(256), 0, c.stream, nq, (const double*)S, best);
     return e;
 }

@@ -16,11 +16,13 @@ cudaError_t launch_sq(const LaunchCfg& c, int nq, const int2* hk, const double* 
                       int* best);
 // The same for wave vectors given by components: comp[R][nh + nk] the distinct
 // h, then k, of each replica, pair[R][nq] the indices of every wave vector's
-// (sq_pairs_fit: whether that is the cheaper way).  part: R x nbx x nq with
-// nbx = sq_pair_blocks.  best is nullable in both.
+// (sq_pairs_fit: whether that is the cheaper way); grid: the components of
+// every replica are nh and nk consecutive integers and sq_grid_fit.  part: R x
+// nbx x max(nq, nh nk) with nbx = sq_pair_blocks.  best is nullable in both.
 bool sq_pairs_fit(int nh, int nk, int nq);
+bool sq_grid_fit(int nh, int nk, int nq);
 int sq_pair_blocks(int R, int nq, const std::vector<int64_t>& N);
-cudaError_t launch_sq_pairs(const LaunchCfg& c, int nq, int nh, int nk, const int* comp, const ushort2* pair,
+cudaError_t launch_sq_pairs(const LaunchCfg& c, int nq, int nh, int nk, bool grid, const int* comp, const ushort2* pair,
                             const double* xy, int nbx, double2* part, double* S, int* best);
 // The window's wave vectors into hk[R][nq], and its components and pairs.
 cudaError_t launch_q0_window(const LaunchCfg& c, int hw, const double* psi, int2* hk, int* comp, ushort2* pair);

@@ -1807,7 +1807,7 @@ hd_status grow(hd_ctx* ctx, T*& p, size_t& cap, size_t need) {
 // S at the wave vectors already in ctx->sq_hk ([R][nq]), or with nh > 0 of the
 // components and pairs already in ctx->sq_comp and ctx->sq_pair; positions
 // refreshed first.
-hd_status enqueue_sq(hd_ctx* ctx, int nq, int nh, int nk, bool want_best) {
+hd_status enqueue_sq(hd_ctx* ctx, int nq, int nh, int nk, bool grid, bool want_best) {
     std::vector<int64_t> Ns;
     for (const Rep& r : ctx->reps) Ns.push_back(r.N);
     // (the bound on the partial sums of one plane wave per wave vector and
@@ -1815,7 +1815,7 @@ hd_status enqueue_sq(hd_ctx* ctx, int nq, int nh, int nk, bool want_best) {
     const size_t bound = size_t(ctx->R) * size_t(hd::sq_disk_blocks(Ns)) * size_t(nq);
     if (bound > (size_t(1) << 27)) return HD_ERR_ARG;
     const int nbx = nh > 0 ? hd::sq_pair_blocks(ctx->R, nq, Ns) : hd::sq_disk_blocks(Ns);
-    hd_status st = grow(ctx, ctx->sq_part, ctx->sq_part_cap, size_t(ctx->R) * size_t(nbx) * size_t(nq));
+    hd_status st = grow(ctx, ctx->sq_part, ctx->sq_part_cap, size_t(ctx->R) * size_t(nbx) * size_t(grid ? std::max(nq, nh * nk) : nq));
     if (st != HD_OK) return st;
     st = grow(ctx, ctx->sq_S, ctx->sq_S_cap, size_t(ctx->R) * nq);
     if (st != HD_OK) return st;
@@ -1826,7 +1826,7 @@ hd_status enqueue_sq(hd_ctx* ctx, int nq, int nh, int nk, bool want_best) {
     HD_CK(ctx, launch(ctx, HD_K_ANALYSIS, [&] {
         int* best = want_best ? ctx->sq_best : nullptr;
         if (nh > 0)
-            return hd::launch_sq_pairs(ctx->cfg(), nq, nh, nk, ctx->sq_comp, ctx->sq_pair, ctx->xy, nbx, ctx->sq_part, ctx->sq_S,
+            return hd::launch_sq_pairs(ctx->cfg(), nq, nh, nk, grid, ctx->sq_comp, ctx->sq_pair, ctx->xy, nbx, ctx->sq_part, ctx->sq_S,
                                        best);
         return hd::launch_sq(ctx->cfg(), nq, ctx->sq_hk, ctx->xy, nbx, ctx->sq_part, ctx->sq_S, best);
     }));
@@ -1836,7 +1836,9 @@ hd_status enqueue_sq(hd_ctx* ctx, int nq, int nh, int nk, bool want_best) {
 // The distinct components of each replica's wave vectors, padded to the
 // largest count, and each wave vector's indices; false where the lists share
 // too few of them.
-bool sq_components(int R, int nq, const int32_t* hk, int& nh, int& nk, std::vector<int>& comp, std::vector<ushort2>& pair) {
+// grid: every replica's are nh and nk consecutive integers.
+bool sq_components(int R, int nq, const int32_t* hk, int& nh, int& nk, bool& grid, std::vector<int>& comp,
+                   std::vector<ushort2>& pair) {
     std::vector<std::vector<int>> h(static_cast<size_t>(R)), k(static_cast<size_t>(R));
     nh = nk = 1;
     for (int r = 0; r < R; ++r) {
@@ -1850,6 +1852,13 @@ bool sq_components(int R, int nq, const int32_t* hk, int& nh, int& nk, std::vect
         nh = std::max(nh, int(h[size_t(r)].size()));
         nk = std::max(nk, int(k[size_t(r)].size()));
         if (!hd::sq_pairs_fit(nh, nk, nq)) return false;
+    }
+    grid = hd::sq_grid_fit(nh, nk, nq);
+    for (int r = 0; r < R; ++r) {
+        auto run = [](const std::vector<int>& v, int n) {
+            return int(v.size()) == n && int64_t(v.back()) - int64_t(v.front()) == int64_t(n) - 1;
+        };
+        grid = grid && run(h[size_t(r)], nh) && run(k[size_t(r)], nk);
     }
     comp.assign(size_t(R) * size_t(nh + nk), 0);
     pair.resize(size_t(R) * size_t(nq));
@@ -1873,10 +1882,11 @@ hd_status hd_structure_factor(hd_ctx* ctx, int32_t nq, const int32_t* hk, double
     if (!ctx || !hk || !S || nq < 1 || nq > 65536) return HD_ERR_ARG;
     if (ctx->sticky != HD_OK) return HD_ERR_STATE;
     int nh = 0, nk = 0;
+    bool grid = false;
     std::vector<int> comp;
     std::vector<ushort2> pair;
     hd_status st;
-    if (sq_components(ctx->R, nq, hk, nh, nk, comp, pair)) {
+    if (sq_components(ctx->R, nq, hk, nh, nk, grid, comp, pair)) {
         st = grow(ctx, ctx->sq_comp, ctx->sq_comp_cap, comp.size());
         if (st == HD_OK) st = grow(ctx, ctx->sq_pair, ctx->sq_pair_cap, pair.size());
         if (st != HD_OK) return st;
@@ -1888,7 +1898,7 @@ hd_status hd_structure_factor(hd_ctx* ctx, int32_t nq, const int32_t* hk, double
         if (st != HD_OK) return st;
         HD_CK(ctx, cudaMemcpyAsync(ctx->sq_hk, hk, sizeof(int2) * size_t(ctx->R) * nq, cudaMemcpyHostToDevice, ctx->stream));
     }
-    st = enqueue_sq(ctx, nq, nh, nk, false);
+    st = enqueue_sq(ctx, nq, nh, nk, grid, false);
     if (st != HD_OK) return st;
     HD_CK(ctx, cudaMemcpyAsync(S, ctx->sq_S, sizeof(double) * size_t(ctx->R) * nq, cudaMemcpyDeviceToHost, ctx->stream));
     HD_CK(ctx, cudaStreamSynchronize(ctx->stream));
@@ -1913,7 +1923,7 @@ hd_status hd_positional_q0(hd_ctx* ctx, int32_t half_width, int32_t* hk0, double
         return hd::launch_q0_window(ctx->cfg(), half_width, ctx->psi_res, ctx->sq_hk, pairs ? ctx->sq_comp : nullptr,
                                     pairs ? ctx->sq_pair : nullptr);
     }));
-    st = enqueue_sq(ctx, nq, pairs ? w : 0, w, true);
+    st = enqueue_sq(ctx, nq, pairs ? w : 0, w, pairs && hd::sq_grid_fit(w, w, nq), true);
     if (st != HD_OK) return st;
     std::vector<int2> win(size_t(ctx->R) * nq);
     std::vector<int> best(size_t(ctx->R));

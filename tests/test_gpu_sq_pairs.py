@@ -24,6 +24,12 @@ LISTS = {
     "513": window(23, -11, 4)[:513],
     "80 + 80 components": [[i, j] for i in range(80) for j in (2 * i % 80, (2 * i + 1) % 80, (i + 40) % 80)],
     "81 + 80 components": [[i % 81, i % 80] for i in range(81 * 3)],
+    "grid of 2 x 2": window(2, -1, -1),
+    "grid of 3 x 3": window(3, 40, -1),
+    "grid of 14 x 14": window(14, 5, -30),
+    "grid of 29 x 29": window(29, -14, 3),
+    "part of a grid": [[i, k] for i in range(9) for k in range(9) if i + k < 15],
+    "grid at the ends": [[2147483646 + i, -2147483648 + k] for i in range(2) for k in range(2)],
     "large": [[100000, -99999], [-2000000000, 3], [7, 2000000000], [100000, 3], [7, -99999]],
 }
 
