@@ -241,9 +241,10 @@ void set_hist_f32_bounds(Rep& r, double e0, double eK) {
 // Tiles of every replica for the tile sweep (see hd_tile.h); false where it
 // cannot run (a box of fewer than six half-cells) or another order of the
 // sweeps is faster.  As few tiles as the staged region allows, since every
-// tile also updates some cells around it; one replica that would leave SMs
-// idle is split further, its longer side first, down to tiles of 16 cells
-// (N = 65,536: 144 tiles 8.8 us per sweep, 72 tiles 10.8).
+// tile also updates some cells around it; one replica whose tiles would leave
+// SMs idle is split into as many as there are SMs, not more (a second round
+// for a few tiles costs a whole one), of eight cells a side at least (us per
+// sweep at N = 262,144: 152 tiles 12.4, 156 13.4; at 65,536: 152 8.2, 72 10.8).
 bool plan_tiles(hd_ctx* ctx, int sms) {
     // The FP64 form stages twice the bytes per cell in tiles half as large, and
     // its frame changes are FP64-bound: per sweep 30.5 us against 42.9 as graph
@@ -258,10 +259,20 @@ bool plan_tiles(hd_ctx* ctx, int sms) {
         const int least = r.hm < 12 ? 1 : 2;  // see wrap_half
         hd::TileGrid g{int32_t(total), std::max(least, (r.m + lim.max_x - 1) / lim.max_x),
                        std::max(least, (r.m + lim.max_y - 1) / lim.max_y)};
-        if (ctx->R == 1)
-            while (int64_t(g.ntx) * g.nty < sms && r.hm / std::max(g.ntx, g.nty) >= 8) {
-                if (r.m / g.ntx > r.m / g.nty) ++g.ntx; else ++g.nty;
+        if (ctx->R == 1) {
+            const int most = std::max(1, r.hm / 4);
+            hd::TileGrid best = g;
+            for (int x = g.ntx; x <= most && x <= sms; ++x) {
+                const int y = std::min(most, sms / x);
+                if (y < g.nty) break;
+                const bool more = x * y > best.ntx * best.nty;
+                if (more || (x * y == best.ntx * best.nty && std::abs(x - y) < std::abs(best.ntx - best.nty))) {
+                    best.ntx = x;
+                    best.nty = y;
+                }
             }
+            g = best;
+        }
         ctx->tiles.push_back(g);
         total += int64_t(g.ntx) * g.nty;
     }
