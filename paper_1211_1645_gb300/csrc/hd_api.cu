@@ -72,6 +72,7 @@ struct hd_ctx {
     bool tiled = false;
     std::vector<hd::TileGrid> tiles;   // [R]
     hd::TileCfg tile_cfg{};
+    int box_hm = 0;                    // the largest half-side, when box_spill is set
     void* box_spill = nullptr;         // set: the boxes are small enough for one block each (launch_sweeps_box)
     bool persist_stall = false;        // test hook (HD_TEST_PERSIST_STALL=1 at creation)
     // analysis scratch, grown on demand and freed with the context
@@ -703,7 +704,7 @@ cudaError_t enqueue_sweeps(hd_ctx* ctx, cudaStream_t s, int64_t n, bool capturin
             if (e == cudaSuccess)
                 e = launch(ctx, HD_K_SWEEP, [&] {
                     if (ctx->box_spill)
-                        return hd::launch_sweeps_box(c, ctx->box_spill, ctx->table, nc, ctx->buf[ctx->cur],
+                        return hd::launch_sweeps_box(c, ctx->box_hm, ctx->box_spill, ctx->table, nc, ctx->buf[ctx->cur],
                                                      ctx->buf[ctx->cur ^ 1], ctx->counters, ctx->err);
                     return hd::launch_sweeps_tile(c, ctx->tile_cfg, ctx->table, nc, ctx->buf[ctx->cur],
                                                   ctx->buf[ctx->cur ^ 1], ctx->counters, ctx->err);
@@ -1073,15 +1074,18 @@ hd_status hd_batch_init(hd_ctx** out, int32_t R, const int64_t* N, const double*
     // The order of the launches left to the library (strips, replica_branches
     // 0): all sweeps of a draw table in one launch, of whole small boxes or of
     // tiles, where the launch boundary of the split kernels costs more than
-    // their work (per sweep at N = 256 5.3 us against 11.1 as a serial graph, at
-    // 65,536 8.8 against 20.8, at 2^20 30 against 35 as 16 strips).
+    // their work (per sweep at N = 256 4.6 us against 11.1 as a serial graph, at
+    // 65,536 8.2 against 20.8, at 2^20 30 against 35 as 16 strips).
     if (ok && split1 && cap == 4 && R <= kMaxTiledReplicas && (R == 1 ? o.strips == 0 : o.replica_branches == 0)) {
         int dev = 0, sms = 0;
         ok = cudaGetDevice(&dev) == cudaSuccess &&
              cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
         unsigned char* spill = nullptr;
-        if (ok && std::all_of(ctx->reps.begin(), ctx->reps.end(), [](const Rep& r) { return r.hm <= hd::box_max_hm(); })) {
-            ok = dev_alloc(ctx, &spill, size_t(R) * hd::box_spill(ctx->fixed));
+        int hm = 0;
+        for (const Rep& r : ctx->reps) hm = std::max(hm, r.hm);
+        if (ok && hm <= hd::box_max_hm(ctx->fixed, R)) {
+            ctx->box_hm = hm;
+            ok = dev_alloc(ctx, &spill, size_t(R) * hd::box_spill(ctx->fixed, hm));
             ctx->box_spill = spill;
             ctx->tiled = true;
         } else if (ok && plan_tiles(ctx, sms)) {

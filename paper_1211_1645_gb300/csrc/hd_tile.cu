@@ -502,7 +502,14 @@ k_sweep_tile(const Rep* __restrict__ reps, const TileGrid* __restrict__ grids, i
 // sweep.
 // ---------------------------------------------------------------------------
 template <bool FIX, int HB>
-using BoxStage = Stage<FIX, HB, HB, 64>;
+using BoxStage = Stage<FIX, HB, HB, HB <= 12 ? 64 : (FIX ? 256 : 160)>;
+
+// Hard cells from registers (hard_cell_ahead), but for small fixed-point boxes
+// (N <= 400), whose few crowded cells cost less as tile_cell takes them: per
+// sweep at N = 256 4.6 us against 4.8; FP64 6.4 -> 6.0, boxes of N = 1024 7.8 -> 7.4
+// fixed and 11.5 -> 11.0 FP64.
+template <bool FIX, int HB>
+constexpr bool kHardRegs = !FIX || HB > 12;
 
 // A cell of the ring around the box, or its source, is (x, y): copy the
 // occupants of entry `from` to entry `to`.
@@ -523,12 +530,11 @@ __device__ __forceinline__ void copy_cell(const S& st, int from, int to) {
 
 template <bool FIX, int HB>
 constexpr size_t box_smem() {
-    return 2 * BoxStage<FIX, HB>::kBytes + size_t(2) * BoxStage<FIX, HB>::NC * (sizeof(P2<FIX>) + 4);
+    return 2 * BoxStage<FIX, HB>::kBytes + size_t(2) * BoxStage<FIX, HB>::NC * (sizeof(P2<FIX>) + (kHardRegs<FIX, HB> ? 8 : 4));
 }
-constexpr int kBoxDrawThreads = 128;
 
-template <bool FIX, int NTC, int HB, int NT>
-__global__ void __launch_bounds__(NT + kBoxDrawThreads)
+template <bool FIX, int NTC, int HB, int NT, int ND>
+__global__ void __launch_bounds__(NT + ND)
 k_sweep_box(const Rep* __restrict__ reps, const Frame* __restrict__ table, int nsweeps, CellBufs g0, CellBufs g1,
             unsigned long long* __restrict__ counters, int* __restrict__ err, void* spill) {
     using S = BoxStage<FIX, HB>;
@@ -553,9 +559,10 @@ k_sweep_box(const Rep* __restrict__ reps, const Frame* __restrict__ table, int n
         ly = 2 * int(row) + int(pl >> 1) + 2;
     };
     auto wrap_local = [m](int v) { return v < 2 ? v + m : (v >= m + 2 ? v - m : v); };
-    // [2][NC] steps, then swap words, by entry of the stage
+    // [2][NC] steps, then first and (kHardRegs) second swap words, by entry of the stage
     P2<FIX>* s_step = reinterpret_cast<P2<FIX>*>(s_raw + 2 * S::kBytes);
     uint32_t* s_swap = reinterpret_cast<uint32_t*>(s_step + 2 * S::NC);
+    uint32_t* s_swap2 = s_swap + 2 * S::NC;
     // frame changes of two sweeps, read ahead
     struct Change {
         double dx, dy;
@@ -574,14 +581,16 @@ k_sweep_box(const Rep* __restrict__ reps, const Frame* __restrict__ table, int n
         for (int i = 0; i < nsweeps; ++i) {
             const uint32_t sweep = s_change[i & 1].sweep;
             if (tid == NT && i + 1 < nsweeps) read_change(i + 1);
-            for (uint32_t e = uint32_t(tid - NT); e < 4u * hh; e += kBoxDrawThreads) {
+            for (uint32_t e = uint32_t(tid - NT); e < 4u * hh; e += ND) {
                 int lx, ly;
                 local(e, lx, ly);
                 const uint32_t cl = uint32_t(ly - 2) * uint32_t(m) + uint32_t(lx - 2);
                 const int at = (i & 1) * S::NC + S::index(lx, ly);
                 const uint4 u = philox(sweep, 0u, cl, kTagTrial, rep.key0, rep.key1);
                 s_step[at] = trial_step<FIX>(rep, u);
-                s_swap[at] = FIX ? u.z : philox(sweep, 0u, cl, kTagShuffle, rep.key0, rep.key1).x;
+                const uint4 v = FIX ? make_uint4(u.z, u.w, 0u, 0u) : philox(sweep, 0u, cl, kTagShuffle, rep.key0, rep.key1);
+                s_swap[at] = v.x;
+                if constexpr (kHardRegs<FIX, HB>) s_swap2[at] = v.y;
             }
             __syncthreads();
         }
@@ -695,29 +704,33 @@ k_sweep_box(const Rep* __restrict__ reps, const Frame* __restrict__ table, int n
                 const int gy = cy == 0u ? m + 2 : (cy == uint32_t(m - 1) ? 1 : 0);
                 const int lx = int(cx) + 2, ly = int(cy) + 2;
                 const int at = (i & 1) * S::NC + e;
-                const uint32_t got = tile_cell<FIX, NTC, hard.value, true, S>(
-                    st, rep, sd.sweep, px, py, hx, hy, w, cy * uint32_t(m) + cx,
-                    [&](int k, const P2<FIX>& q, int32_t id) {
-                        // in id order, ids and positions together
-                        if (k < 2) {
-                            const typename S::Stored v = st.stored(q);
-                            st.set(e, k, v);
-                            reinterpret_cast<int32_t*>(st.id)[2 * e + k] = id;
-                            if (gx) st.set(S::index(gx, ly), k, v);
-                            if (gy) st.set(S::index(lx, gy), k, v);
-                            if (gx && gy) st.set(S::index(gx, gy), k, v);
-                        } else {
-                            PoolEntry<FIX>* x = st.extra(w, e, k);
-                            x->p = q;
-                            x->id = id;
-                            if (x >= st.spill && x < st.spill + 2 * S::NC) {  // the copies share a pool entry, not the spill area's
-                                if (gx) st.extra(w, S::index(gx, ly), k)->p = q;
-                                if (gy) st.extra(w, S::index(lx, gy), k)->p = q;
-                                if (gx && gy) st.extra(w, S::index(gx, gy), k)->p = q;
-                            }
+                const Drawn<FIX> pre{s_step[at], s_swap[at], kHardRegs<FIX, HB> ? s_swap2[at] : 0u};
+                auto emit = [&](int k, const P2<FIX>& q, int32_t id) {
+                    // in id order, ids and positions together
+                    if (k < 2) {
+                        const typename S::Stored v = st.stored(q);
+                        st.set(e, k, v);
+                        reinterpret_cast<int32_t*>(st.id)[2 * e + k] = id;
+                        if (gx) st.set(S::index(gx, ly), k, v);
+                        if (gy) st.set(S::index(lx, gy), k, v);
+                        if (gx && gy) st.set(S::index(gx, gy), k, v);
+                    } else {
+                        PoolEntry<FIX>* x = st.extra(w, e, k);
+                        x->p = q;
+                        x->id = id;
+                        if (x >= st.spill && x < st.spill + 2 * S::NC) {  // the copies share a pool entry, not the spill area's
+                            if (gx) st.extra(w, S::index(gx, ly), k)->p = q;
+                            if (gy) st.extra(w, S::index(lx, gy), k)->p = q;
+                            if (gx && gy) st.extra(w, S::index(gx, gy), k)->p = q;
                         }
-                    },
-                    Drawn<FIX>{s_step[at], s_swap[at]});
+                    }
+                };
+                const uint32_t cl = cy * uint32_t(m) + cx;
+                uint32_t got;
+                if constexpr (hard.value && kHardRegs<FIX, HB>)
+                    got = hard_cell_ahead<FIX, NTC, S>(st, rep, sd.sweep, px, py, hx, hy, w, cl, emit, pre);
+                else
+                    got = tile_cell<FIX, NTC, hard.value, true, S>(st, rep, sd.sweep, px, py, hx, hy, w, cl, emit, pre);
                 att += uint32_t(rep.nt);
                 acc += got;
             };
@@ -763,7 +776,11 @@ k_sweep_box(const Rep* __restrict__ reps, const Frame* __restrict__ table, int n
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-constexpr int kBoxHalf = 12, kBoxThreads = 256;  // half-cells per axis staged (hm + 2 used)
+// Half-cells per axis staged (hm + 2 used), sweeping threads and drawing threads.
+// The large shape holds N = 1024 (m = 32) in 130 KB (FP64 228 KB) of shared memory: one block
+// per SM, so as many threads as its passes have cells, twice.
+struct SmallBox { static constexpr int HB = 12, NT = 256, ND = 128; };
+struct LargeBox { static constexpr int HB = 18, NT = 512, ND = 256; };
 
 namespace {
 
@@ -800,35 +817,49 @@ cudaError_t tile_t(const LaunchCfg& c, const TileCfg& t, const Frame* table, int
                     uint32_t(t.total), a, b, counters, err, t.sync, t.spill, kTilePolls);
 }
 
-template <bool FIX, int NTC, int HB, int NT>
+template <class B, bool FIX, int NTC>
 cudaError_t box_t(const LaunchCfg& c, void* spill, const Frame* table, int nsweeps, CellBufs a, CellBufs b,
                   unsigned long long* counters, int* err) {
-    constexpr size_t smem = box_smem<FIX, HB>();
+    constexpr size_t smem = box_smem<FIX, B::HB>();
+    constexpr auto kernel = k_sweep_box<FIX, NTC, B::HB, B::NT, B::ND>;
     static std::once_flag attr_once;
-    std::call_once(attr_once, [] {
-        cudaFuncSetAttribute(k_sweep_box<FIX, NTC, HB, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    });
-    return launch_k(k_sweep_box<FIX, NTC, HB, NT>, dim3(c.R), dim3(NT + kBoxDrawThreads), smem, c.stream, c.reps, table, nsweeps, a, b,
-                    counters, err, spill);
+    std::call_once(attr_once, [] { cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)); });
+    return launch_k(kernel, dim3(c.R), dim3(B::NT + B::ND), smem, c.stream, c.reps, table, nsweeps, a, b, counters, err, spill);
+}
+
+template <class B>
+cudaError_t boxes(const LaunchCfg& c, void* spill, const Frame* table, int nsweeps, CellBufs a, CellBufs b,
+                  unsigned long long* counters, int* err) {
+    if (c.fixed)
+        return c.ntc == 1 ? box_t<B, true, 1>(c, spill, table, nsweeps, a, b, counters, err)
+                          : box_t<B, true, 0>(c, spill, table, nsweeps, a, b, counters, err);
+    return c.ntc == 1 ? box_t<B, false, 1>(c, spill, table, nsweeps, a, b, counters, err)
+                      : box_t<B, false, 0>(c, spill, table, nsweeps, a, b, counters, err);
+}
+
+template <class B>
+size_t spill_of(bool fixed) {
+    return fixed ? size_t(4) * BoxStage<true, B::HB>::NC * sizeof(PoolEntry<true>)
+                 : size_t(4) * BoxStage<false, B::HB>::NC * sizeof(PoolEntry<false>);
 }
 
 }  // namespace
 
-int box_max_hm() { return kBoxHalf - 2; }
+// One replica beyond the small box: a block's latency against that of several
+// tiles.  Fixed form, per sweep as a box and as tiles: N = 600 9.6 and 11.3 us,
+// 700 6.1 and 6.6, 900 7.3 and 7.8, 1024 7.4 and 7.6.  FP64: 500 12.8 and 15.0, 600 14.9
+// and 16.2, 800 15.9 and 16.4, 900 10.6 and 10.6, 1024 11.0 and 10.3.  Several replicas
+// share the GPU, and a block each is less work than four tiles each: 32 of
+// N = 1024 7.7 and 9.8 us (FP64 11.5 and 13.5), 152 of them 7.7 and 35.6, 700 37 and 170.
+int box_max_hm(bool fixed, int R) { return fixed || R > 1 ? LargeBox::HB - 2 : LargeBox::HB - 4; }
 
-size_t box_spill(bool fixed) {
-    return fixed ? size_t(4) * BoxStage<true, kBoxHalf>::NC * sizeof(PoolEntry<true>)
-                 : size_t(4) * BoxStage<false, kBoxHalf>::NC * sizeof(PoolEntry<false>);
-}
+size_t box_spill(bool fixed, int hm) { return hm <= SmallBox::HB - 2 ? spill_of<SmallBox>(fixed) : spill_of<LargeBox>(fixed); }
 
-cudaError_t launch_sweeps_box(const LaunchCfg& c, void* spill, const Frame* table, int nsweeps, CellBufs from, CellBufs to,
-                              unsigned long long* counters, int* err) {
-    if (nsweeps < 1 || nsweeps > kMaxChunk || c.cap != 4) return cudaErrorInvalidValue;
-    if (c.fixed)
-        return c.ntc == 1 ? box_t<true, 1, kBoxHalf, kBoxThreads>(c, spill, table, nsweeps, from, to, counters, err)
-                          : box_t<true, 0, kBoxHalf, kBoxThreads>(c, spill, table, nsweeps, from, to, counters, err);
-    return c.ntc == 1 ? box_t<false, 1, kBoxHalf, kBoxThreads>(c, spill, table, nsweeps, from, to, counters, err)
-                      : box_t<false, 0, kBoxHalf, kBoxThreads>(c, spill, table, nsweeps, from, to, counters, err);
+cudaError_t launch_sweeps_box(const LaunchCfg& c, int hm, void* spill, const Frame* table, int nsweeps, CellBufs from,
+                              CellBufs to, unsigned long long* counters, int* err) {
+    if (nsweeps < 1 || nsweeps > kMaxChunk || c.cap != 4 || hm > LargeBox::HB - 2) return cudaErrorInvalidValue;
+    return hm <= SmallBox::HB - 2 ? boxes<SmallBox>(c, spill, table, nsweeps, from, to, counters, err)
+                                  : boxes<LargeBox>(c, spill, table, nsweeps, from, to, counters, err);
 }
 
 TileLimits tile_limits(bool fixed) {

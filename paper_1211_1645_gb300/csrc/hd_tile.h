@@ -41,13 +41,13 @@ size_t tile_sync_words(int64_t total);
 cudaError_t launch_sweeps_tile(const LaunchCfg& c, const TileCfg& t, const Frame* table, int nsweeps, CellBufs from,
                                CellBufs to, unsigned long long* counters, int* err);
 
-// Small boxes (half-side hm <= box_max_hm() for every replica): each box kept in
-// one block's shared memory over all sweeps of the launch.  spill: R x
-// box_spill bytes.  As launch_sweeps_tile, but the generation not written last
+// Small boxes (half-side hm <= box_max_hm for every replica): each box kept in
+// one block's shared memory over all sweeps of the launch.  hm: the largest
+// half-side of the replicas.  spill: R x box_spill bytes.  As launch_sweeps_tile, but the generation not written last
 // is left as it was.
-int box_max_hm();
-size_t box_spill(bool fixed);
-cudaError_t launch_sweeps_box(const LaunchCfg& c, void* spill, const Frame* table, int nsweeps, CellBufs from, CellBufs to,
-                              unsigned long long* counters, int* err);
+int box_max_hm(bool fixed, int R);
+size_t box_spill(bool fixed, int hm);
+cudaError_t launch_sweeps_box(const LaunchCfg& c, int hm, void* spill, const Frame* table, int nsweeps, CellBufs from,
+                              CellBufs to, unsigned long long* counters, int* err);
 
 }  // namespace hd

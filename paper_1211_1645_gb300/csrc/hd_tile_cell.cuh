@@ -365,6 +365,7 @@ template <bool FIX>
 struct Drawn {
     P2<FIX> step;
     uint32_t swap;
+    uint32_t swap2 = 0u;  // the second word of the shuffle (hard_cell_ahead)
 };
 
 // One active cell: plane (px, py), half-row hy, half-column hx, word w, Philox
@@ -465,6 +466,108 @@ __device__ __forceinline__ uint32_t tile_cell(const S& st, const TileRep<FIX>& r
     }
     emit(0, q0, ids.x);
     if (two) emit(1, q1, ids.y);
+    return acc;
+}
+
+// A hard cell whose first trial's draws were made ahead, all of its occupants in
+// registers: one path for one to four disks, so that the few threads of a pass
+// that have such cells run it together.  Arguments and results as of tile_cell.
+template <bool FIX, int NTC, class S, class Emit>
+__device__ __forceinline__ uint32_t hard_cell_ahead(const S& st, const TileRep<FIX>& rep, uint32_t sweep, int px, int py,
+                                                    int hx, int hy, uint32_t w, uint32_t cl, Emit&& emit,
+                                                    const Drawn<FIX>& pre) {
+    const int e = ((py << 1) | px) * S::NP + hy * S::HP + hx;
+    const int n = min(int(w & 15u), 4);
+    const NbrBase<S> nb(px, py, hx, hy);
+    const int2 ids = st.id[e];
+    P2<FIX> P[4] = {st.get(e, 0), st.get(e, 1)};  // slots at or beyond n are no disks
+    int32_t I[4] = {ids.x, ids.y, 0, 0};
+    P[2] = P[3] = P[0];
+    uint32_t order = 0x3210u;  // position -> slot, Fisher-Yates as try_cell_in
+    if (n > 2) {
+#pragma unroll
+        for (int k = 2; k < 4; ++k) {
+            if (k >= n) continue;
+            const PoolEntry<FIX>* x = st.extra(w, e, k);
+            P[k] = x->p;
+            I[k] = x->id;
+        }
+        sort_by_id<FIX, 4>(P, I, n);
+        uint32_t third = 0u;
+        if (n > 3) {
+            const uint4 a = philox(sweep, 0u, cl, kTagShuffle, rep.key0, rep.key1);
+            third = FIX ? a.x : a.z;
+        }
+#pragma unroll
+        for (int k = 3; k >= 1; --k) {
+            if (k >= n) continue;
+            const int i = n - 1 - k;
+            const uint32_t j = bounded(i == 0 ? pre.swap : (i == 1 ? pre.swap2 : third), uint32_t(k + 1));
+            const uint32_t vk = (order >> (4 * k)) & 0xFu, vj = (order >> (4 * j)) & 0xFu;
+            order &= ~((0xFu << (4 * k)) | (0xFu << (4 * j)));
+            order |= (vj << (4 * k)) | (vk << (4 * j));
+        }
+    } else if (n == 2) {
+        if (ids.y < ids.x) {
+            const P2<FIX> t = P[0];
+            P[0] = P[1];
+            P[1] = t;
+            I[0] = ids.y;
+            I[1] = ids.x;
+        }
+        if ((pre.swap >> 31) == 0u) order = 0x3201u;
+    }
+    const RegCell<FIX, 4> cell{P};
+    uint32_t acc = 0;
+    const int nt = NTC > 0 ? NTC : rep.nt;
+    for (int t = 0; t < nt; ++t) {
+        const P2<FIX> step =
+            t == 0 ? pre.step : trial_step<FIX>(rep, philox(sweep, uint32_t(t), cl, kTagTrial, rep.key0, rep.key1));
+        const int slot = int((order >> (4 * (t == 0 ? 0 : t % n))) & 0xFu);
+        const P2<FIX> me = cell.pick(slot);
+        P2<FIX> np;
+        bool ok;
+        if constexpr (FIX) {
+            np.x = me.x + step.x;
+            np.y = me.y + step.y;
+            ok = uint32_t(np.x) < uint32_t(rep.W) && uint32_t(np.y) < uint32_t(rep.W);
+            auto own = [&](int q) { ok &= pair_clear_at<FIX>(P[q], 0, 0, np, rep) | (q >= n) | (q == slot); };
+            own(0);
+            own(1);
+            if (n > 2) {
+                own(2);
+                own(3);
+            }
+        } else {
+            np.x = __dadd_rn(me.x, step.x);
+            np.y = __dadd_rn(me.y, step.y);
+            ok = nonneg_bits(np.x) && below_pos_bits(np.x, rep.w) && nonneg_bits(np.y) && below_pos_bits(np.y, rep.w);
+            const float fx = image<FIX>(np.x), fy = image<FIX>(np.y);
+            float least = kFarFloat;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const float rx = __fsub_rn(image<FIX>(P[q].x), fx), ry = __fsub_rn(image<FIX>(P[q].y), fy);
+                if (q < n && q != slot) least = fminf(least, __fmaf_rn(rx, rx, __fmul_rn(ry, ry)));
+            }
+            ok = ok && least >= rep.d2_lo;
+            if (ok && least < rep.d2_hi) {  // rare: some pair is within the band
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    if (q < n && q != slot) ok = ok && pair_clear_at<FIX>(P[q], 0, 0, np, rep);
+            }
+        }
+        if (ok) ok = tile_clear<FIX, S>(st, rep, nb, np, np, false, (w >> kCrowdShift) & 0xFFu, 2 * hx + px, 2 * hy + py);
+        if (ok) {
+            cell.put(slot, np);
+            ++acc;
+        }
+    }
+    emit(0, P[0], I[0]);
+    if (n > 1) emit(1, P[1], I[1]);
+    if (n > 2) {
+        emit(2, P[2], I[2]);
+        if (n > 3) emit(3, P[3], I[3]);
+    }
     return acc;
 }
 
