@@ -242,10 +242,13 @@ void set_hist_f32_bounds(Rep& r, double e0, double eK) {
 // Tiles of every replica for the tile sweep (see hd_tile.h); false where it
 // cannot run (a box of fewer than six half-cells) or another order of the
 // sweeps is faster.  As few tiles as the staged region allows, since every
-// tile also updates some cells around it; one replica whose tiles would leave
-// SMs idle is split into as many as there are SMs, not more (a second round
-// for a few tiles costs a whole one), of eight cells a side at least (us per
-// sweep at N = 262,144: 152 tiles 12.4, 156 13.4; at 65,536: 152 8.2, 72 10.8).
+// tile also updates some cells around it; tiles that would leave SMs idle are
+// split into as many as there are SMs, not more (a second round for a few tiles
+// costs a whole one), of eight cells a side at least (us per sweep at
+// N = 262,144: 152 tiles 12.4, 156 13.4; at 65,536: 152 8.2, 72 10.8).  Several
+// replicas share the idle SMs by their cells (us per sweep with the fewest tiles
+// and with shares: two of N = 16,384 17.9 -> 8.1, eight 18.4 -> 10.9, three of
+// 65,536 22.5 -> 11.9; FP64 22.7 -> 11.5, 22.9 -> 16.5, 22.9 -> 18.3).
 bool plan_tiles(hd_ctx* ctx, int sms) {
     // The FP64 form stages twice the bytes per cell in tiles half as large, and
     // its frame changes are FP64-bound: per sweep 30.5 us against 42.9 as graph
@@ -253,28 +256,35 @@ bool plan_tiles(hd_ctx* ctx, int sms) {
     // 1,048,576.
     if (!ctx->fixed && ctx->Ctot > kTileCells64) return false;
     const hd::TileLimits lim = hd::tile_limits(ctx->fixed);
-    int64_t total = 0;
+    int64_t fewest = 0, total = 0;
     ctx->tiles.clear();
     for (const Rep& r : ctx->reps) {
         if (r.hm < 6) return false;
         const int least = r.hm < 12 ? 1 : 2;  // see wrap_half
-        hd::TileGrid g{int32_t(total), std::max(least, (r.m + lim.max_x - 1) / lim.max_x),
-                       std::max(least, (r.m + lim.max_y - 1) / lim.max_y)};
-        if (ctx->R == 1) {
-            const int most = std::max(1, r.hm / 4);
-            hd::TileGrid best = g;
-            for (int x = g.ntx; x <= most && x <= sms; ++x) {
-                const int y = std::min(most, sms / x);
-                if (y < g.nty) break;
-                const bool more = x * y > best.ntx * best.nty;
-                if (more || (x * y == best.ntx * best.nty && std::abs(x - y) < std::abs(best.ntx - best.nty))) {
-                    best.ntx = x;
-                    best.nty = y;
-                }
-            }
-            g = best;
-        }
+        const hd::TileGrid g{0, std::max(least, (r.m + lim.max_x - 1) / lim.max_x),
+                             std::max(least, (r.m + lim.max_y - 1) / lim.max_y)};
         ctx->tiles.push_back(g);
+        fewest += int64_t(g.ntx) * g.nty;
+    }
+    for (size_t i = 0; i < ctx->reps.size(); ++i) {
+        const Rep& r = ctx->reps[i];
+        hd::TileGrid& g = ctx->tiles[i];
+        // its share of the SMs that the fewest tiles would leave idle
+        const int64_t spare = sms > fewest ? int64_t(double(sms - fewest) * (double(r.m) * r.m) / double(ctx->Ctot)) : 0;
+        const int budget = int(std::min<int64_t>(sms, int64_t(g.ntx) * g.nty + spare));
+        const int most = std::max(1, r.hm / 4);
+        hd::TileGrid best = g;
+        for (int x = g.ntx; spare > 0 && x <= most && x <= budget; ++x) {
+            const int y = std::min(most, budget / x);
+            if (y < g.nty) break;
+            const bool more = x * y > best.ntx * best.nty;
+            if (more || (x * y == best.ntx * best.nty && std::abs(x - y) < std::abs(best.ntx - best.nty))) {
+                best.ntx = x;
+                best.nty = y;
+            }
+        }
+        g = best;
+        g.first = int32_t(total);
         total += int64_t(g.ntx) * g.nty;
     }
     ctx->tile_cfg.total = total;
