@@ -24,7 +24,7 @@ namespace hd {
 // the partial sums of the chunks are added in order by k_acf_norm.  What bounds
 // it is FP64: four fused multiply-adds per term at two lanes per clock and SM.
 // One thread per lag over all T instead ran a serial chain of loads and adds
-// (T = 4000, 401 lags, four replicas: 2.31 ms, here 0.06).
+// (T = 4000, 401 lags, four replicas: 2.31 ms, here 0.07).
 constexpr int kAcfLags = 128, kAcfChunk = 128;
 
 __global__ void __launch_bounds__(kAcfLags)
@@ -268,7 +268,7 @@ k_sq_amp(const Rep* __restrict__ reps, bool fixed, int nq, const int2* __restric
 // distinct h and k (15 FP64 operations each here) and four fused
 // multiply-adds per (h, k), against ~100 FP64-pipe operations for the division
 // and the sine and cosine of every (h, k) itself.  FP64 rate is the bound:
-// N = 65,536 and 441 wave vectors of 21 x 21 components 2.88 ms before, 0.31
+// N = 65,536 and 441 wave vectors of 21 x 21 components 2.88 ms before, 0.33
 // here.  The turn x / L is kept to 96 bits, so that h x / L mod 1 is exact to
 // 2^-64 for every 32-bit h (the division in double loses h 2^-53 of a turn).
 // ---------------------------------------------------------------------------
@@ -727,7 +727,7 @@ k_poscorr(const Rep* __restrict__ reps, int R, const uint8_t* __restrict__ cnt, 
 // k_poscorr on the global positions.  Three FP64 operations per pair remain.
 // N = 16,384, 40 windows of 0.5 out to 20 sigma: 13.3 ms with a division, two
 // square roots' worth of FP64 and a dozen shared FP64 atomics per ordered pair,
-// 0.25 here.
+// 0.18 here.
 // ---------------------------------------------------------------------------
 constexpr size_t kCorrSmem = 112 * 1024;  // two blocks per SM at least
 constexpr size_t kCorrBytes = 12;         // a thread's sum and count of one interval

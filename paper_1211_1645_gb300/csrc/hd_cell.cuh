@@ -94,8 +94,9 @@ __device__ __forceinline__ void global_position(const Rep& rep, const Frame& f, 
     } else {
         X = __dadd_rn(__dadd_rn(__dmul_rn(double(cx), rep.w), q.x), f.sx);
         Y = __dadd_rn(__dadd_rn(__dmul_rn(double(cy), rep.w), q.y), f.sy);
-        if (X >= rep.L) X = __dsub_rn(X, rep.L);
-        if (Y >= rep.L) Y = __dsub_rn(Y, rep.L);
+        // both non-negative: compared as bit patterns, off the FP64 pipe
+        if (!below_pos_bits(X, rep.L)) X = __dsub_rn(X, rep.L);
+        if (!below_pos_bits(Y, rep.L)) Y = __dsub_rn(Y, rep.L);
     }
 }
 

@@ -152,6 +152,12 @@ k_pass(const Rep* __restrict__ reps, const uint16_t* __restrict__ rep_of, const 
 
 // ---------------------------------------------------------------------------
 // Global positions from the cell frame: X = (cx w + u) + shift, wrapped once.
+// What bounds the FP64 form is the FP64 pipe, which takes a warp's instruction
+// for 16 cycles whatever lanes it serves: slot by slot a warp of cells ran the
+// arithmetic three or four times over, mostly for the few cells of more than
+// one disk.  There a block lists its disks first and takes one per lane
+// (N = 2^20: 44 -> 35 us, now as much the scattered stores); in the fixed form
+// the list costs more than it saves (N = 262,144: 8.8 us, with the list 9.7).
 // ---------------------------------------------------------------------------
 template <bool FIX, int CAP>
 __global__ void __launch_bounds__(256)
@@ -161,20 +167,48 @@ k_positions(const Rep* __restrict__ reps, int R, const Frame* __restrict__ cur, 
     const int r = find_rep<kGridCell>(reps, R, blockIdx.x);
     const Rep rep = reps[r];
     const int m = rep.m;
-    const uint32_t a = uint32_t(blockIdx.x - rep.blk_cell) * blockDim.x + threadIdx.x;
-    if (a >= uint32_t(m) * uint32_t(m)) return;
-    int cx, cy;
-    cell_coords(rep, a, cx, cy);
+    const uint32_t a0 = uint32_t(blockIdx.x - rep.blk_cell) * blockDim.x, a = a0 + threadIdx.x;
     const Frame f = cur[r];
-    const uint32_t cell = rep.coff + a;
-    const int n = min(int(cnt[cell]), CAP);
-    for (int k = 0; k < n; ++k) {
-        const P2<FIX> q = pos[size_t(k) * rep.stride32 + cell];
-        const int64_t id = rep.id_off + pid[size_t(k) * rep.stride32 + cell];
+    const int n = a < uint32_t(m) * uint32_t(m) ? min(int(cnt[rep.coff + a]), CAP) : 0;
+    auto write = [&](uint32_t own, int k) {
+        const size_t from = size_t(k) * rep.stride32 + (rep.coff + own);
+        const P2<FIX> q = pos[from];
+        const int64_t id = rep.id_off + pid[from];
+        int cx, cy;
+        cell_coords(rep, own, cx, cy);
         double X, Y;
         global_position<FIX>(rep, f, cx, cy, q, X, Y);
-        xy[2 * id] = __dmul_rn(X, rep.sigma);
-        xy[2 * id + 1] = __dmul_rn(Y, rep.sigma);
+        if (rep.sigma != 1.0) {
+            X = __dmul_rn(X, rep.sigma);
+            Y = __dmul_rn(Y, rep.sigma);
+        }
+        xy[2 * id] = X;
+        xy[2 * id + 1] = Y;
+    };
+    if constexpr (FIX) {
+        for (int k = 0; k < n; ++k) write(a, k);
+    } else {
+        __shared__ uint16_t s_list[256 * CAP];  // thread of the cell << 4 | slot
+        __shared__ int s_n;
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();
+        uint32_t mask[CAP];
+        int listed = 0, at = 0;
+#pragma unroll
+        for (int k = 0; k < CAP; ++k) {
+            mask[k] = __ballot_sync(0xffffffffu, n > k);
+            listed += __popc(mask[k]);
+        }
+        const uint32_t lane = threadIdx.x & 31u;
+        if (lane == 0u) at = atomicAdd(&s_n, listed);
+        at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+        for (int k = 0; k < CAP; ++k) {
+            if (n > k) s_list[at + __popc(mask[k] & ((1u << lane) - 1u))] = uint16_t(threadIdx.x << 4 | k);
+            at += __popc(mask[k]);
+        }
+        __syncthreads();
+        for (int d = int(threadIdx.x); d < s_n; d += int(blockDim.x)) write(a0 + (s_list[d] >> 4), s_list[d] & 15);
     }
 }
 
