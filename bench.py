@@ -325,7 +325,7 @@ def time_extras(args, rank, world, dev):
                             "trial_moves_per_s": c["trial_moves_per_s"]} for c in stable]}
     best, table = autotune(args.N, args.eta, args.delta, args.seed + rank, precision=args.form,
                            cell_mins=(2.0, 2.2, 2.4), kernels=("split", "persistent"), block_threads=(128, 256),
-                           threads_per_cell=(1, 2), strips=(1, 8, 16, 24), sweeps=args.sweeps_per_step, steps=2)
+                           threads_per_cell=(1, 2), strips=(0, 1, 8, 16, 24), sweeps=args.sweeps_per_step, steps=2)
     if best:
         rt = time_form(args, args.form, rank, world, steps, warm, cell_min=best["cell_min"],
                        block_threads=best["block_threads"], sweep_kernel=best["sweep_kernel"],

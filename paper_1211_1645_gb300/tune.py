@@ -11,7 +11,8 @@ steps of the library on the current GPU:
   per block of the split kernels, the threads per active cell of the
   split colour pass (1, or a group of 2, 4 or 8 lanes that split the overlap
   tests and combine them with a warp ballot), and for the split one-thread
-  pass the strips of the step graph's wavefront (hd_opts.strips);
+  pass the strips of the step graph's wavefront (hd_opts.strips; 0 among
+  the candidates: the library's own order, mostly one launch of many sweeps);
 * for a batch of replicas at different state points, such as the
   equation-of-state scan of Sec. IV.A (``autotune_replicas``): first each
   replica's own cell side, timed on that replica alone, then the threads per
