@@ -109,7 +109,8 @@ typedef struct hd_opts {
                                 the sweeps of a draw table (up to 256) run as one
                                 launch, of a box that fits one block's shared
                                 memory or of tiles of cells staged there (FP64: up
-                                to 655,360 cells); else strips, 16 when the colour
+                                to 655,360 cells; fewer where cells hold more than
+                                a disk on average); else strips, 16 when the colour
                                 pass is 1.5 to 3.5 waves of resident blocks deep, 8
                                 when it is deeper, none when it is shallower;
                                 1: none; 2 .. 64: K strips (at most m / 2, and

@@ -42,6 +42,9 @@ constexpr int kAutoStrips = 16;   // strips chosen when the colour pass is 1.5 t
 constexpr int kAutoStripsDeep = 8;  // ... and when it is deeper
 constexpr int kMaxBranches = 64;  // replicas on concurrent branches of a captured step
 constexpr int kMaxTiledReplicas = 1024;       // replicas of a context on the tile or box sweep (bounds its scratch)
+constexpr int kBranchedReplicas = 16;         // see plan_tiles
+constexpr double kCrowdedTiles = 9e5;         // disks times disks per cell of a crowded context on the tile or box sweep
+constexpr double kCrowdedTiles64 = 7e5;       // ... FP64 form
 constexpr int64_t kTileCells64 = 640 * 1024;  // cells of an FP64 context up to which the tile sweep is the faster
 
 struct Plan {
@@ -266,6 +269,11 @@ bool plan_tiles(hd_ctx* ctx, int sms) {
         ctx->tiles.push_back(g);
         fewest += int64_t(g.ntx) * g.nty;
     }
+    // A few large fixed-point replicas of between one and two tiles per SM: a sweep
+    // is two rounds of tiles, and graph branches take no longer (us per sweep, as
+    // tiles and branches: ten of 100,000 32.0 and 30.0, four of 262,144 32.9 and
+    // 30.5, sixteen of 65,536 36.8 and 36.8 measured; twenty of 100,000 71 and 75).
+    if (ctx->fixed && ctx->R > 1 && ctx->R <= kBranchedReplicas && fewest > sms && fewest < 2 * sms) return false;
     for (size_t i = 0; i < ctx->reps.size(); ++i) {
         const Rep& r = ctx->reps[i];
         hd::TileGrid& g = ctx->tiles[i];
@@ -1086,7 +1094,17 @@ hd_status hd_batch_init(hd_ctx** out, int32_t R, const int64_t* N, const double*
     // tiles, where the launch boundary of the split kernels costs more than
     // their work (per sweep at N = 256 4.6 us against 11.1 as a serial graph, at
     // 65,536 8.2 against 20.8, at 2^20 30 against 35 as 16 strips).
-    if (ok && split1 && cap == 4 && R <= kMaxTiledReplicas && (R == 1 ? o.strips == 0 : o.replica_branches == 0)) {
+    // Not for large systems of more than a disk per cell (cells wider than they
+    // need be): crowded cells and their neighbours take the blocks' longer path,
+    // two and more trials each in the cells around a tile too (us per sweep as
+    // tiles and as strips, fixed form: N = 2^20 at 1.08 disks per cell 58 and 53, at
+    // 1.5 117 and 88; 524,288 at 1.5 66 and 71, at 1.76 80 and 79; FP64: 524,288 at
+    // 1.29 92 and 103, at 1.52 133 and 122).
+    double crowd = 0.0;
+    for (const Rep& r : ctx->reps) crowd += double(r.N) * double(r.N) / (double(r.m) * r.m);
+    const bool crowded = ctx->Ntot > ctx->Ctot && crowd > (ctx->fixed ? kCrowdedTiles : kCrowdedTiles64);
+    if (ok && split1 && cap == 4 && !crowded && R <= kMaxTiledReplicas &&
+        (R == 1 ? o.strips == 0 : o.replica_branches == 0)) {
         int dev = 0, sms = 0;
         ok = cudaGetDevice(&dev) == cudaSuccess &&
              cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess;
