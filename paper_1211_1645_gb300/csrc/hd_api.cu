@@ -2033,17 +2033,19 @@ hd_status hd_positional_corr(hd_ctx* ctx, const int32_t* hk0, int32_t nr, double
     const Range range("hd_positional_corr");
     if (!ctx || !hk0 || !C || nr < 1 || nr > 1024 || !(dr > 0.0)) return HD_ERR_ARG;
     if (ctx->sticky != HD_OK) return HD_ERR_STATE;
-    // cell reach that holds every pair within the largest window, r_nr + 1 (sigma units)
-    const double rmax = double(nr) * dr + 1.0;
+    // cell reach that holds every pair within the largest window, r_nr + 1 in
+    // units of sigma, with a cell to spare: the pair kernel takes distances in
+    // the cell frame, which are the minimum image's up to half the box
+    const double rmax = double(nr) * (dr / ctx->sigma) + 1.0;
     int reach = 0;
-    for (const Rep& r : ctx->reps) reach = std::max(reach, int(std::ceil(rmax / r.w)) + 1);
+    for (const Rep& r : ctx->reps) {
+        const double cells = std::ceil(rmax / r.w) + 1.0;  // compared before it is an integer: dr may be anything
+        if (!(2.0 * cells + 1.0 <= double(r.m))) return HD_ERR_REACH;
+        reach = std::max(reach, int(cells));
+    }
     for (const Rep& r : ctx->reps)
         if (2 * reach + 1 > r.m) return HD_ERR_REACH;
-    // the pair kernel takes distances in the cell frame, which are the minimum
-    // image's up to half the box: the windows (r in units of sigma) end a cell
-    // short of the reach
-    bool pairs = hd::corr_pairs_fit(nr);
-    for (const Rep& r : ctx->reps) pairs = pairs && double(nr) * (dr / ctx->sigma) + 1.0 <= double(reach - 1) * r.w;
+    const bool pairs = hd::corr_pairs_fit(nr);
     hd_status st;
     if (!pairs) {
         st = enqueue_chi(ctx, hk0);
