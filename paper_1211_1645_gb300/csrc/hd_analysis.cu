@@ -8,7 +8,6 @@
 #include <math_constants.h>
 
 #include <algorithm>
-#include <mutex>
 #include <vector>
 
 #include "hd_kernels.h"
@@ -1049,13 +1048,9 @@ cudaError_t launch_sq(const LaunchCfg& c, int nq, const int2* hk, const double* 
 
 cudaError_t launch_sq_pairs(const LaunchCfg& c, int nq, int nh, int nk, bool grid, const int* comp, const ushort2* pair,
                             const double* xy, int nbx, double2* part, double* S, int* best) {
-    static std::once_flag attr_once;
-    std::call_once(attr_once, [] {
-        const int most = int((kPairDisks * (kPairMax + 1) + kTurnTable) * sizeof(double2));
-        cudaFuncSetAttribute(k_sq_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-        cudaFuncSetAttribute(k_sq_grid, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    });
-    cudaError_t e;
+    static OncePerDevice once;
+    cudaError_t e = allow_smem(once, (kPairDisks * (kPairMax + 1) + kTurnTable) * sizeof(double2), k_sq_pairs, k_sq_grid);
+    if (e != cudaSuccess) return e;
     if (grid)
         e = launch_k(k_sq_grid, dim3(unsigned(nbx), 1, unsigned(c.R)), dim3(kPairThreads),
                      size_t(kPairDisks * (nk + 1 + nh / 2) + kTurnTable) * sizeof(double2), c.stream, c.reps, c.fixed, nh, nk,
@@ -1083,11 +1078,9 @@ cudaError_t launch_chi(const LaunchCfg& c, int64_t Ntot, const int2* hk0, const 
 template <int CAP>
 static cudaError_t poscorr_t(const LaunchCfg& c, CellBufs cells, const double* xy, const double2* chi, int nr,
                              double dr, int reach, double* acc) {
-    static std::once_flag attr_once;
-    std::call_once(attr_once, [] {
-        cudaFuncSetAttribute(k_poscorr<CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(3 * kMaxCorrWindows * sizeof(double)));
-    });
+    static OncePerDevice once;
+    const cudaError_t e = allow_smem(once, 3 * kMaxCorrWindows * sizeof(double), k_poscorr<CAP>);
+    if (e != cudaSuccess) return e;
     return launch_k(k_poscorr<CAP>, dim3(c.blocks_cell), dim3(c.threads), size_t(3 * nr) * sizeof(double), c.stream,
                     c.reps, c.R, (const uint8_t*)cells.cnt, (const int32_t*)cells.pid, xy, chi, nr, dr, reach, acc);
 }
@@ -1105,10 +1098,9 @@ static cudaError_t corr_stage_t(const LaunchCfg& c, unsigned cells, const Frame*
 template <int CAP, int NT>
 static cudaError_t corr_pairs_t(const LaunchCfg& c, unsigned cells, CellBufs b, const double2* gpos, const double2* chi,
                                 const float2* off, int nr, double dr, int reach, double2* acc) {
-    static std::once_flag attr_once;
-    std::call_once(attr_once, [] {
-        cudaFuncSetAttribute(k_corr_pairs<CAP, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kCorrSmem));
-    });
+    static OncePerDevice once;
+    const cudaError_t e = allow_smem(once, kCorrSmem, k_corr_pairs<CAP, NT>);
+    if (e != cudaSuccess) return e;
     // a little under one cell per thread: at liquid densities a block's disks
     // are then a single round of its threads
     const int cells_per_block = NT * 7 / 8;

@@ -1119,15 +1119,17 @@ hd_status hd_batch_init(hd_ctx** out, int32_t R, const int64_t* N, const double*
         } else if (ok && plan_tiles(ctx, sms)) {
             hd::TileCfg& t = ctx->tile_cfg;
             hd::TileGrid* grids = nullptr;
-            ok = hd::tile_blocks(ctx->cfg(), &t.blocks) == cudaSuccess && t.blocks > 0;
-            t.blocks = int(std::min<int64_t>(t.blocks, t.total));
-            ok = ok && dev_alloc(ctx, &grids, size_t(R));
-            ok = ok && dev_alloc(ctx, &t.sync, hd::tile_sync_words(t.total));
-            ok = ok && dev_alloc(ctx, &spill, size_t(t.blocks) * hd::tile_limits(ctx->fixed).spill);
-            ok = ok && cudaMemcpy(grids, ctx->tiles.data(), sizeof(hd::TileGrid) * size_t(R), cudaMemcpyHostToDevice) == cudaSuccess;
-            t.grids = grids;
-            t.spill = spill;
-            ctx->tiled = true;
+            ok = hd::tile_blocks(ctx->cfg(), &t.blocks) == cudaSuccess;
+            if (t.blocks > 0) {  // else no block is ever resident here: the former order of the launches
+                t.blocks = int(std::min<int64_t>(t.blocks, t.total));
+                ok = ok && dev_alloc(ctx, &grids, size_t(R));
+                ok = ok && dev_alloc(ctx, &t.sync, hd::tile_sync_words(t.total));
+                ok = ok && dev_alloc(ctx, &spill, size_t(t.blocks) * hd::tile_limits(ctx->fixed).spill);
+                ok = ok && cudaMemcpy(grids, ctx->tiles.data(), sizeof(hd::TileGrid) * size_t(R), cudaMemcpyHostToDevice) == cudaSuccess;
+                t.grids = grids;
+                t.spill = spill;
+                ctx->tiled = true;
+            }
         }
         if (ctx->tiled) ctx->strips = 1;
     }

@@ -258,13 +258,9 @@ template <bool FIX, int CAP, int T, int NT>
 static cudaError_t fused_t(const LaunchCfg& c, const Frame* table, int j, CellBufs a, CellBufs b,
                            unsigned long long* counters, int* err) {
     constexpr size_t smem = Fused<FIX, CAP, T>::kSmem;
-    static bool configured = false;
-    if (!configured) {
-        const cudaError_t e = cudaFuncSetAttribute(k_sweep_fused<FIX, CAP, T, NT>,
-                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-        if (e != cudaSuccess) return e;
-        configured = true;
-    }
+    static OncePerDevice once;
+    const cudaError_t e = allow_smem(once, smem, k_sweep_fused<FIX, CAP, T, NT>);
+    if (e != cudaSuccess) return e;
     return launch_k(k_sweep_fused<FIX, CAP, T, NT>, dim3(c.blocks_tile), dim3(NT), smem, c.stream, c.reps, c.R, table,
                     j, (const uint8_t*)a.cnt, (const P2<FIX>*)a.pos, (const int32_t*)a.pid, b.cnt, (P2<FIX>*)b.pos,
                     b.pid, counters, err);

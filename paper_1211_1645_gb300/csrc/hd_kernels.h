@@ -9,6 +9,7 @@
 
 #include "hd_device.cuh"
 #include "hd_exact.cuh"
+#include "hd_once.h"
 
 namespace hd {
 
@@ -67,6 +68,20 @@ cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sme
     cfg.attrs = attr;
     cfg.numAttrs = (s != nullptr && !g_no_pdl) ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
+// The kernels' dynamic shared-memory limit on the current device (an attribute
+// of the kernel there), set once per device.
+template <class... K>
+cudaError_t allow_smem(OncePerDevice& once, size_t bytes, K... kernels) {
+    int dev = 0;
+    const cudaError_t got = cudaGetDevice(&dev);
+    if (got != cudaSuccess) return got;
+    return once(dev, [&] {
+        cudaError_t e = cudaSuccess;
+        ((e = e == cudaSuccess ? cudaFuncSetAttribute(kernels, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes)) : e), ...);
+        return e;
+    });
 }
 
 cudaError_t launch_draws(const LaunchCfg& c, Frame* table, Frame* cur, uint64_t* sweep_ctr, int nchunk);

@@ -6,7 +6,6 @@
 // Pair vectors are formed in the cell frame: for disks i and j whose cells
 // differ by (dcx, dcy), r = (u_j + dcx * w) - u_i, which is exact in the
 // fixed-point form and has one fixed rounding order in FP64.
-#include <mutex>
 #include <type_traits>
 
 #include "hd_kernels.h"
@@ -861,11 +860,9 @@ k_psi6_reduce(const Rep* __restrict__ reps, unsigned long long* __restrict__ tot
 template <bool FIX, int CAP>
 static cudaError_t hist_t(const LaunchCfg& c, const HistCfg& h, CellBufs cells, unsigned long long* hist) {
     if (h.halo <= kHistMaxHalo) {
-        static std::once_flag attr_once;
-        std::call_once(attr_once, [] {
-            cudaFuncSetAttribute(k_hist_tile<FIX, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 int(hist_stage_bytes<FIX, CAP>(kHistMaxHalo, kMaxFitBins)));
-        });
+        static OncePerDevice once;
+        const cudaError_t e = allow_smem(once, hist_stage_bytes<FIX, CAP>(kHistMaxHalo, kMaxFitBins), k_hist_tile<FIX, CAP>);
+        if (e != cudaSuccess) return e;
         return launch_k(k_hist_tile<FIX, CAP>, dim3(c.blocks_t32), dim3(kTileThreads),
                         hist_stage_bytes<FIX, CAP>(h.halo, h.K), c.stream, c.reps, c.R, h.K, h.edges,
                         h.edgesF, (const uint8_t*)cells.cnt, (const P2<FIX>*)cells.pos, (const int32_t*)cells.pid,
@@ -900,10 +897,9 @@ int psi6_rows() { return kPsiThreads / 32; }
 template <bool FIX, int CAP>
 static cudaError_t psi6_t(const LaunchCfg& c, CellBufs cells, double2* local, unsigned long long* total, int* err) {
     constexpr size_t smem = psi6_stage_bytes<FIX, CAP>(kPsiThreads / 32);
-    static std::once_flag attr_once;
-    std::call_once(attr_once, [] {
-        cudaFuncSetAttribute(k_psi6<FIX, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
-    });
+    static OncePerDevice once;
+    const cudaError_t e = allow_smem(once, smem, k_psi6<FIX, CAP>);
+    if (e != cudaSuccess) return e;
     return launch_k(k_psi6<FIX, CAP>, dim3(c.blocks_t32), dim3(kPsiThreads), smem, c.stream, c.reps, c.R,
                     (const uint8_t*)cells.cnt, (const P2<FIX>*)cells.pos, (const int32_t*)cells.pid, local, total,
                     err);

@@ -16,7 +16,6 @@
 // loads and pair tests over G lanes (shorter per-lane dependency chains,
 // more loads in flight per cell) and repeats the cell's common work (the
 // generator, the shuffle, the boundary test) on every lane.
-#include <mutex>
 
 #include "hd_cell.cuh"
 #include "hd_kernels.h"
@@ -184,13 +183,10 @@ static cudaError_t pass_group_t(const LaunchCfg& c, const Frame* table, int j, i
     const int threads = c.threads * G;
     if (threads > kGroupMaxThreads) return cudaErrorInvalidConfiguration;
     const size_t smem = group_smem<FIX, CAP, G>(threads);
-    static std::once_flag attr_once;
-    std::call_once(attr_once, [&] {
-        cudaFuncSetAttribute(k_pass_group<FIX, CAP, NTC, true, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(group_smem<FIX, CAP, G>(kGroupMaxThreads)));
-        cudaFuncSetAttribute(k_pass_group<FIX, CAP, NTC, false, G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(group_smem<FIX, CAP, G>(kGroupMaxThreads)));
-    });
+    static OncePerDevice once;
+    const cudaError_t e = allow_smem(once, group_smem<FIX, CAP, G>(kGroupMaxThreads), k_pass_group<FIX, CAP, NTC, true, G>,
+                                     k_pass_group<FIX, CAP, NTC, false, G>);
+    if (e != cudaSuccess) return e;
     if (c.R == 1)
         return launch_k(k_pass_group<FIX, CAP, NTC, true, G>, dim3(c.blocks_act), dim3(threads), smem, c.stream,
                         c.reps, c.rep_of_act, *c.rep0, table, j, p, (const uint8_t*)cells.cnt, (P2<FIX>*)cells.pos,

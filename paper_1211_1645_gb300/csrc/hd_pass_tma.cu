@@ -15,7 +15,6 @@
 // each thread then finds its neighbours at fixed offsets from its own index.
 // A half-column outside [0, m/2) (the periodic wrap at a row end) and slots
 // beyond the second are read from global memory instead.
-#include <mutex>
 
 #include "hd_cell.cuh"
 #include "hd_kernels.h"
@@ -245,11 +244,9 @@ template <bool FIX, int CAP, bool NT1>
 static cudaError_t pass_tma_t(const LaunchCfg& c, const Frame* table, int j, int p, CellBufs cells,
                               unsigned long long* counters, int* err) {
     const size_t smem = seg_smem_bytes<FIX>(c.threads);
-    static std::once_flag attr_once;
-    std::call_once(attr_once, [] {
-        cudaFuncSetAttribute(k_pass_tma<FIX, CAP, NT1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(seg_smem_bytes<FIX>(256)));
-    });
+    static OncePerDevice once;
+    const cudaError_t e = allow_smem(once, seg_smem_bytes<FIX>(256), k_pass_tma<FIX, CAP, NT1>);
+    if (e != cudaSuccess) return e;
     return launch_k(k_pass_tma<FIX, CAP, NT1>, dim3(c.blocks_seg), dim3(c.threads), smem, c.stream, c.reps, c.R,
                     table, j, p, (const uint8_t*)cells.cnt, (P2<FIX>*)cells.pos, cells.pid, counters, err);
 }

@@ -43,7 +43,6 @@
 // only) and the fixed form's neighbour slots are staged with cp.async (a weak
 // load in the memory model), all after the acquire that orders them behind
 // the items they depend on.
-#include <mutex>
 
 #include "hd_kernels.h"
 #include "hd_sweep_cell.cuh"
@@ -175,14 +174,13 @@ k_sweep_persist(const Rep* __restrict__ reps, int R, const Rep rep1, const Frame
 namespace {
 
 template <bool FIX, int CAP, int NTC>
+cudaError_t persist_allow() {
+    static OncePerDevice once;
+    return allow_smem(once, pass_smem<FIX, CAP>(256), k_sweep_persist<FIX, CAP, NTC, true>, k_sweep_persist<FIX, CAP, NTC, false>);
+}
+
+template <bool FIX, int CAP, int NTC>
 auto persist_kernel(const LaunchCfg& c) {
-    static std::once_flag attr_once;
-    std::call_once(attr_once, [] {
-        cudaFuncSetAttribute(k_sweep_persist<FIX, CAP, NTC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(pass_smem<FIX, CAP>(256)));
-        cudaFuncSetAttribute(k_sweep_persist<FIX, CAP, NTC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(pass_smem<FIX, CAP>(256)));
-    });
     return c.R == 1 ? k_sweep_persist<FIX, CAP, NTC, true> : k_sweep_persist<FIX, CAP, NTC, false>;
 }
 
@@ -192,6 +190,8 @@ cudaError_t persist_t(const LaunchCfg& c, const Frame* table, int nsweeps, CellB
     if (c.persist_blocks < 1) return cudaErrorInvalidConfiguration;
     const uint32_t NI = uint32_t(c.blocks_seg);
     const int blocks = int(std::min<uint64_t>(uint64_t(c.persist_blocks), 5ull * uint64_t(nsweeps) * NI));
+    const cudaError_t e = persist_allow<FIX, CAP, NTC>();
+    if (e != cudaSuccess) return e;
     return launch_k(persist_kernel<FIX, CAP, NTC>(c), dim3(blocks), dim3(c.threads), pass_smem<FIX, CAP>(c.threads),
                     c.stream, c.reps, c.R, c.R == 1 ? *c.rep0 : Rep{}, table, nsweeps, NI, a, b, counters, err, sync,
                     c.persist_stall ? 1u << 12 : kPersistPolls, c.persist_stall ? 0 : -1);
@@ -209,6 +209,7 @@ cudaError_t persist_grid_t(const LaunchCfg& c, int* blocks) {
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = persist_allow<FIX, CAP, NTC>();
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, persist_kernel<FIX, CAP, NTC>(c), c.threads,
                                                           pass_smem<FIX, CAP>(c.threads));

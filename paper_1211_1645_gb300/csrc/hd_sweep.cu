@@ -15,7 +15,6 @@
 // in the sweep's random order.  Cells of one colour are never neighbours, so
 // every thread of a pass owns its cell outright and only reads the
 // (unchanging) cells of the other colours.
-#include <mutex>
 
 #include "hd_kernels.h"
 #include "hd_sweep_cell.cuh"
@@ -246,13 +245,9 @@ template <bool FIX, int CAP, int NTC>
 static cudaError_t pass_t(const LaunchCfg& c, const Frame* table, int j, int p, CellBufs cells,
                           unsigned long long* counters) {
     const size_t smem = pass_smem<FIX, CAP>(c.threads);
-    static std::once_flag attr_once;
-    std::call_once(attr_once, [&] {
-        cudaFuncSetAttribute(k_pass<FIX, CAP, NTC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(pass_smem<FIX, CAP>(256)));
-        cudaFuncSetAttribute(k_pass<FIX, CAP, NTC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(pass_smem<FIX, CAP>(256)));
-    });
+    static OncePerDevice once;
+    const cudaError_t e = allow_smem(once, pass_smem<FIX, CAP>(256), k_pass<FIX, CAP, NTC, true>, k_pass<FIX, CAP, NTC, false>);
+    if (e != cudaSuccess) return e;
     if (c.R == 1) {
         // a strip covers its active-cell range; the whole plane otherwise
         const int blocks = c.act_hi != ~0u ? int((c.act_hi - c.act_lo + uint32_t(c.threads) - 1) / uint32_t(c.threads))

@@ -26,7 +26,6 @@
 // up after `polls` polls sets bit 16 of err and an abort word, and every
 // block leaves.
 #include <algorithm>
-#include <mutex>
 
 #include "hd_kernels.h"
 #include "hd_tile.h"
@@ -785,14 +784,13 @@ struct LargeBox { static constexpr int HB = 18, NT = 512, ND = 256; };
 namespace {
 
 template <bool FIX, int NTC>
+cudaError_t tile_allow() {
+    static OncePerDevice once;
+    return allow_smem(once, TileStage<FIX>::kBytes, k_sweep_tile<FIX, NTC, true>, k_sweep_tile<FIX, NTC, false>);
+}
+
+template <bool FIX, int NTC>
 auto tile_kernel(bool one) {
-    static std::once_flag attr_once;
-    std::call_once(attr_once, [] {
-        cudaFuncSetAttribute(k_sweep_tile<FIX, NTC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(TileStage<FIX>::kBytes));
-        cudaFuncSetAttribute(k_sweep_tile<FIX, NTC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(TileStage<FIX>::kBytes));
-    });
     return one ? k_sweep_tile<FIX, NTC, true> : k_sweep_tile<FIX, NTC, false>;
 }
 
@@ -801,6 +799,7 @@ cudaError_t tile_blocks_t(bool one, int* blocks) {
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = tile_allow<FIX, NTC>();
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tile_kernel<FIX, NTC>(one), TileShape<FIX>::NT,
                                                           TileStage<FIX>::kBytes);
@@ -812,6 +811,8 @@ template <bool FIX, int NTC>
 cudaError_t tile_t(const LaunchCfg& c, const TileCfg& t, const Frame* table, int nsweeps, CellBufs a, CellBufs b,
                    unsigned long long* counters, int* err) {
     const int blocks = int(std::min<int64_t>(t.blocks, t.total));
+    const cudaError_t e = tile_allow<FIX, NTC>();
+    if (e != cudaSuccess) return e;
     return launch_k(tile_kernel<FIX, NTC>(c.R == 1), dim3(blocks), dim3(TileShape<FIX>::NT), TileStage<FIX>::kBytes,
                     c.stream, c.reps, (const TileGrid*)t.grids, c.R, c.R == 1 ? *c.rep0 : Rep{}, t.grid0, table, nsweeps,
                     uint32_t(t.total), a, b, counters, err, t.sync, t.spill, kTilePolls);
@@ -822,8 +823,9 @@ cudaError_t box_t(const LaunchCfg& c, void* spill, const Frame* table, int nswee
                   unsigned long long* counters, int* err) {
     constexpr size_t smem = box_smem<FIX, B::HB>();
     constexpr auto kernel = k_sweep_box<FIX, NTC, B::HB, B::NT, B::ND>;
-    static std::once_flag attr_once;
-    std::call_once(attr_once, [] { cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)); });
+    static OncePerDevice once;
+    const cudaError_t e = allow_smem(once, smem, kernel);
+    if (e != cudaSuccess) return e;
     return launch_k(kernel, dim3(c.R), dim3(B::NT + B::ND), smem, c.stream, c.reps, table, nsweeps, a, b, counters, err, spill);
 }
 
