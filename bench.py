@@ -24,8 +24,7 @@ with the local psi_j field per step).
 Roofline: after the timed steps two more steps replay as profiled graphs
 (a timing event around every kernel node); each kernel class is charged its
 share of those event times x the graph-timed ms_per_step (sweeps that ran as
-one launch: what the measurement kernels leave of the step, per sweep), and
-the dominant class's time per launch gives its achieved rates against three roofs (HBM
+one launch: from two profiled calls of hd_sweep, per sweep), and the dominant class's time per launch gives its achieved rates against three roofs (HBM
 copy bandwidth, L2-resident copy bandwidth, warp-instruction issue).  The
 binding roof is picked from the committed ncu counters of that kernel, which
 `roofline.ncu` repeats while the kernel's sources are unchanged.
@@ -246,12 +245,18 @@ def time_form(args, form, rank, world, steps, warmup, sampler=None, N=None, eta=
     kt = sysg.kernel_times()
     sysg.profile(False)
     if l1["sweep"][1] > l0["sweep"][1]:
-        # the timed steps ran their sweeps as one launch each; the profiled
-        # replays time the split kernels instead, so only their measurement
-        # kernels are kept and the sweeps are charged the rest of the step
-        kt = {k: v for k, v in kt.items() if k not in ("draws", "rebuild", "pass") and v[1]}
-        rest = ms / steps * PROFILED_STEPS - sum(v[0] for v in kt.values())
-        kt["sweep"] = (max(rest, 0.0), S * PROFILED_STEPS)
+        # the timed steps ran many sweeps per launch; the profiled replays time
+        # the split kernels instead, so only their measurement kernels are kept,
+        # and the sweeps are timed as hd_sweep launches them
+        sysg.profile(True)
+        for _ in range(PROFILED_STEPS):
+            flush.zero_()
+            sysg.sweep(S)
+        sw = sysg.kernel_times()
+        sysg.profile(False)
+        kt = {k: v for k, v in kt.items() if k not in ("rebuild", "pass") and v[1]}
+        kt["draws"] = sw["draws"]
+        kt["sweep"] = (sw["sweep"][0], S * PROFILED_STEPS)
     geo = sysg.geometry()
     series = sysg.series()
     final_xy = sysg.positions() if keep_positions else None

@@ -456,7 +456,9 @@ hd_status hd_psi6_mean_noalloc(const double *psi_local_device, int64_t N, double
  * Instrumentation (no counterpart in the paper).  The library counts every
  * kernel it launches, by class.  With profiling enabled it also brackets each
  * launch with CUDA events on the context stream; hd_kernel_times then
- * synchronises and reports the summed device time per class.  Enabling
+ * synchronises and reports the summed device time per class.  hd_sweep makes
+ * the same launches as without profiling; hd_run's steps run the split kernels
+ * instead (see hd_run).  Enabling
  * (enable != 0) resets both tallies; disabling keeps them readable.
  * ms[HD_KERNEL_CLASSES] and launches[HD_KERNEL_CLASSES] are host arrays, either
  * may be NULL.

@@ -708,12 +708,12 @@ cudaError_t enqueue_strips(hd_ctx* ctx, cudaStream_t s, int nc) {
 // the table's sweeps in one tile-sweep or persistent launch, or per sweep
 // either one fused launch or a rebuild and four colour passes).
 // While a step graph is captured (not for a profiled graph, whose event nodes
-// time each kernel in order), the sweeps of a one-replica context with strips
-// run as a graph wavefront, and those of a batch with replica branches as
-// one branch per replica.
+// time each split kernel in order), the sweeps of a one-replica context with
+// strips run as a graph wavefront, and those of a batch with replica branches
+// as one branch per replica.
 cudaError_t enqueue_sweeps(hd_ctx* ctx, cudaStream_t s, int64_t n, bool capturing) {
     const hd::LaunchCfg c = ctx->cfg(s);
-    if (ctx->tiled && !ctx->profiling) {
+    if (ctx->tiled && !ctx->prof_capture) {
         cudaError_t e = cudaSuccess;
         for (int64_t left = n; left > 0 && e == cudaSuccess;) {
             const int nc = int(std::min<int64_t>(left, hd::kMaxChunk));
@@ -732,7 +732,7 @@ cudaError_t enqueue_sweeps(hd_ctx* ctx, cudaStream_t s, int64_t n, bool capturin
         }
         return e;
     }
-    if (ctx->tiled && n > 0) {  // profiled: the split kernels, whose rebuild expects the other generation cleared
+    if (ctx->tiled && n > 0) {  // a profiled step: the split kernels, whose rebuild expects the other generation cleared
         const cudaError_t e = cudaMemsetAsync(ctx->buf[ctx->cur ^ 1].cnt, 0, size_t(ctx->Ctot) + kCellPad, s);
         if (e != cudaSuccess) return e;
     }
