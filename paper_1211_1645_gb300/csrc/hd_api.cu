@@ -1128,6 +1128,12 @@ hd_status hd_batch_init(hd_ctx** out, int32_t R, const int64_t* N, const double*
                 ok = ok && cudaMemcpy(grids, ctx->tiles.data(), sizeof(hd::TileGrid) * size_t(R), cudaMemcpyHostToDevice) == cudaSuccess;
                 t.grids = grids;
                 t.spill = spill;
+                // Test hook for the bounded waits: with the environment variable
+                // HD_TEST_TILE_STALL=1 at creation, the first work item of every launch is
+                // never taken and the waits give up after 4096 polls, so that sweeps
+                // report HD_ERR_TIMEOUT.
+                const char* stall = std::getenv("HD_TEST_TILE_STALL");
+                t.stall = stall && stall[0] == '1' && stall[1] == '\0';
                 ctx->tiled = true;
             }
         }

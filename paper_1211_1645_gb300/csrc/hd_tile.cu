@@ -815,7 +815,7 @@ cudaError_t tile_t(const LaunchCfg& c, const TileCfg& t, const Frame* table, int
     if (e != cudaSuccess) return e;
     return launch_k(tile_kernel<FIX, NTC>(c.R == 1), dim3(blocks), dim3(TileShape<FIX>::NT), TileStage<FIX>::kBytes,
                     c.stream, c.reps, (const TileGrid*)t.grids, c.R, c.R == 1 ? *c.rep0 : Rep{}, t.grid0, table, nsweeps,
-                    uint32_t(t.total), a, b, counters, err, t.sync, t.spill, kTilePolls);
+                    uint32_t(t.total), a, b, counters, err, t.sync, t.spill, t.stall ? 1u << 12 : kTilePolls);
 }
 
 template <class B, bool FIX, int NTC>
@@ -883,7 +883,8 @@ size_t tile_sync_words(int64_t total) { return size_t(2 + total); }
 cudaError_t launch_sweeps_tile(const LaunchCfg& c, const TileCfg& t, const Frame* table, int nsweeps, CellBufs from,
                                CellBufs to, unsigned long long* counters, int* err) {
     if (nsweeps < 1 || nsweeps > kMaxChunk || c.cap != 4) return cudaErrorInvalidValue;
-    const cudaError_t e = cudaMemsetAsync(t.sync, 0, tile_sync_words(t.total) * sizeof(uint32_t), c.stream);
+    cudaError_t e = cudaMemsetAsync(t.sync, 0, tile_sync_words(t.total) * sizeof(uint32_t), c.stream);
+    if (e == cudaSuccess && t.stall) e = cudaMemsetAsync(t.sync, 1, 1, c.stream);  // the next ticket is 1
     if (e != cudaSuccess) return e;
     if (c.fixed)
         return c.ntc == 1 ? tile_t<true, 1>(c, t, table, nsweeps, from, to, counters, err)

@@ -29,6 +29,7 @@ struct TileCfg {
     int blocks;             // blocks resident at once
     uint32_t* sync;         // tile_sync_words(total): ticket, abort word, finished sweeps per tile
     void* spill;            // blocks x TileLimits::spill bytes
+    bool stall;             // test hook: ticket 0 is never taken, and waits give up early
 };
 
 // Blocks resident at once of the kernel that c selects.
