@@ -235,11 +235,12 @@ void set_f32_bounds(Rep& r) {
 }
 
 // The histogram's range [e0, eK) (sigma units) widened by the margin of pairs
-// hist_R cells apart.
+// hist_R cells apart, and the psi_6 margin (candidates two cells apart).
 void set_hist_f32_bounds(Rep& r, double e0, double eK) {
     const double M = hd::cells_f32_margin(r.w, r.hist_R);
     r.h_lo = std::nextafter(float(e0 - M), -HUGE_VALF);
     r.h_hi = std::nextafter(float(eK + M), HUGE_VALF);
+    r.psi_m = std::nextafter(float(hd::cells_f32_margin(r.w, 2)), HUGE_VALF);
 }
 
 // Tiles of every replica for the tile sweep (see hd_tile.h); false where it

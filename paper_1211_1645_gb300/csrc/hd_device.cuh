@@ -53,8 +53,9 @@ struct Rep {
     uint32_t key0, key1;
     // Float pre-tests (pair_clear, tile_clear, k_hist_tile): the cell side in
     // float; floats bracketing (2 sigma)^2 = 4, and the histogram's squared
-    // range [edge_0, edge_K), by the error bounds of the float estimates of d^2
-    float wf, d2_lo, d2_hi, h_lo, h_hi;
+    // range [edge_0, edge_K), by the error bounds of the float estimates of d^2;
+    // that bound for pairs two cells apart (psi_6, FP64 form)
+    float wf, d2_lo, d2_hi, h_lo, h_hi, psi_m;
     float wf_sigma;  // the cell side in units of sigma (wf is in the tile sweep's in the fixed form)
     double w_inv;    // 1 / w rounded
 };

@@ -524,7 +524,10 @@ struct PsiStage {
 // The general search of a disk's six nearest: ordered insertion of every
 // candidate by (r^2, id) from the staged rings 0, 1, 2, then rings in global
 // memory until the sixth is certified.  Out of line: the float search below
-// leaves it about one disk in a thousand.
+// leaves it about one disk in a thousand where cells hold up to four disks; wider
+// cells all come here.  In the FP64 form a candidate whose float estimate of
+// r^2 exceeds the sixth key by more than the estimate's error bound is farther
+// in FP64 too and is left out before its FP64 arithmetic.
 template <bool FIX, int CAP>
 static __device__ __noinline__ bool nearest_general(const Rep& rep, const PsiStage<FIX>& st, const uint8_t* cnt,
                                                     const P2<FIX>* pos, const int32_t* pid, int own, int cx, int cy,
@@ -533,6 +536,11 @@ static __device__ __noinline__ bool nearest_general(const Rep& rep, const PsiSta
     Nbr<FIX> nb;
     nb.n = 0;
     bool ok = false;
+    float mfx = 0.0f, mfy = 0.0f;  // FP64 form: float images of the disk's offsets
+    if constexpr (!FIX) {
+        mfx = approx_f32(me.x);
+        mfy = approx_f32(me.y);
+    }
     if (rmax >= 2) {
 #pragma unroll 1
         for (int ring = 0; ring <= 2; ++ring) {
@@ -550,6 +558,13 @@ static __device__ __noinline__ bool nearest_general(const Rep& rep, const PsiSta
                             const int32_t ry = (o.y + dcy * rep.W) - me.y;
                             nb.insert(int64_t(rx) * rx + int64_t(ry) * ry, idq, rx, ry);
                         } else {
+                            if (nb.n == 6) {  // (approx_f32 truncates; the product rounds up past the key itself)
+                                const float sx = __fsub_rn(__fadd_rn(approx_f32(o.x), __fmul_rn(float(dcx), rep.wf)), mfx);
+                                const float sy = __fsub_rn(__fadd_rn(approx_f32(o.y), __fmul_rn(float(dcy), rep.wf)), mfy);
+                                const float d2f = __fadd_rn(__fmul_rn(sx, sx), __fmul_rn(sy, sy));
+                                const float k5 = __fmul_ru(approx_f32(__longlong_as_double(nb.key[5])), 1.0f + 0x1p-19f);
+                                if (d2f > __fadd_ru(k5, rep.psi_m)) continue;
+                            }
                             const double rx = __dsub_rn(__dadd_rn(o.x, __dmul_rn(double(dcx), rep.w)), me.x);
                             const double ry = __dsub_rn(__dadd_rn(o.y, __dmul_rn(double(dcy), rep.w)), me.y);
                             nb.insert(__double_as_longlong(__dadd_rn(__dmul_rn(rx, rx), __dmul_rn(ry, ry))), idq, rx, ry);
