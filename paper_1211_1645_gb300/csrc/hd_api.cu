@@ -943,6 +943,7 @@ hd_status hd_batch_init(hd_ctx** out, int32_t R, const int64_t* N, const double*
     }
     int64_t cell_off = 0, id_off = 0;
     int blk_cell = 0, blk_act = 0, blk_tile = 0, blk_t32 = 0, blk_seg = 0, band0 = 0;
+    const int psi_rows = hd::psi6_rows(ctx->fixed, cap);
     for (int r = 0; r < R; ++r) {
         Rep rep = plans[size_t(r)].rep;
         rep.cell_off = cell_off;
@@ -960,7 +961,7 @@ hd_status hd_batch_init(hd_ctx** out, int32_t R, const int64_t* N, const double*
             rep.tx_mul = uint32_t((((uint64_t(1) << l) - uint64_t(rep.tiles_x)) << 32) / uint64_t(rep.tiles_x) + 1u);
             rep.tx_sh = l - 1;
         }
-        blk_t32 += int(int64_t(rep.tiles_x) * ((rep.m + hd::psi6_rows() - 1) / hd::psi6_rows()));
+        blk_t32 += int(int64_t(rep.tiles_x) * ((rep.m + psi_rows - 1) / psi_rows));
         rep.blk_seg = blk_seg;
         rep.nseg = (rep.hm + ctx->threads - 1) / ctx->threads;
         rep.segw = (rep.hm + rep.nseg - 1) / rep.nseg;

@@ -35,7 +35,7 @@ struct Rep {
     int32_t W, D;       // fixed point: cell side, maximum step (units 2^-24 sigma)
     int32_t hist_R;     // cell reach of the contact histogram
     int32_t hm_sh;
-    int32_t blk_t32;    // first block of the replica in 32-column tile grids (32 x psi6_rows() cells)
+    int32_t blk_t32;    // first block of the replica in 32-column tile grids (32 x psi6_rows cells)
     int32_t tiles_x;    // such tiles per row of cells, ceil(m / 32)
     uint32_t tx_mul;    // tx_mul, tx_sh: divide by tiles_x >= 2 with div_by
     int32_t tx_sh;

@@ -34,7 +34,7 @@ struct LaunchCfg {
     int blocks_cell;   // whole-cell grid size (all replicas)
     int blocks_act;    // active-cell grid size (all replicas)
     int blocks_tile;   // fused-sweep tile grid size (all replicas)
-    int blocks_t32;    // 32 x psi6_rows() cell-tile grid size (all replicas)
+    int blocks_t32;    // 32 x psi6_rows cell-tile grid size (all replicas)
     int blocks_seg;    // half-row segment grid size of one colour pass (all replicas)
     int persist_blocks;  // grid of the persistent sweep (resident blocks), from persist_grid
     bool persist_stall;  // test hook: the persistent sweep withholds one item and gives up waiting early
@@ -143,7 +143,7 @@ cudaError_t launch_fit(const LaunchCfg& c, int K, const double* qr, const unsign
 // replica's once, divides by N and leaves total zero.  psi6_rows: rows of cells
 // of the 32-column tile grid (blk_t32, blocks_t32).
 size_t psi6_total_words(int R);
-int psi6_rows();
+int psi6_rows(bool fixed, int cap);
 cudaError_t launch_psi6(const LaunchCfg& c, CellBufs cells, double2* local, unsigned long long* total, int* err);
 cudaError_t launch_psi6_reduce(const LaunchCfg& c, unsigned long long* total, double* res);
 // Append (beta P / rho, g(2 sigma+), Re Psi_6, Im Psi_6) of every replica to

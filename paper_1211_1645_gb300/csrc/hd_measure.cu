@@ -26,7 +26,7 @@ constexpr int kMaxFitBins = 512;
 // One thread per cell scans the (2R+1)^2 stencil; counts gather in a shared
 // histogram and are flushed with one atomic per non-empty bin and block.
 // k_hist_global reads the stencil from global memory (any reach R);
-// k_hist_tile (reach up to kHistMaxHalo) first stages the block's 32 x 8
+// k_hist_tile (reach up to kHistMaxHalo) first stages the block's
 // tile of cells and a halo of R cells in shared memory, like k_psi6.
 // ---------------------------------------------------------------------------
 template <bool FIX, int CAP>
@@ -130,11 +130,16 @@ __device__ __forceinline__ int tile_disk_list(const uint8_t* s_n, int SX, int ha
     return total;
 }
 
-constexpr int kTileThreads = 256;  // a 32 x 8 tile of cells, one thread per cell
+// A tile of 32 x 8 cells, one thread per cell; 32 x 4 in the FP64 form where cells
+// hold up to nine disks: about two each, so that an SM's FP64 work is that of its
+// few blocks (psi_6, one call at cells of 2.9 sigma: N = 16,384 165 us with eight
+// rows, 149 with four; N = 2^20 1186 and 1279; the fixed form 99 and 99, 332 and 396).
+template <bool FIX, int CAP>
+constexpr int kTileThreads = FIX || CAP == 4 ? 256 : 128;
 
 template <bool FIX, int CAP>
 __host__ __device__ constexpr size_t hist_stage_bytes(int halo, int K) {
-    return size_t(32 + 2 * halo) * size_t(kTileThreads / 32 + 2 * halo) *
+    return size_t(32 + 2 * halo) * size_t(kTileThreads<FIX, CAP> / 32 + 2 * halo) *
                (CAP * (sizeof(P2<FIX>) + (FIX ? 0 : sizeof(float2) + sizeof(int32_t))) + 1) +
            16 + size_t(K + 1) * 8 + size_t(K) * 4;
 }
@@ -168,7 +173,7 @@ __device__ __forceinline__ int hist_bin_fp64(const double2& o, const double2& me
 // arithmetic once per such pair with one lane in it (57% of the FP64 pipe).
 // N = 2^20: FP64 133 -> 78 us; the fixed form 52, with the queue 59.
 template <bool FIX, int CAP>
-__global__ void __launch_bounds__(kTileThreads)
+__global__ void __launch_bounds__(kTileThreads<FIX, CAP>)
 k_hist_tile(const Rep* __restrict__ reps, int R, int K, const double* __restrict__ edges,
             const long long* __restrict__ edgesF, const uint8_t* __restrict__ cnt, const P2<FIX>* __restrict__ pos,
             const int32_t* __restrict__ pid, unsigned long long* __restrict__ hist, int H) {
@@ -177,7 +182,7 @@ k_hist_tile(const Rep* __restrict__ reps, int R, int K, const double* __restrict
     const int r = find_rep<kGridT32>(reps, R, blockIdx.x);
     const Rep& rep = reps[r];
     const int m = rep.m;
-    constexpr int rows = kTileThreads / 32;
+    constexpr int rows = kTileThreads<FIX, CAP> / 32;
     int X0, Y0;
     tile32_origin(rep, uint32_t(blockIdx.x - rep.blk_t32), rows, X0, Y0);
     const int SX = 32 + 2 * H, nS = SX * (rows + 2 * H);
@@ -189,12 +194,12 @@ k_hist_tile(const Rep* __restrict__ reps, int R, int K, const double* __restrict
     using E = std::conditional_t<FIX, long long, double>;
     E* s_edge = reinterpret_cast<E*>(s_raw + ((size_t(CAP) * nS * (sizeof(P2<FIX>) + (FIX ? 0 : sizeof(float2) + 4)) + nS + 15) & ~size_t(15)));
     unsigned int* s_bins = reinterpret_cast<unsigned int*>(s_edge + (K + 1));
-    for (int b = threadIdx.x; b <= K; b += kTileThreads) {
+    for (int b = threadIdx.x; b <= K; b += kTileThreads<FIX, CAP>) {
         if constexpr (FIX) s_edge[b] = edgesF[b];
         else s_edge[b] = edges[b];
         if (b < K) s_bins[b] = 0u;
     }
-    for (int t = threadIdx.x; t < nS; t += kTileThreads) {
+    for (int t = threadIdx.x; t < nS; t += kTileThreads<FIX, CAP>) {
         const int sy = t / SX, sx = t - sy * SX;
         const uint32_t c = uint32_t(rep.coff) + row_part(rep, wrap_cell(Y0 - H + sy, m)) +
                            col_part(rep, wrap_cell(X0 - H + sx, m));
@@ -211,13 +216,13 @@ k_hist_tile(const Rep* __restrict__ reps, int R, int K, const double* __restrict
         if (!FIX && n == 0) s_img[t] = make_float2(__uint_as_float(0x7F800000u), 0.0f);  // slot 0 is tested in any case
     }
     __syncthreads();
-    __shared__ uint16_t s_list[kTileThreads * CAP];
+    __shared__ uint16_t s_list[kTileThreads<FIX, CAP> * CAP];
     __shared__ int s_warp[8];
     const int D = tile_disk_list(s_n, SX, H, X0, Y0, m, s_list, s_warp);
     const int RR = rep.hist_R;
     if constexpr (FIX) {
         const long long lo_edge = s_edge[0], hi_edge = s_edge[K];
-        for (int d = threadIdx.x; d < D; d += kTileThreads) {
+        for (int d = threadIdx.x; d < D; d += kTileThreads<FIX, CAP>) {
             const int own = int(s_list[d] >> 4), k = int(s_list[d] & 15u);
             const int2 me = s_pos[k * nS + own];
             for (int dcy = 0; dcy <= RR; ++dcy) {
@@ -241,7 +246,7 @@ k_hist_tile(const Rep* __restrict__ reps, int R, int K, const double* __restrict
             }
         }
     } else {
-        __shared__ uint32_t s_queue[kTileThreads / 32][64];  // own entry | other entry << 16
+        __shared__ uint32_t s_queue[kTileThreads<FIX, CAP> / 32][64];  // own entry | other entry << 16
         const int lane = int(threadIdx.x & 31u), warp = int(threadIdx.x >> 5);
         uint32_t* queue = s_queue[warp];
         int queued = 0;  // the same in every lane
@@ -257,7 +262,7 @@ k_hist_tile(const Rep* __restrict__ reps, int R, int K, const double* __restrict
                 if (bin >= 0) atomicAdd(&s_bins[bin], 1u);
             }
         };
-        for (int base = warp * 32; base < D; base += kTileThreads) {
+        for (int base = warp * 32; base < D; base += kTileThreads<FIX, CAP>) {
             const int d = base + lane;
             const bool live = d < D;
             const int own = live ? int(s_list[d] >> 4) : 0, k = live ? int(s_list[d] & 15u) : 0;
@@ -299,7 +304,7 @@ k_hist_tile(const Rep* __restrict__ reps, int R, int K, const double* __restrict
         bin_queued(queued);
     }
     __syncthreads();
-    for (int b = threadIdx.x; b < K; b += kTileThreads)
+    for (int b = threadIdx.x; b < K; b += kTileThreads<FIX, CAP>)
         if (s_bins[b]) atomicAdd(&hist[size_t(r) * K + b], (unsigned long long)s_bins[b]);
 }
 
@@ -504,7 +509,6 @@ __device__ __forceinline__ bool ring_covers(const Rep& rep, const Nbr<FIX>& nb, 
 // cells plus a halo of two cells (the 5 x 5 stencil of every tile cell).
 constexpr int kPsiHalo = 2;
 constexpr int kPsiSX = 32 + 2 * kPsiHalo;
-constexpr int kPsiThreads = kTileThreads;  // eight rows: 1.7 staged cells per cell
 
 template <bool FIX, int CAP>
 __host__ __device__ constexpr size_t psi6_stage_bytes(int rows) {
@@ -523,16 +527,17 @@ struct PsiStage {
 
 // The general search of a disk's six nearest: ordered insertion of every
 // candidate by (r^2, id) from the staged rings 0, 1, 2, then rings in global
-// memory until the sixth is certified.  Out of line: the float search below
-// leaves it about one disk in a thousand where cells hold up to four disks; wider
-// cells all come here.  In the FP64 form a candidate whose float estimate of
+// memory until the sixth is certified.  Where cells hold up to four disks the
+// float search below leaves it about one disk in a thousand, so it is called out
+// of line (nearest_general); the disks of wider cells all take it, in line (FP64,
+// N = 16,384 at cells of 2.9 sigma, one call with eight rows of cells per block: out of line 183 us, in line 165).  In the FP64 form a candidate whose float estimate of
 // r^2 exceeds the sixth key by more than the estimate's error bound is farther
 // in FP64 too and is left out before its FP64 arithmetic.
 template <bool FIX, int CAP>
-static __device__ __noinline__ bool nearest_general(const Rep& rep, const PsiStage<FIX>& st, const uint8_t* cnt,
-                                                    const P2<FIX>* pos, const int32_t* pid, int own, int cx, int cy,
-                                                    P2<FIX> me, int32_t idme, int rmax, typename Nbr<FIX>::Off* ox,
-                                                    typename Nbr<FIX>::Off* oy) {
+__device__ __forceinline__ bool nearest_inserted(const Rep& rep, const PsiStage<FIX>& st, const uint8_t* cnt,
+                                                 const P2<FIX>* pos, const int32_t* pid, int own, int cx, int cy,
+                                                 const P2<FIX>& me, int32_t idme, int rmax,
+                                                 typename Nbr<FIX>::Off (&ox)[6], typename Nbr<FIX>::Off (&oy)[6]) {
     Nbr<FIX> nb;
     nb.n = 0;
     bool ok = false;
@@ -590,6 +595,21 @@ static __device__ __noinline__ bool nearest_general(const Rep& rep, const PsiSta
     for (int q = 0; q < 6; ++q) {
         ox[q] = nb.rx[q];
         oy[q] = nb.ry[q];
+    }
+    return ok;
+}
+
+template <bool FIX, int CAP>
+static __device__ __noinline__ bool nearest_general(const Rep& rep, const PsiStage<FIX>& st, const uint8_t* cnt,
+                                                    const P2<FIX>* pos, const int32_t* pid, int own, int cx, int cy,
+                                                    P2<FIX> me, int32_t idme, int rmax, typename Nbr<FIX>::Off* ox,
+                                                    typename Nbr<FIX>::Off* oy) {
+    typename Nbr<FIX>::Off x[6], y[6];
+    const bool ok = nearest_inserted<FIX, CAP>(rep, st, cnt, pos, pid, own, cx, cy, me, idme, rmax, x, y);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+        ox[q] = x[q];
+        oy[q] = y[q];
     }
     return ok;
 }
@@ -713,7 +733,7 @@ constexpr int kPsiWords = 16;
 // = 2^20, 58 -> 47 at 262,144.  The FP64 form is bound by the FP64 pipe (84%
 // busy, mostly the fourteen correctly rounded divisions per disk): 952 -> 668.
 template <bool FIX, int CAP>
-__global__ void __launch_bounds__(kPsiThreads, FIX ? 4 : 2)
+__global__ void __launch_bounds__(kTileThreads<FIX, CAP>, (FIX ? 1024 : 512) / kTileThreads<FIX, CAP>)
 k_psi6(const Rep* __restrict__ reps, int R, const uint8_t* __restrict__ cnt, const P2<FIX>* __restrict__ pos,
        const int32_t* __restrict__ pid, double2* __restrict__ local, unsigned long long* __restrict__ total,
        int* __restrict__ err) {
@@ -722,7 +742,7 @@ k_psi6(const Rep* __restrict__ reps, int R, const uint8_t* __restrict__ cnt, con
     const int r = find_rep<kGridT32>(reps, R, blockIdx.x);
     const Rep& rep = reps[r];
     const int m = rep.m;
-    constexpr int rows = kPsiThreads / 32;
+    constexpr int rows = kTileThreads<FIX, CAP> / 32;
     int X0, Y0;
     tile32_origin(rep, uint32_t(blockIdx.x - rep.blk_t32), rows, X0, Y0);
     constexpr int nS = kPsiSX * (rows + 2 * kPsiHalo);
@@ -730,7 +750,7 @@ k_psi6(const Rep* __restrict__ reps, int R, const uint8_t* __restrict__ cnt, con
     float2* s_img = reinterpret_cast<float2*>(s_pos + size_t(CAP) * nS);   // [2][nS]
     int32_t* s_id = reinterpret_cast<int32_t*>(s_img + size_t(2) * nS);    // [CAP][nS]
     uint8_t* s_n = reinterpret_cast<uint8_t*>(s_id + size_t(CAP) * nS);    // [nS]
-    for (int t = threadIdx.x; t < nS; t += kPsiThreads) {
+    for (int t = threadIdx.x; t < nS; t += kTileThreads<FIX, CAP>) {
         const int sy = t / kPsiSX, sx = t - sy * kPsiSX;
         const uint32_t c = uint32_t(rep.coff) + row_part(rep, wrap_cell(Y0 - kPsiHalo + sy, m)) +
                            col_part(rep, wrap_cell(X0 - kPsiHalo + sx, m));
@@ -752,7 +772,7 @@ k_psi6(const Rep* __restrict__ reps, int R, const uint8_t* __restrict__ cnt, con
     }
     __syncthreads();
 
-    __shared__ uint16_t s_list[kPsiThreads * CAP];
+    __shared__ uint16_t s_list[kTileThreads<FIX, CAP> * CAP];
     __shared__ int s_warp[8];
     const int D = tile_disk_list(s_n, kPsiSX, kPsiHalo, X0, Y0, m, s_list, s_warp);
     const PsiStage<FIX> st{s_img, s_pos, s_id, s_n, nS};
@@ -762,23 +782,27 @@ k_psi6(const Rep* __restrict__ reps, int R, const uint8_t* __restrict__ cnt, con
         const int lim = int((int64_t(1) << 31) / rep.W) - 1;
         if (lim < rmax) rmax = lim;
     }
-    for (int d = threadIdx.x; d < D; d += kPsiThreads) {
+    for (int d = threadIdx.x; d < D; d += kTileThreads<FIX, CAP>) {
         const int own = int(s_list[d] >> 4), k = int(s_list[d] & 15u);
         const P2<FIX> me = s_pos[k * nS + own];
         const int32_t idme = s_id[k * nS + own];
         typename Nbr<FIX>::Off rx[6], ry[6];
         bool ok = false;
-        if (CAP == 4 && rmax >= 2) ok = nearest_float<FIX, CAP>(rep, st, own, k, me, rx, ry);
-        if (!ok) {
-            const int sy = own / kPsiSX;
-            const int cx = X0 + (own - sy * kPsiSX) - kPsiHalo, cy = Y0 + sy - kPsiHalo;
-            typename Nbr<FIX>::Off gx[6], gy[6];
-            ok = nearest_general<FIX, CAP>(rep, st, cnt, pos, pid, own, cx, cy, me, idme, rmax, gx, gy);
+        const int sy = own / kPsiSX;
+        const int cx = X0 + (own - sy * kPsiSX) - kPsiHalo, cy = Y0 + sy - kPsiHalo;
+        if constexpr (CAP == 4) {
+            if (rmax >= 2) ok = nearest_float<FIX, CAP>(rep, st, own, k, me, rx, ry);
+            if (!ok) {
+                typename Nbr<FIX>::Off gx[6], gy[6];
+                ok = nearest_general<FIX, CAP>(rep, st, cnt, pos, pid, own, cx, cy, me, idme, rmax, gx, gy);
 #pragma unroll
-            for (int q = 0; q < 6; ++q) {
-                rx[q] = gx[q];
-                ry[q] = gy[q];
+                for (int q = 0; q < 6; ++q) {
+                    rx[q] = gx[q];
+                    ry[q] = gy[q];
+                }
             }
+        } else {
+            ok = nearest_inserted<FIX, CAP>(rep, st, cnt, pos, pid, own, cx, cy, me, idme, rmax, rx, ry);
         }
         double pre, pim;
         if (!ok) {
@@ -878,7 +902,7 @@ static cudaError_t hist_t(const LaunchCfg& c, const HistCfg& h, CellBufs cells, 
         static OncePerDevice once;
         const cudaError_t e = allow_smem(once, hist_stage_bytes<FIX, CAP>(kHistMaxHalo, kMaxFitBins), k_hist_tile<FIX, CAP>);
         if (e != cudaSuccess) return e;
-        return launch_k(k_hist_tile<FIX, CAP>, dim3(c.blocks_t32), dim3(kTileThreads),
+        return launch_k(k_hist_tile<FIX, CAP>, dim3(c.blocks_t32), dim3(kTileThreads<FIX, CAP>),
                         hist_stage_bytes<FIX, CAP>(h.halo, h.K), c.stream, c.reps, c.R, h.K, h.edges,
                         h.edgesF, (const uint8_t*)cells.cnt, (const P2<FIX>*)cells.pos, (const int32_t*)cells.pid,
                         hist, h.halo);
@@ -907,15 +931,15 @@ cudaError_t launch_fit(const LaunchCfg& c, int K, const double* qr, const unsign
 }
 
 size_t psi6_total_words(int R) { return size_t(R) * kPsiWords; }
-int psi6_rows() { return kPsiThreads / 32; }
+int psi6_rows(bool fixed, int cap) { return (fixed || cap == 4 ? kTileThreads<true, 4> : kTileThreads<false, 9>) / 32; }
 
 template <bool FIX, int CAP>
 static cudaError_t psi6_t(const LaunchCfg& c, CellBufs cells, double2* local, unsigned long long* total, int* err) {
-    constexpr size_t smem = psi6_stage_bytes<FIX, CAP>(kPsiThreads / 32);
+    constexpr size_t smem = psi6_stage_bytes<FIX, CAP>(kTileThreads<FIX, CAP> / 32);
     static OncePerDevice once;
     const cudaError_t e = allow_smem(once, smem, k_psi6<FIX, CAP>);
     if (e != cudaSuccess) return e;
-    return launch_k(k_psi6<FIX, CAP>, dim3(c.blocks_t32), dim3(kPsiThreads), smem, c.stream, c.reps, c.R,
+    return launch_k(k_psi6<FIX, CAP>, dim3(c.blocks_t32), dim3(kTileThreads<FIX, CAP>), smem, c.stream, c.reps, c.R,
                     (const uint8_t*)cells.cnt, (const P2<FIX>*)cells.pos, (const int32_t*)cells.pid, local, total,
                     err);
 }

@@ -8,7 +8,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("form", ["fixed", "fp64"])
-@pytest.mark.parametrize("N, eta, cell_min", [(256, 0.70, 2.9), (1024, 0.5, 3.3), (3000, 0.71, 4.2)])
+@pytest.mark.parametrize("N, eta, cell_min", [(256, 0.70, 2.9), (1024, 0.5, 3.3), (3000, 0.71, 3.9)])
 @pytest.mark.parametrize("noise", [0.0, 2.0 ** -24, 1e-5, None])
 def test_wide_cells_match_the_oracle(oracle_mod, form, N, eta, cell_min, noise):
     import paper_1211_1645_gb300 as hd
