@@ -45,6 +45,7 @@ constexpr int kMaxTiledReplicas = 1024;       // replicas of a context on the ti
 constexpr int kBranchedReplicas = 16;         // see plan_tiles
 constexpr double kCrowdedTiles = 9e5;         // disks times disks per cell of a crowded context on the tile or box sweep
 constexpr double kCrowdedTiles64 = 7e5;       // ... FP64 form
+constexpr int64_t kSqPairDisks = 128;  // disks per replica from which wave vectors are looked over for shared components
 constexpr int64_t kTileCells64 = 640 * 1024;  // cells of an FP64 context up to which the tile sweep is the faster
 
 struct Plan {
@@ -1857,16 +1858,19 @@ hd_status grow(hd_ctx* ctx, T*& p, size_t& cap, size_t need) {
     return HD_OK;
 }
 
+// Whether a call takes nq wave vectors: the bound on the partial sums of one
+// plane wave per wave vector and disk, also where fewer are made.
+bool sq_accepted(const std::vector<int64_t>& N, int nq) {
+    return N.size() * size_t(hd::sq_disk_blocks(N)) * size_t(nq) <= (size_t(1) << 27);
+}
+
 // S at the wave vectors already in ctx->sq_hk ([R][nq]), or with nh > 0 of the
 // components and pairs already in ctx->sq_comp and ctx->sq_pair; positions
 // refreshed first.
 hd_status enqueue_sq(hd_ctx* ctx, int nq, int nh, int nk, bool grid, bool want_best) {
     std::vector<int64_t> Ns;
     for (const Rep& r : ctx->reps) Ns.push_back(r.N);
-    // (the bound on the partial sums of one plane wave per wave vector and
-    // disk, which decides what the call accepts)
-    const size_t bound = size_t(ctx->R) * size_t(hd::sq_disk_blocks(Ns)) * size_t(nq);
-    if (bound > (size_t(1) << 27)) return HD_ERR_ARG;
+    if (!sq_accepted(Ns, nq)) return HD_ERR_ARG;
     const int nbx = nh > 0 ? hd::sq_pair_blocks(ctx->R, nq, Ns) : hd::sq_disk_blocks(Ns);
     hd_status st = grow(ctx, ctx->sq_part, ctx->sq_part_cap, size_t(ctx->R) * size_t(nbx) * size_t(grid ? std::max(nq, nh * nk) : nq));
     if (st != HD_OK) return st;
@@ -1886,45 +1890,92 @@ hd_status enqueue_sq(hd_ctx* ctx, int nq, int nh, int nk, bool grid, bool want_b
     return HD_OK;
 }
 
+// The distinct values among one component of a list of wave vectors, in order of
+// appearance: an open-addressing table of a few hundred places (lists of more
+// distinct values than sq_pairs_fit takes are given up early).
+class Distinct {
+    static constexpr uint32_t kPlaces = 512;
+    int value_[kPlaces];
+    int16_t entry_[kPlaces];  // -1: free
+
+public:
+    std::vector<int> values;
+    void clear() {
+        std::fill(entry_, entry_ + kPlaces, int16_t(-1));
+        values.clear();
+    }
+    // entry of v, entered if new; -1 when the table is three quarters full
+    int enter(int v) {
+        for (uint32_t p = (uint32_t(v) * 2654435769u) >> 23;; p = (p + 1u) % kPlaces) {
+            if (entry_[p] < 0) {
+                if (values.size() >= kPlaces * 3 / 4) return -1;
+                value_[p] = v;
+                entry_[p] = int16_t(values.size());
+                values.push_back(v);
+                return entry_[p];
+            }
+            if (value_[p] == v) return entry_[p];
+        }
+    }
+};
+
 // The distinct components of each replica's wave vectors, padded to the
 // largest count, and each wave vector's indices; false where the lists share
-// too few of them.
+// too few of them, or the replicas are so small that looking costs more than
+// a plane wave per wave vector and disk.
 // grid: every replica's are nh and nk consecutive integers.
-bool sq_components(int R, int nq, const int32_t* hk, int& nh, int& nk, bool& grid, std::vector<int>& comp,
-                   std::vector<ushort2>& pair) {
-    std::vector<std::vector<int>> h(static_cast<size_t>(R)), k(static_cast<size_t>(R));
+bool sq_components(const std::vector<int64_t>& N, int nq, const int32_t* hk, int& nh, int& nk, bool& grid,
+                   std::vector<int>& comp, std::vector<ushort2>& pair) {
+    const int R = int(N.size());
+    int64_t disks = 0;
+    for (int64_t n : N) disks += n;
+    if (disks < kSqPairDisks * R) return false;
     nh = nk = 1;
+    pair.resize(size_t(R) * size_t(nq));
+    std::vector<std::vector<int>> list[2];
+    list[0].resize(size_t(R));
+    list[1].resize(size_t(R));
+    grid = true;
+    Distinct seen[2];
     for (int r = 0; r < R; ++r) {
-        for (int c = 0; c < 2; ++c) {
-            std::vector<int>& v = c == 0 ? h[size_t(r)] : k[size_t(r)];
-            v.resize(size_t(nq));
-            for (int q = 0; q < nq; ++q) v[size_t(q)] = hk[2 * (size_t(r) * nq + size_t(q)) + size_t(c)];
-            std::sort(v.begin(), v.end());
-            v.erase(std::unique(v.begin(), v.end()), v.end());
+        seen[0].clear();
+        seen[1].clear();
+        const int32_t* v = hk + 2 * size_t(r) * size_t(nq);
+        ushort2* to = pair.data() + size_t(r) * size_t(nq);
+        for (int q = 0; q < nq; ++q) {
+            const int h = seen[0].enter(v[2 * q]), k = seen[1].enter(v[2 * q + 1]);
+            if (h < 0 || k < 0) return false;
+            if (h >= nh || k >= nk) {  // more than any replica before
+                nh = std::max(nh, h + 1);
+                nk = std::max(nk, k + 1);
+                if (!hd::sq_pairs_fit(nh, nk, nq)) return false;
+            }
+            to[q].x = (unsigned short)h;
+            to[q].y = (unsigned short)k;
         }
-        nh = std::max(nh, int(h[size_t(r)].size()));
-        nk = std::max(nk, int(k[size_t(r)].size()));
-        if (!hd::sq_pairs_fit(nh, nk, nq)) return false;
+        // entries in order of appearance to indices in ascending order
+        std::vector<unsigned short> rank[2];
+        for (int c = 0; c < 2; ++c) {
+            std::vector<int>& sorted = list[c][size_t(r)];
+            sorted = seen[c].values;
+            std::sort(sorted.begin(), sorted.end());
+            for (int x : seen[c].values)
+                rank[c].push_back((unsigned short)(std::lower_bound(sorted.begin(), sorted.end(), x) - sorted.begin()));
+        }
+        for (int q = 0; q < nq; ++q) {
+            to[q].x = rank[0][to[q].x];
+            to[q].y = rank[1][to[q].y];
+        }
     }
     grid = hd::sq_grid_fit(nh, nk, nq);
-    for (int r = 0; r < R; ++r) {
-        auto run = [](const std::vector<int>& v, int n) {
-            return int(v.size()) == n && int64_t(v.back()) - int64_t(v.front()) == int64_t(n) - 1;
-        };
-        grid = grid && run(h[size_t(r)], nh) && run(k[size_t(r)], nk);
-    }
     comp.assign(size_t(R) * size_t(nh + nk), 0);
-    pair.resize(size_t(R) * size_t(nq));
-    for (int r = 0; r < R; ++r) {
-        const std::vector<int>&hr = h[size_t(r)], &kr = k[size_t(r)];
-        std::copy(hr.begin(), hr.end(), comp.begin() + size_t(r) * size_t(nh + nk));
-        std::copy(kr.begin(), kr.end(), comp.begin() + size_t(r) * size_t(nh + nk) + size_t(nh));
-        for (int q = 0; q < nq; ++q) {
-            const size_t at = size_t(r) * nq + size_t(q);
-            pair[at].x = (unsigned short)(std::lower_bound(hr.begin(), hr.end(), hk[2 * at]) - hr.begin());
-            pair[at].y = (unsigned short)(std::lower_bound(kr.begin(), kr.end(), hk[2 * at + 1]) - kr.begin());
+    for (int r = 0; r < R; ++r)
+        for (int c = 0; c < 2; ++c) {
+            const std::vector<int>& v = list[c][size_t(r)];
+            grid = grid && int(v.size()) == (c == 0 ? nh : nk) &&
+                   int64_t(v.back()) - int64_t(v.front()) == int64_t(v.size()) - 1;
+            std::copy(v.begin(), v.end(), comp.begin() + std::ptrdiff_t(r) * (nh + nk) + (c == 0 ? 0 : nh));
         }
-    }
     return true;
 }
 
@@ -1934,12 +1985,19 @@ hd_status hd_structure_factor(hd_ctx* ctx, int32_t nq, const int32_t* hk, double
     const Range range("hd_structure_factor");
     if (!ctx || !hk || !S || nq < 1 || nq > 65536) return HD_ERR_ARG;
     if (ctx->sticky != HD_OK) return HD_ERR_STATE;
+    std::vector<int64_t> Ns;
+    for (const Rep& r : ctx->reps) Ns.push_back(r.N);
+    if (!sq_accepted(Ns, nq)) return HD_ERR_ARG;
     int nh = 0, nk = 0;
-    bool grid = false;
+    bool grid = false, shared = false;
     std::vector<int> comp;
     std::vector<ushort2> pair;
+    try {
+        shared = sq_components(Ns, nq, hk, nh, nk, grid, comp, pair);
+    } catch (const std::bad_alloc&) {  // no host memory for the indices: one plane wave per wave vector and disk
+    }
     hd_status st;
-    if (sq_components(ctx->R, nq, hk, nh, nk, grid, comp, pair)) {
+    if (shared) {
         st = grow(ctx, ctx->sq_comp, ctx->sq_comp_cap, comp.size());
         if (st == HD_OK) st = grow(ctx, ctx->sq_pair, ctx->sq_pair_cap, pair.size());
         if (st != HD_OK) return st;
