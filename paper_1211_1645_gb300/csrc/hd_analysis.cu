@@ -28,7 +28,7 @@ constexpr int kAcfLags = 128, kAcfChunk = 128;
 
 __global__ void __launch_bounds__(kAcfLags)
 k_acf_sums(const double* __restrict__ series, int R, int64_t T, int64_t max_lag, int64_t len, double2* __restrict__ part) {
-    pdl_begin();
+    pdl_begin(series);
     __shared__ double2 s_a[kAcfChunk], s_c[kAcfChunk + kAcfLags];
     const int r = blockIdx.y;
     const int64_t d0 = int64_t(blockIdx.x) * kAcfLags, d = d0 + threadIdx.x;
@@ -65,7 +65,7 @@ k_acf_sums(const double* __restrict__ series, int R, int64_t T, int64_t max_lag,
 // in order; blockIdx.y = replica.  Every block adds up S(0) itself.
 __global__ void __launch_bounds__(128)
 k_acf_norm(int R, int64_t T, int64_t max_lag, int chunks, const double2* __restrict__ part, double2* __restrict__ C) {
-    pdl_begin();
+    pdl_begin(part);
     __shared__ double s_zero[128];
     const int r = blockIdx.y;
     const size_t row = size_t(max_lag + 1), step = size_t(R) * row;
@@ -104,7 +104,7 @@ __device__ __forceinline__ double lane_sum(double v) {
 // (NaN with fewer than two such lags or a slope >= 0).  One warp per replica.
 __global__ void __launch_bounds__(32)
 k_acf_tau(int64_t max_lag, int64_t lag_lo, int64_t lag_hi, const double2* __restrict__ C, double* __restrict__ tau) {
-    pdl_begin();
+    pdl_begin(C);
     const double2* row = C + size_t(blockIdx.x) * size_t(max_lag + 1);
     const int lane = int(threadIdx.x);
     double sx = 0.0, sy = 0.0, cnt = 0.0;
@@ -142,7 +142,7 @@ k_acf_tau(int64_t max_lag, int64_t lag_lo, int64_t lag_hi, const double2* __rest
 __global__ void __launch_bounds__(256)
 k_field_accum(const Rep* __restrict__ reps, int R, int64_t Ntot, bool fixed, int bins, const double* __restrict__ xy,
               const double2* __restrict__ psi, double* __restrict__ acc) {
-    pdl_begin();
+    pdl_begin(xy, psi);
     const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= Ntot) return;
     int lo = 0, hi = R - 1;  // replica of global id i: last one with id_off <= i
@@ -174,7 +174,7 @@ k_field_accum(const Rep* __restrict__ reps, int R, int64_t Ntot, bool fixed, int
 // Coarse field, means: out[r][iy][ix] = (sum Re, sum Im) / count, NaN if empty.
 __global__ void __launch_bounds__(256)
 k_field_norm(int64_t cells, const double* __restrict__ acc, double2* __restrict__ out) {
-    pdl_begin();
+    pdl_begin(acc);
     const int64_t c = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (c >= cells) return;
     const double n = acc[3 * c + 2];
@@ -222,7 +222,7 @@ constexpr int kSqChunk = 16;  // wave vectors per block of the amplitude kernel
 __global__ void __launch_bounds__(256)
 k_sq_amp(const Rep* __restrict__ reps, bool fixed, int nq, const int2* __restrict__ hk, const double* __restrict__ xy,
          int nbx, double2* __restrict__ part) {
-    pdl_begin();
+    pdl_begin(hk, xy);
     const int r = blockIdx.z;
     const Rep& rep = reps[r];
     const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
@@ -339,7 +339,7 @@ __device__ __forceinline__ double2 turn_wave(const Turn& t, int h, const double2
 __global__ void __launch_bounds__(kPairThreads)
 k_sq_pairs(const Rep* __restrict__ reps, bool fixed, int nq, int nh, int nk, const int* __restrict__ comp,
            const ushort2* __restrict__ pair, const double* __restrict__ xy, double2* __restrict__ part) {
-    pdl_begin();
+    pdl_begin(comp, pair, xy);
     extern __shared__ double2 s_wave[];  // [kPairDisks][nh + nk], then the table
     __shared__ Turn s_turn[kPairDisks][2];
     const int r = blockIdx.z, nc = nh + nk, tid = int(threadIdx.x);
@@ -428,7 +428,7 @@ k_sq_pairs(const Rep* __restrict__ reps, bool fixed, int nq, int nh, int nk, con
 __global__ void __launch_bounds__(kPairThreads)
 k_sq_grid(const Rep* __restrict__ reps, bool fixed, int nh, int nk, const int* __restrict__ comp,
           const double* __restrict__ xy, double2* __restrict__ part) {
-    pdl_begin();
+    pdl_begin(comp, xy);
     extern __shared__ double2 s_wave[];  // [kPairDisks][nk + 1 + J], then the table
     __shared__ Turn s_turn[kPairDisks][2];
     const int r = blockIdx.z, tid = int(threadIdx.x);
@@ -536,7 +536,7 @@ k_sq_grid(const Rep* __restrict__ reps, bool fixed, int nh, int nk, const int* _
 __global__ void __launch_bounds__(256)
 k_sq_sum(const Rep* __restrict__ reps, int nq, int nbx, bool by_disks, const double2* __restrict__ part, int row_len, int nk,
          const ushort2* __restrict__ pair, double* __restrict__ S) {
-    pdl_begin();
+    pdl_begin(part, pair);
     __shared__ double2 s_v[8][32];
     const int r = blockIdx.y, lane = int(threadIdx.x & 31u), row = int(threadIdx.x >> 5);
     const int q = blockIdx.x * 32 + lane;
@@ -570,7 +570,7 @@ k_sq_sum(const Rep* __restrict__ reps, int nq, int nbx, bool by_disks, const dou
 // best[r] = first q of largest S_r(q).  One block per replica.
 __global__ void __launch_bounds__(256)
 k_sq_best(int nq, const double* __restrict__ S, int* __restrict__ best) {
-    pdl_begin();
+    pdl_begin(S);
     const int r = blockIdx.x;
     __shared__ double s_v[256];
     __shared__ int s_i[256];
@@ -608,7 +608,7 @@ k_sq_best(int nq, const double* __restrict__ S, int* __restrict__ best) {
 __global__ void __launch_bounds__(128)
 k_q0_window(const Rep* __restrict__ reps, int hw, const double* __restrict__ psi, int2* __restrict__ hk,
             int* __restrict__ comp, ushort2* __restrict__ pair) {
-    pdl_begin();
+    pdl_begin(psi);
     const int r = blockIdx.x;
     const Rep& rep = reps[r];
     const double L = rep.Lm;
@@ -634,7 +634,7 @@ k_q0_window(const Rep* __restrict__ reps, int hw, const double* __restrict__ psi
 __global__ void __launch_bounds__(256)
 k_chi(const Rep* __restrict__ reps, int R, int64_t Ntot, bool fixed, const int2* __restrict__ hk0,
       const double* __restrict__ xy, double2* __restrict__ chi) {
-    pdl_begin();
+    pdl_begin(hk0, xy);
     const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= Ntot) return;
     const int r = rep_of_id(reps, R, i);
@@ -656,7 +656,7 @@ k_poscorr(const Rep* __restrict__ reps, int R, const uint8_t* __restrict__ cnt, 
           const double* __restrict__ xy, const double2* __restrict__ chi, int nr, double dr, int reach,
           double* __restrict__ acc) {
     extern __shared__ double s_acc[];  // [nr][3]
-    pdl_begin();
+    pdl_begin(cnt, pid, xy, chi);
     for (int k = threadIdx.x; k < 3 * nr; k += blockDim.x) s_acc[k] = 0.0;
     __syncthreads();
     const int r = find_rep<kGridCell>(reps, R, blockIdx.x);
@@ -745,7 +745,7 @@ __global__ void __launch_bounds__(256)
 k_corr_stage(const Rep* __restrict__ reps, const Frame* __restrict__ cur, const uint8_t* __restrict__ cnt,
              const P2<FIX>* __restrict__ pos, const int2* __restrict__ hk0, double2* __restrict__ gpos,
              double2* __restrict__ chi, float2* __restrict__ off) {
-    pdl_begin();
+    pdl_begin(cur, cnt, pos, hk0);
     const int r = blockIdx.y;
     const Rep& rep = reps[r];
     const int m = rep.m;
@@ -810,7 +810,7 @@ k_corr_pairs(const Rep* __restrict__ reps, const uint8_t* __restrict__ cnt, cons
     uint32_t* s_cnt = reinterpret_cast<uint32_t*>(s_sum + size_t(bins) * NT);
     __shared__ uint16_t s_list[NT * CAP];
     __shared__ int s_n;
-    pdl_begin();
+    pdl_begin(cnt, gpos, chi, off);
     const int r = blockIdx.y, tid = int(threadIdx.x);
     const Rep& rep = reps[r];
     const int m = rep.m;
@@ -930,7 +930,7 @@ k_corr_pairs(const Rep* __restrict__ reps, const uint8_t* __restrict__ cnt, cons
 __global__ void __launch_bounds__(128)
 k_corr_windows(int nr, double dr, const double2* __restrict__ acc, double2* __restrict__ out) {
     extern __shared__ double2 s_acc2[];  // [2 nr + 1] sums, then [2 nr] bounds
-    pdl_begin();
+    pdl_begin(acc);
     const int r = blockIdx.y, bins = 2 * nr + 1, k = int(blockIdx.x * blockDim.x + threadIdx.x);
     double* lo2 = reinterpret_cast<double*>(s_acc2 + bins);
     double* hi2 = lo2 + nr;
@@ -967,7 +967,7 @@ k_corr_windows(int nr, double dr, const double2* __restrict__ acc, double2* __re
 
 __global__ void __launch_bounds__(256)
 k_corr_norm(int64_t n, const double* __restrict__ acc, double2* __restrict__ out) {
-    pdl_begin();
+    pdl_begin(acc);
     const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const double c = acc[3 * i + 2];

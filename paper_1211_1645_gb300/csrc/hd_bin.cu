@@ -74,7 +74,7 @@ template <bool FIX, int CAP>
 __global__ void __launch_bounds__(256)
 k_bin(const Rep* __restrict__ reps, int R, int64_t Ntot, double sigma, const double* __restrict__ xy,
       uint8_t* __restrict__ cnt, P2<FIX>* __restrict__ pos, int32_t* __restrict__ pid, int* __restrict__ err) {
-    pdl_begin();
+    pdl_begin(xy, cnt);
     const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
     if (i >= Ntot) return;
     int lo = 0, hi = R - 1;  // replica of global id i: last one with id_off <= i

@@ -21,15 +21,39 @@ using P2 = std::conditional_t<FIX, int2, double2>;
 // disk at liquid densities); higher slots only when the cell is that full.
 constexpr int kEagerSlots = 2;
 
-// Loads of cell data.  COH = false: through the read-only data path, valid
-// while no block of the launch writes the cells it reads (one launch per
-// rebuild and per colour pass).  COH = true: coherent loads cached in L2 only
-// (ld.global.cg), for a launch whose blocks read cells that other blocks
-// wrote earlier in the same launch, ordered by acquire / release flags.
+// Loads of cell data.  COH = false: ordinary loads, where no other block of the
+// launch writes the cells it reads (one launch per rebuild and per colour pass);
+// not read-only ones, and kept after the wait of pdl_begin by their order, since
+// the launch before may still be writing when this one's blocks start.  (N = 2^20,
+// FP64 colour pass 16.0 us so, 17.0 through pointers given to the wait; the fixed
+// rebuild 15.0 and 16.4, and 14.4 when its loads were free to come before it.)
+// COH = true: coherent loads cached in L2 only (ld.global.cg), for a launch whose
+// blocks read cells that other blocks wrote earlier in the same launch, ordered
+// by acquire / release flags.
+__device__ __forceinline__ uint8_t ld_in_order(const uint8_t* p) {
+    uint32_t v;
+    asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return uint8_t(v);
+}
+__device__ __forceinline__ int32_t ld_in_order(const int32_t* p) {
+    int32_t v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ int2 ld_in_order(const int2* p) {
+    int2 v;
+    asm volatile("ld.global.v2.s32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ double2 ld_in_order(const double2* p) {
+    double2 v;
+    asm volatile("ld.global.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p) : "memory");
+    return v;
+}
 template <bool COH, class T>
 __device__ __forceinline__ T ld_cell(const T* p) {
     if constexpr (COH) return __ldcg(p);
-    else return __ldg(p);
+    else return ld_in_order(p);
 }
 
 // One cell as loaded by a thread: occupancy and the first kEagerSlots slots

@@ -92,9 +92,28 @@ __device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, u
 // scheduled once every block of this one has started, and wait until the
 // previous kernel has completed and its memory is visible.  Both are no-ops
 // when the launch did not opt in.
-__device__ __forceinline__ void pdl_begin() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+// The pointers through which a kernel reads what earlier kernels write are given
+// to the wait and come back as new values: a load through a __restrict__
+// parameter, and a read-only (non-coherent) load anyway, may otherwise be moved
+// before the wait, which no statement about other memory holds back.  (Seen as
+// passes that took the draw table of the launch before, in step graphs of one
+// sweep, whose six kernels are launched close enough together.)  For the same
+// reason such data is not read with __ldg.
+template <class T>
+__device__ __forceinline__ void after_wait(T& pointer) {
+    size_t at = __cvta_generic_to_global(pointer);  // (as a global address, so that the loads stay global ones)
+    asm volatile("" : "+l"(at) : : "memory");
+    pointer = static_cast<T>(__cvta_global_to_generic(at));
+}
+template <class... P>
+__device__ __forceinline__ void pdl_wait(P&... pointers) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    (after_wait(pointers), ...);
+}
+template <class... P>
+__device__ __forceinline__ void pdl_begin(P&... pointers) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_wait(pointers...);
 }
 
 // A float within a relative 2^-20 of x (|x| < 2^128), from the high word of

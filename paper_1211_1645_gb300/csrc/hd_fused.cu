@@ -77,7 +77,7 @@ k_sweep_fused(const Rep* __restrict__ reps, int R, const Frame* __restrict__ tab
     uint8_t* s_cnt = smem + F::kPosBytes + F::kPidBytes;                                // [NC]
     uint16_t* s_list = reinterpret_cast<uint16_t*>(s_cnt + F::kCntBytes);              // [2][H*H]
     __shared__ int s_len[2];
-    pdl_begin();
+    pdl_begin(table, cnt_o, pos_o, pid_o);
 
     const int r = find_rep<kGridTile>(reps, R, blockIdx.x);
     const Rep rep = reps[r];

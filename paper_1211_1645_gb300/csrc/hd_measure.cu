@@ -35,7 +35,7 @@ k_hist_global(const Rep* __restrict__ reps, int R, int K, const double* __restri
        const long long* __restrict__ edgesF, const uint8_t* __restrict__ cnt, const P2<FIX>* __restrict__ pos,
        const int32_t* __restrict__ pid, unsigned long long* __restrict__ hist) {
     extern __shared__ unsigned int s_bins[];
-    pdl_begin();
+    pdl_begin(cnt, pos, pid);
     for (int b = threadIdx.x; b < K; b += blockDim.x) s_bins[b] = 0u;
     __syncthreads();
     const int r = find_rep<kGridCell>(reps, R, blockIdx.x);
@@ -178,7 +178,7 @@ k_hist_tile(const Rep* __restrict__ reps, int R, int K, const double* __restrict
             const long long* __restrict__ edgesF, const uint8_t* __restrict__ cnt, const P2<FIX>* __restrict__ pos,
             const int32_t* __restrict__ pid, unsigned long long* __restrict__ hist, int H) {
     extern __shared__ __align__(16) unsigned char s_raw[];
-    pdl_begin();
+    pdl_begin(cnt, pos, pid);
     const int r = find_rep<kGridT32>(reps, R, blockIdx.x);
     const Rep& rep = reps[r];
     const int m = rep.m;
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(32) k_fit_factor(int K, double* __restrict__ w
 
 __global__ void __launch_bounds__(32) k_fit(const Rep* __restrict__ reps, int K, const double* __restrict__ weight,
                                             const unsigned long long* __restrict__ hist, double* __restrict__ res) {
-    pdl_begin();
+    pdl_begin(hist);
     const int r = blockIdx.x, lane = threadIdx.x;
     const Rep& rep = reps[r];
     const double PI = 3.14159265358979323846;
@@ -738,7 +738,7 @@ k_psi6(const Rep* __restrict__ reps, int R, const uint8_t* __restrict__ cnt, con
        const int32_t* __restrict__ pid, double2* __restrict__ local, unsigned long long* __restrict__ total,
        int* __restrict__ err) {
     extern __shared__ __align__(16) unsigned char s_raw[];
-    pdl_begin();
+    pdl_begin(cnt, pos, pid);
     const int r = find_rep<kGridT32>(reps, R, blockIdx.x);
     const Rep& rep = reps[r];
     const int m = rep.m;
@@ -869,7 +869,7 @@ k_psi6(const Rep* __restrict__ reps, int R, const uint8_t* __restrict__ cnt, con
 // N (the oracle's order of operations).  One block of one warp per replica.
 __global__ void __launch_bounds__(32)
 k_psi6_reduce(const Rep* __restrict__ reps, unsigned long long* __restrict__ total, double* __restrict__ res) {
-    pdl_begin();
+    pdl_begin(total);
     const int r = blockIdx.x, lane = int(threadIdx.x);
     unsigned long long* w = total + size_t(r) * kPsiWords;
     __shared__ unsigned long long s_w[kPsiWords];
@@ -951,7 +951,7 @@ cudaError_t launch_psi6(const LaunchCfg& c, CellBufs cells, double2* local, unsi
 
 __global__ void k_record(int R, const double* __restrict__ fit, const double* __restrict__ psi,
                          double* __restrict__ series, int64_t* __restrict__ len, int64_t cap, int* __restrict__ err) {
-    pdl_begin();
+    pdl_begin(fit, psi, len);
     const int64_t idx = *len;
     const int r = threadIdx.x;
     if (r < R && idx < cap) {

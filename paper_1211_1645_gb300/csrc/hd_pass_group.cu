@@ -52,7 +52,7 @@ k_pass_group(const Rep* __restrict__ reps, const uint16_t* __restrict__ rep_of, 
              int32_t* pid, unsigned long long* __restrict__ counters) {
     static_assert(G == 2 || G == 4 || G == 8, "a group is 2, 4 or 8 lanes of one warp");
     constexpr int NQ = 8 / G;  // neighbours per lane
-    pdl_begin();
+    pdl_begin(table, cnt, pos, pid);
     extern __shared__ __align__(16) unsigned char s_raw[];
     int2* s_nbr = reinterpret_cast<int2*>(s_raw);
     P2<FIX>* s_crowd = reinterpret_cast<P2<FIX>*>(
@@ -110,7 +110,7 @@ k_pass_group(const Rep* __restrict__ reps, const uint16_t* __restrict__ rep_of, 
                         ok &= pair_clear<FIX>(mine[2 * k], ox, oy, np, rep) | (ni < 1);
                         ok &= pair_clear<FIX>(mine[2 * k + 1], ox, oy, np, rep) | (ni < 2);
                         for (int s2 = kEagerSlots; s2 < ni; ++s2)
-                            ok &= pair_clear<FIX>(__ldg(pos + size_t(s2) * rep.stride32 + nbr_cell(i)), ox, oy, np,
+                            ok &= pair_clear<FIX>(pos[size_t(s2) * rep.stride32 + nbr_cell(i)], ox, oy, np,
                                                   rep);
                     }
                 } else {

@@ -59,7 +59,7 @@ k_pass_tma(const Rep* __restrict__ reps, int R, const Frame* __restrict__ table,
     __shared__ int s_poff[kSegs], s_coff[kSegs];  // staged index of half-column hc: hc + off
     __shared__ uint32_t s_base[kSegs];             // first cell index of each segment's row
 
-    pdl_begin();
+    pdl_begin(table, cnt, pos, pid);
     const int r = find_rep<kGridSeg>(reps, R, blockIdx.x);
     const Rep rep = reps[r];
     const int hm = rep.hm;
@@ -162,7 +162,7 @@ k_pass_tma(const Rep* __restrict__ reps, int R, const Frame* __restrict__ table,
             const int k = nbr_seg(i), hc = nbr_hc(i);
             int nn;
             if (!edge || (hc >= 0 && hc < hm)) nn = s_n[k * cc + hc + coff[k]];
-            else nn = __ldg(cnt + sbase[k] + uint32_t(hc < 0 ? hc + hm : hc - hm));
+            else nn = cnt[sbase[k] + uint32_t(hc < 0 ? hc + hm : hc - hm)];
             nocc |= uint32_t(min(nn, CAP)) << (4 * q);
         }
         if (n > 0) {
@@ -200,8 +200,8 @@ k_pass_tma(const Rep* __restrict__ reps, int R, const Frame* __restrict__ table,
                         c = s_p1[k * pc + lp];
                     } else {  // periodic wrap at a row end
                         const uint32_t ci = sbase[k] + uint32_t(hc < 0 ? hc + hm : hc - hm);
-                        a = __ldg(pos + ci);
-                        c = __ldg(pos + size_t(rep.stride32) + ci);
+                        a = pos[ci];
+                        c = pos[size_t(rep.stride32) + ci];
                     }
                     ok &= pair_clear<FIX>(a, dx, dy, np, rep) | (nn < 1);
                     ok &= pair_clear<FIX>(c, dx, dy, np, rep) | (nn < 2);
@@ -216,7 +216,7 @@ k_pass_tma(const Rep* __restrict__ reps, int R, const Frame* __restrict__ table,
                         const int nn = int(nocc >> (4 * q)) & 0xF;
                         const uint32_t ci = sbase[k] + uint32_t(hc < 0 ? hc + hm : (hc >= hm ? hc - hm : hc));
                         for (int s2 = kEagerSlots; s2 < nn; ++s2)
-                            ok &= pair_clear<FIX>(__ldg(pos + size_t(s2) * rep.stride32 + ci), i % 3 - 1, i / 3 - 1, np,
+                            ok &= pair_clear<FIX>(pos[size_t(s2) * rep.stride32 + ci], i % 3 - 1, i / 3 - 1, np,
                                                   rep);
                     }
                 }

@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(256, 4)
 k_sweep_persist(const Rep* __restrict__ reps, int R, const Rep rep1, const Frame* __restrict__ table, int nsweeps,
                 uint32_t NI, CellBufs g0, CellBufs g1, unsigned long long* __restrict__ counters,
                 int* __restrict__ err, uint32_t* sync, uint32_t polls, int stall_band) {
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait(table);
     extern __shared__ __align__(16) unsigned char s_raw[];
     P2<FIX>* s_crowd = reinterpret_cast<P2<FIX>*>(s_raw + size_t(blockDim.x) * nbr_bytes_per_thread<FIX>());
     int32_t* s_crowd_id = reinterpret_cast<int32_t*>(s_crowd + size_t(blockDim.x) * CAP);

@@ -23,7 +23,7 @@ namespace hd {
 
 __global__ void k_draws(const Rep* __restrict__ reps, int R, Frame* __restrict__ table,
                         Frame* __restrict__ cur, uint64_t* __restrict__ sweep_ctr, int nchunk) {
-    pdl_begin();
+    pdl_begin(table, cur, sweep_ctr);
     // one block per replica, one thread per sweep of the chunk: every sweep's
     // draws come from its own generator block
     const int r = blockIdx.x;
@@ -92,7 +92,7 @@ k_rebuild(const Rep* __restrict__ reps, const uint16_t* __restrict__ rep_of, con
           uint8_t* __restrict__ cnt_o, const P2<FIX>* __restrict__ pos_o, const int32_t* __restrict__ pid_o,
           uint8_t* __restrict__ cnt_n, P2<FIX>* __restrict__ pos_n, int32_t* __restrict__ pid_n,
           int* __restrict__ err) {
-    pdl_begin();
+    pdl_begin(table);
     const int r = ONE ? 0 : int(rep_of[blockIdx.x]);
     const Rep rep = ONE ? rep1 : reps[r];
     uint32_t a[2];
@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(256)
 k_pass(const Rep* __restrict__ reps, const uint16_t* __restrict__ rep_of, const Rep rep1,
        const Frame* __restrict__ table, int j, int p, uint32_t a_lo, uint32_t a_hi,
        const uint8_t* __restrict__ cnt, P2<FIX>* pos, int32_t* pid, unsigned long long* __restrict__ counters) {
-    pdl_begin();
+    pdl_begin(table);
     extern __shared__ __align__(16) unsigned char s_raw[];
     P2<FIX>* s_crowd = reinterpret_cast<P2<FIX>*>(s_raw + size_t(blockDim.x) * nbr_bytes_per_thread<FIX>());
     int32_t* s_crowd_id = reinterpret_cast<int32_t*>(s_crowd + size_t(blockDim.x) * CAP);
@@ -162,7 +162,7 @@ template <bool FIX, int CAP>
 __global__ void __launch_bounds__(256)
 k_positions(const Rep* __restrict__ reps, int R, const Frame* __restrict__ cur, const uint8_t* __restrict__ cnt,
             const P2<FIX>* __restrict__ pos, const int32_t* __restrict__ pid, double* __restrict__ xy) {
-    pdl_begin();
+    pdl_begin(cur, cnt, pos, pid);
     const int r = find_rep<kGridCell>(reps, R, blockIdx.x);
     const Rep rep = reps[r];
     const int m = rep.m;

@@ -284,7 +284,7 @@ k_sweep_tile(const Rep* __restrict__ reps, const TileGrid* __restrict__ grids, i
     using Sh = TileShape<FIX>;
     using S = TileStage<FIX>;
     constexpr int NT = Sh::NT - 32;  // threads that sweep; the last warp looks ahead
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait(table);
     extern __shared__ __align__(16) unsigned char s_raw[];
     const S st(s_raw, static_cast<PoolEntry<FIX>*>(spill) + size_t(blockIdx.x) * 2 * S::NC);
     __shared__ TileItem s_item[2];
@@ -537,7 +537,7 @@ __global__ void __launch_bounds__(NT + ND)
 k_sweep_box(const Rep* __restrict__ reps, const Frame* __restrict__ table, int nsweeps, CellBufs g0, CellBufs g1,
             unsigned long long* __restrict__ counters, int* __restrict__ err, void* spill) {
     using S = BoxStage<FIX, HB>;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    pdl_wait(table);
     extern __shared__ __align__(16) unsigned char s_raw[];
     PoolEntry<FIX>* far = static_cast<PoolEntry<FIX>*>(spill) + size_t(blockIdx.x) * 4 * S::NC;
     const int tid = int(threadIdx.x), r = int(blockIdx.x);
