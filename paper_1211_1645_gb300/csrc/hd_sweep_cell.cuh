@@ -276,8 +276,13 @@ __device__ __forceinline__ void pass_cell(const Rep& rep, const Frame& f, int co
                     const int oy = int((0x2A540u >> (2 * i)) & 3u) - 1;  // i / 3 - 1
                     const int ni = int(nocc >> (4 * q)) & 0xF;
                     const uint32_t ci = rep.coff + row_part(rep, wrap_cell(cy + oy, m)) + col_part(rep, wrap_cell(cx + ox, m));
-                    for (int k = 1; k < ni && ok; ++k)
-                        ok = pair_clear<FIX>(ld_cell<COH>(pos + size_t(k) * rep.stride32 + ci), ox, oy, np, rep);
+                    for (int k = 1; k < ni && ok; ++k) {
+                        // (ordered after the wait by its address, which follows from the
+                        // sweep's frame, so not kept in the order of the other loads: crowded
+                        // batches, 304 of N = 2000 at cells of 2.5 sigma, 43.6 -> 32.7 us)
+                        const P2<FIX>* o = pos + size_t(k) * rep.stride32 + ci;
+                        ok = pair_clear<FIX>(COH ? ld_cell<COH>(o) : *o, ox, oy, np, rep);
+                    }
                 }
             }
             return ok;
