@@ -110,7 +110,9 @@ typedef struct hd_opts {
                                 launch, of a box that fits one block's shared
                                 memory or of tiles of cells staged there (FP64: up
                                 to 655,360 cells; fewer where cells hold more than
-                                a disk on average); else strips, 16 when the colour
+                                a disk on average), in calls for which that is the
+                                faster: not in steps of one sweep or two of most
+                                fixed-form systems; else strips, 16 when the colour
                                 pass is 1.5 to 3.5 waves of resident blocks deep, 8
                                 when it is deeper, none when it is shallower;
                                 1: none; 2 .. 64: K strips (at most m / 2, and
@@ -123,9 +125,10 @@ typedef struct hd_opts {
                                 concurrently (independent chains, Sec. IV.A's
                                 scan); the measurement stays one batched launch.
                                 Same chains.  0: the library chooses (the one-launch
-                                sweeps as for strips 0, up to 1024 replicas; else
-                                branches where they apply); 1: one batched launch
-                                per phase [0]                                   */
+                                sweeps as for strips 0, up to 1024 replicas, in calls
+                                whose boxes or tiles the GPU takes in a few rounds;
+                                else branches where they apply, up to 64 replicas);
+                                1: one batched launch per phase [0]             */
 } hd_opts;
 
 /* The one-launch sweeps of strips = 0 and replica_branches = 0 wait for
@@ -142,7 +145,8 @@ typedef struct hd_geometry {
     int32_t hist_bins;  /* K of the contact histogram                             */
     int32_t graph_branches; /* concurrent branches of the sweeps of hd_run's step
                                graphs: the strips of a one-replica context, the
-                               replicas of a batch with replica branches, else 1 */
+                               replicas of a batch with replica branches, else 1
+                               (also where longer steps are one launch)          */
     double L;           /* box side in sigma (fixed form: m * W * 2^-24)          */
     double w;           /* cell side in sigma                                     */
     double delta;       /* maximum displacement per axis in sigma (realised)      */

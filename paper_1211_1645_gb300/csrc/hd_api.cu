@@ -16,6 +16,7 @@
 #include "hd_analysis.h"
 #include "hd_bin.h"
 #include "hd_bounds.h"
+#include "hd_route.h"
 #include "hd_tile.h"
 
 using hd::CellBufs;
@@ -45,6 +46,7 @@ constexpr int kMaxTiledReplicas = 1024;       // replicas of a context on the ti
 constexpr int kBranchedReplicas = 16;         // see plan_tiles
 constexpr double kCrowdedTiles = 9e5;         // disks times disks per cell of a crowded context on the tile or box sweep
 constexpr double kCrowdedTiles64 = 7e5;       // ... FP64 form
+constexpr double kCrowdedBatch = 4e5;         // ... of a batch on the tile sweep
 constexpr int64_t kSqPairDisks = 128;  // disks per replica from which wave vectors are looked over for shared components
 constexpr int64_t kTileCells64 = 640 * 1024;  // cells of an FP64 context up to which the tile sweep is the faster
 
@@ -74,6 +76,8 @@ struct hd_ctx {
     // the tile sweep (hd_tile.cu): the sweeps of contexts whose options leave
     // the order of the launches to the library
     bool tiled = false;
+    hd::SweepShape shape{};            // what decides it call by call (hd_route.h)
+    bool other_clear = true;           // the occupancy of the generation not current is zero, as the split rebuild needs it
     std::vector<hd::TileGrid> tiles;   // [R]
     hd::TileCfg tile_cfg{};
     int box_hm = 0;                    // the largest half-side, when box_spill is set
@@ -148,6 +152,7 @@ struct hd_ctx {
         int parity;
         bool local;     // the measurement keeps the psi_6 field
         bool profiled;
+        bool one;       // its sweeps are one-launch sweeps
         cudaGraphExec_t exec;
         int64_t launches[HD_KERNEL_CLASSES];
         size_t ev0;
@@ -706,6 +711,22 @@ cudaError_t enqueue_strips(hd_ctx* ctx, cudaStream_t s, int nc) {
     return e;
 }
 
+// Whether n sweeps of a call of hd_sweep, or of a step being captured, run as
+// one launch per draw table (not in a profiled step, which times the phases).
+bool one_launch(const hd_ctx* ctx, int64_t n, bool step) {
+    return ctx->tiled && !(step && ctx->profiling) && n > 0 && hd::one_launch_pays(ctx->shape, n, step);
+}
+
+// Before and after sweeps of either order are enqueued on the context stream
+// (a captured step: before and after its launch): the split rebuild expects the
+// other generation's occupancy cleared and leaves it so, the one-launch sweeps
+// leave it as it was a sweep ago.
+cudaError_t before_sweeps(hd_ctx* ctx, bool one) {
+    if (one || ctx->other_clear) return cudaSuccess;
+    return cudaMemsetAsync(ctx->buf[ctx->cur ^ 1].cnt, 0, size_t(ctx->Ctot) + kCellPad, ctx->stream);
+}
+void after_sweeps(hd_ctx* ctx, bool one) { ctx->other_clear = !one; }
+
 // Enqueue n sweeps on stream s (draw tables of up to kMaxChunk sweeps, then
 // the table's sweeps in one tile-sweep or persistent launch, or per sweep
 // either one fused launch or a rebuild and four colour passes).
@@ -715,7 +736,7 @@ cudaError_t enqueue_strips(hd_ctx* ctx, cudaStream_t s, int nc) {
 // as one branch per replica.
 cudaError_t enqueue_sweeps(hd_ctx* ctx, cudaStream_t s, int64_t n, bool capturing) {
     const hd::LaunchCfg c = ctx->cfg(s);
-    if (ctx->tiled && !ctx->prof_capture) {
+    if (one_launch(ctx, n, capturing)) {
         cudaError_t e = cudaSuccess;
         for (int64_t left = n; left > 0 && e == cudaSuccess;) {
             const int nc = int(std::min<int64_t>(left, hd::kMaxChunk));
@@ -733,10 +754,6 @@ cudaError_t enqueue_sweeps(hd_ctx* ctx, cudaStream_t s, int64_t n, bool capturin
             left -= nc;
         }
         return e;
-    }
-    if (ctx->tiled && n > 0) {  // a profiled step: the split kernels, whose rebuild expects the other generation cleared
-        const cudaError_t e = cudaMemsetAsync(ctx->buf[ctx->cur ^ 1].cnt, 0, size_t(ctx->Ctot) + kCellPad, s);
-        if (e != cudaSuccess) return e;
     }
     const bool wave = capturing && !ctx->prof_capture && (ctx->strips > 1 || ctx->branches);
     if (wave) {
@@ -1119,7 +1136,7 @@ hd_status hd_batch_init(hd_ctx** out, int32_t R, const int64_t* N, const double*
             ok = dev_alloc(ctx, &spill, size_t(R) * hd::box_spill(ctx->fixed, hm));
             ctx->box_spill = spill;
             ctx->tiled = true;
-        } else if (ok && plan_tiles(ctx, sms)) {
+        } else if (ok && !(R > 1 && ctx->Ntot > ctx->Ctot && crowd > kCrowdedBatch) && plan_tiles(ctx, sms)) {
             hd::TileCfg& t = ctx->tile_cfg;
             hd::TileGrid* grids = nullptr;
             ok = hd::tile_blocks(ctx->cfg(), &t.blocks) == cudaSuccess;
@@ -1140,12 +1157,21 @@ hd_status hd_batch_init(hd_ctx** out, int32_t R, const int64_t* N, const double*
                 ctx->tiled = true;
             }
         }
-        if (ctx->tiled) ctx->strips = 1;
+        hd::SweepShape& s = ctx->shape;
+        s.box = ctx->box_spill != nullptr;
+        s.fixed = ctx->fixed;
+        s.crowded = ctx->Ntot > ctx->Ctot;
+        s.R = R;
+        s.hm = hm;
+        s.rounds = s.box ? double((R + sms - 1) / std::max(1, sms)) : double(ctx->tile_cfg.total) / std::max(1, sms);
+        s.tile = s.box ? 0.0 : double(ctx->Ctot) / double(std::max<int64_t>(1, ctx->tile_cfg.total));
+        s.replica = double(ctx->Ctot) / R;
     }
     // the branches' streams and events exist before any step is captured
     // (one side stream at least: the measurement's psi_6 branch)
-    ok = ok && ensure_side(ctx, std::max(1, ctx->strips > 1 ? ctx->strips : (ctx->branches && !ctx->tiled ? R : 1)),
-                           ctx->strips > 1) == cudaSuccess;
+    // (those of a context on the one-launch sweeps when a step first needs them)
+    ok = ok && ensure_side(ctx, ctx->tiled ? 1 : std::max(1, ctx->strips > 1 ? ctx->strips : (ctx->branches ? R : 1)),
+                           !ctx->tiled && ctx->strips > 1) == cudaSuccess;
     if (!ok) {
         free_ctx(ctx);
         return HD_ERR_CUDA;
@@ -1243,7 +1269,10 @@ hd_status hd_sweep(hd_ctx* ctx, int64_t n) {
     const Range range("hd_sweep");
     if (!ctx || n < 0) return HD_ERR_ARG;
     if (ctx->sticky != HD_OK) return HD_ERR_STATE;
+    const bool one = one_launch(ctx, n, false);
+    if (n > 0) HD_CK(ctx, before_sweeps(ctx, one));
     HD_CK(ctx, enqueue_sweeps(ctx, ctx->stream, n, false));
+    if (n > 0) after_sweeps(ctx, one);
     for (auto& s : ctx->sweeps) s += n;
     return HD_OK;
 }
@@ -1338,12 +1367,14 @@ hd_status hd_set_positions(hd_ctx* ctx, const double* xy) {
     const int bad = flag & (hd::kErrBinOverflow | hd::kErrBinInput);
     if (bad) {
         HD_CK(ctx, cudaMemsetAsync(to.cnt, 0, cnt_bytes, ctx->stream));  // the rebuild expects it cleared
+        ctx->other_clear = true;
         const int keep = flag & ~bad;
         HD_CK(ctx, cudaMemcpyAsync(ctx->err, &keep, sizeof(int), cudaMemcpyHostToDevice, ctx->stream));
         HD_CK(ctx, cudaStreamSynchronize(ctx->stream));
         return (bad & hd::kErrBinInput) ? HD_ERR_ARG : HD_ERR_OVERFLOW;
     }
     ctx->cur ^= 1;
+    ctx->other_clear = true;
     // the generation left behind must be cleared for the next rebuild; the
     // frame is unshifted (stream-ordered before any later work: no wait)
     HD_CK(ctx, cudaMemsetAsync(ctx->buf[ctx->cur ^ 1].cnt, 0, cnt_bytes, ctx->stream));
@@ -1374,7 +1405,8 @@ hd_status hd_get_geometry(hd_ctx* ctx, int32_t r, hd_geometry* g) {
     g->trials_per_cell = rep.nt;
     g->precision = ctx->fixed ? HD_FIXED32 : HD_FP64;
     g->hist_bins = ctx->K;
-    g->graph_branches = ctx->strips > 1 ? ctx->strips : (ctx->branches ? ctx->R : 1);
+    // (a one-replica context on the one-launch sweeps has strips only in steps too short for those)
+    g->graph_branches = ctx->tiled && ctx->R == 1 ? 1 : ctx->strips > 1 ? ctx->strips : (ctx->branches ? ctx->R : 1);
     g->L = ctx->fixed ? double(rep.LF) / kFx : rep.L;
     g->w = ctx->fixed ? double(rep.W) / kFx : rep.w;
     g->delta = ctx->fixed ? double(rep.D) / kFx : rep.delta;
@@ -1433,6 +1465,10 @@ hd_status hd_run(hd_ctx* ctx, int64_t steps, int32_t sweeps_per_step, int32_t me
             ng.local = local;
             ng.parity = parity;
             ng.profiled = prof;
+            ng.one = one_launch(ctx, sweeps_per_step, true);
+            if (ctx->tiled && !ng.one && !prof)  // the branches' streams and events exist before the capture
+                HD_CK(ctx, ensure_side(ctx, std::max(1, ctx->strips > 1 ? ctx->strips : (ctx->branches ? ctx->R : 1)),
+                                       ctx->strips > 1));
             ng.ev0 = ctx->gev_used;
             if (prof) {  // two events per launch: draws, 5 per sweep, the measurement
                 const size_t bound = 2 * (size_t(sweeps_per_step) * 5 + size_t(sweeps_per_step) / hd::kMaxChunk + 16);
@@ -1471,7 +1507,9 @@ hd_status hd_run(hd_ctx* ctx, int64_t steps, int32_t sweeps_per_step, int32_t me
             ctx->graphs.push_back(std::move(ng));
             g = &ctx->graphs.back();
         }
+        if (sweeps_per_step > 0) HD_CK(ctx, before_sweeps(ctx, g->one));
         HD_CK(ctx, cudaGraphLaunch(g->exec, ctx->stream));
+        if (sweeps_per_step > 0) after_sweeps(ctx, g->one);
         for (int c = 0; c < HD_KERNEL_CLASSES; ++c) ctx->launches[c] += g->launches[c];
         if (sweeps_per_step & 1) ctx->cur ^= 1;
         if (prof) {  // read this replay's kernel times before the next one
@@ -1714,6 +1752,7 @@ hd_status hd_restore(hd_ctx* ctx, const void* buf, size_t bytes) {
     p += slots * sizeof(int32_t);
     // the other generation's occupancy must be zero for the next scatter rebuild
     HD_CK(ctx, cudaMemset(ctx->buf[ctx->cur ^ 1].cnt, 0, size_t(ctx->Ctot) + kCellPad));
+    ctx->other_clear = true;
     HD_CK(ctx, cudaMemcpy(ctx->frame, p, sizeof(Frame) * size_t(ctx->R), cudaMemcpyHostToDevice));
     p += sizeof(Frame) * size_t(ctx->R);
     HD_CK(ctx, cudaMemcpy(ctx->sweep_ctr, p, sizeof(uint64_t) * size_t(ctx->R), cudaMemcpyHostToDevice));

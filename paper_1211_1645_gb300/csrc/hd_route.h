@@ -32,10 +32,11 @@ struct SweepShape {
 // 1000 of N = 1000 2058 and 1835.  A call of hd_sweep makes a launch per phase from
 // the host (31 us per sweep at least): 1000 of N = 1000 1352 and 1183.  One sweep:
 // 304 of N = 100 45 and 37, 500 49 and 51 (N = 1000 56 and 65).  Crowded, fixed, N = 400
-// at cells of 2.5 sigma, 12 sweeps: 304 480 and 402, 608 549 and 783.
+// at cells of 2.5 sigma, 12 sweeps: 304 480 and 402, 608 549 and 783 (from hd_sweep 518 and
+// 399, 628 and 773).
 inline bool one_launch_boxes(const SweepShape& s, int64_t n, bool step) {
     double most = 1e9;
-    if (s.crowded) most = 2;
+    if (s.crowded) most = step || n < 3 ? 2 : 3;
     else if (n == 1) most = s.fixed || step ? 2 : 3;
     else if (n == 2) most = step ? 3 : (s.fixed ? 4 : 5);
     else if (step) most = s.fixed ? 4 : (s.hm < 13 ? 5 : 7);
