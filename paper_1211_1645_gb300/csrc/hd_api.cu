@@ -78,6 +78,7 @@ struct hd_ctx {
     bool tiled = false;
     hd::SweepShape shape{};            // what decides it call by call (hd_route.h)
     bool other_clear = true;           // the occupancy of the generation not current is zero, as the split rebuild needs it
+    bool replayed = false;             // calls were captured by the caller, whose replays this does not see
     std::vector<hd::TileGrid> tiles;   // [R]
     hd::TileCfg tile_cfg{};
     int box_hm = 0;                    // the largest half-side, when box_spill is set
@@ -721,8 +722,16 @@ bool one_launch(const hd_ctx* ctx, int64_t n, bool step) {
 // (a captured step: before and after its launch): the split rebuild expects the
 // other generation's occupancy cleared and leaves it so, the one-launch sweeps
 // leave it as it was a sweep ago.
+// Sweeps that the caller captures may run at any time after, so from then on it is
+// cleared before every split rebuild.
 cudaError_t before_sweeps(hd_ctx* ctx, bool one) {
-    if (one || ctx->other_clear) return cudaSuccess;
+    if (ctx->tiled && !ctx->replayed) {
+        cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+        const cudaError_t e = cudaStreamIsCapturing(ctx->stream, &status);
+        if (e != cudaSuccess) return e;
+        ctx->replayed = status != cudaStreamCaptureStatusNone;
+    }
+    if (one || (ctx->other_clear && !ctx->replayed)) return cudaSuccess;
     return cudaMemsetAsync(ctx->buf[ctx->cur ^ 1].cnt, 0, size_t(ctx->Ctot) + kCellPad, ctx->stream);
 }
 void after_sweeps(hd_ctx* ctx, bool one) { ctx->other_clear = !one; }
