@@ -254,9 +254,10 @@ def time_form(args, form, rank, world, steps, warmup, sampler=None, N=None, eta=
             sysg.sweep(S)
         sw = sysg.kernel_times()
         sysg.profile(False)
-        kt = {k: v for k, v in kt.items() if k not in ("rebuild", "pass") and v[1]}
-        kt["draws"] = sw["draws"]
-        kt["sweep"] = (sw["sweep"][0], S * PROFILED_STEPS)
+        if sw["sweep"][1]:
+            kt = {k: v for k, v in kt.items() if k not in ("rebuild", "pass") and v[1]}
+            kt["draws"] = sw["draws"]
+            kt["sweep"] = (sw["sweep"][0], S * PROFILED_STEPS)
     geo = sysg.geometry()
     series = sysg.series()
     final_xy = sysg.positions() if keep_positions else None

@@ -43,7 +43,7 @@ constexpr int kAutoStrips = 16;   // strips chosen when the colour pass is 1.5 t
 constexpr int kAutoStripsDeep = 8;  // ... and when it is deeper
 constexpr int kMaxBranches = 64;  // replicas on concurrent branches of a captured step
 constexpr int kMaxTiledReplicas = 1024;       // replicas of a context on the tile or box sweep (bounds its scratch)
-constexpr int kBranchedReplicas = 16;         // see plan_tiles
+constexpr int kBranchedReplicas = 16;         // largest batch measured for the rule in plan_tiles
 constexpr double kCrowdedTiles = 9e5;         // disks times disks per cell of a crowded context on the tile or box sweep
 constexpr double kCrowdedTiles64 = 7e5;       // ... FP64 form
 constexpr double kCrowdedBatch = 4e5;         // ... of a batch on the tile sweep
@@ -261,10 +261,12 @@ void set_hist_f32_bounds(Rep& r, double e0, double eK) {
 // and with shares: two of N = 16,384 17.9 -> 8.1, eight 18.4 -> 10.9, three of
 // 65,536 22.5 -> 11.9; FP64 22.7 -> 11.5, 22.9 -> 16.5, 22.9 -> 18.3).
 bool plan_tiles(hd_ctx* ctx, int sms) {
-    // The FP64 form stages twice the bytes per cell in tiles half as large, and
-    // its frame changes are FP64-bound: per sweep 30.5 us against 42.9 as graph
-    // branches at N = 524,288, 46.5 against ~48 at 786,432, 62 against 54 at
-    // 1,048,576.
+    // The FP64 form stages twice the bytes per cell in tiles half as large.  Per
+    // sweep, tiles and strips of the step graph: 30.5 us and 42.9 at N = 524,288
+    // (575,000 cells), 46.5 and about 48 at 786,432 (862,000), 62 and 54 at 1,048,576
+    // (1,150,000): the line is drawn where the tiles are clearly ahead.  What
+    // bounds them is not the FP64 pipe (30% busy at 524,288) but the barriers
+    // between a tile's phases (41% of issue slots used).
     if (!ctx->fixed && ctx->Ctot > kTileCells64) return false;
     const hd::TileLimits lim = hd::tile_limits(ctx->fixed);
     int64_t fewest = 0, total = 0;

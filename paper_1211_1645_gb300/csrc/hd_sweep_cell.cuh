@@ -241,8 +241,8 @@ __device__ __forceinline__ void pass_cell(const Rep& rep, const Frame& f, int co
                 // Neighbours holding more than kEagerSlots disks (rare): a
                 // nibble n >= 3 is the one whose n + 5 sets its bit 3.
                 // Only those neighbours are visited (bit 4q + 3 of the mask):
-                // nearly every warp has a lane with one, but a lane rarely
-                // has more than one.
+                // a lane rarely has more than one, and at cells of 2.001 sigma one
+                // lane in 4e4 has any.
                 for (uint32_t cm = (nocc + 0x55555555u) & 0x88888888u; cm != 0u; cm &= cm - 1u) {
                     const int q = (__ffs(int(cm)) - 1) >> 2;
                     const int i = q + (q >= 4 ? 1 : 0);

@@ -49,8 +49,9 @@ __device__ __forceinline__ void red_release_add(uint32_t* p, uint32_t v) {
 
 // Staging capacity and launch shape of one form: one block per SM with as large
 // a staged region as its shared memory holds, since the cells around a tile
-// are worked on twice (fixed form: 104 x 68 cells, tiles of up to 96 x 60, 1.18
-// staged cells per owned one).  Measured at N = 2^20, fixed form, us per sweep:
+// are worked on twice (fixed form: 104 x 68 cells, tiles of up to 96 x 60; over the
+// 24 colour orders, the 12 x 18 tiles of N = 2^20 load 1.14 cells and update 1.06 for
+// each they own).  Measured at N = 2^20, fixed form, us per sweep:
 // 768 threads at 80 registers 29.0, 640 31.3, 992 at 64 registers 32.0 (spills);
 // two blocks of 384 threads and half the region each 29.7, three of 256 39.7.
 template <bool FIX>
@@ -393,9 +394,10 @@ k_sweep_tile(const Rep* __restrict__ reps, const TileGrid* __restrict__ grids, i
                 if (uint32_t(lx - lo0x) < nx0 && uint32_t(ly - lo0y) < ny0)
                     over |= !st.place(lx, ly, S::index(lx, ly), p, id);
             };
-            // Slot 0 of every old cell first; a cell of more disks (about one
-            // in eight) is queued, and the warp takes its further slots 32
-            // cells at a time, so that its lanes stay together.
+            // Slot 0 of every old cell first; a cell of more disks (4 to 5% of
+            // those of 2.00 to 2.02 sigma at eta = 0.70 to 0.716, 9% at N = 256) is
+            // queued, and the warp takes its further slots 32 cells at a time,
+            // so that its lanes stay together.
             const uint32_t cells = it.lcells;
             const int lane = tid & 31;
             uint32_t* queue = s_queue[tid >> 5];

@@ -21,7 +21,9 @@
 //   more than two disks; bits 12..21 and 22..31 where slots 2 and 3 are kept:
 //   entry e of the block's pool as e + 1, or kFar for the block's global
 //   spill area.
-// About 1% of the cells hold three disks at liquid densities, so the pool is
+// Cells of three disks are rare unless cells are clearly wider than 2 sigma (counted
+// over random frames of relaxed chains: 4e-6 of the cells at 2.001 sigma, eta = 0.716;
+// 2e-5 at 2.024, 0.70; 4e-4 at 2.094, N = 1000; 1e-3 at 2.119, N = 256), so the pool is
 // small; the spill area keeps any accepted configuration correct.
 #pragma once
 
@@ -63,9 +65,9 @@ struct Stage {
     PoolEntry<FIX>* spill;  // global, [2 NC]
     uint32_t* pool_n;
     // The hard cells of each colour plane: those that hold more than two disks
-    // or have a neighbour that does (about 9% at liquid densities).  A pass
-    // gives them warps of their own: one such lane in nearly every warp made
-    // all of them walk the rare paths.  hard_n[4] is set when a list or the
+    // or have a neighbour that does (3e-5 of the cells at 2.001 sigma, 0.7% at N = 256,
+    // most where cells are wide).  A pass gives them warps of their own, so that
+    // the others do not walk the rare paths with them.  hard_n[4] is set when a list or the
     // pool overflowed; the passes then look at every cell for them.
     uint16_t* hard;       // [4][HARD] hy * HP + hx
     uint32_t* hard_n;     // [5]
