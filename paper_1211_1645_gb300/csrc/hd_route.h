@@ -12,6 +12,7 @@
 #pragma once
 
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 
 namespace hd {
@@ -57,10 +58,12 @@ inline bool one_launch_branched(const SweepShape& s, int64_t n) {
     if (n >= 3) return true;
     // One or two sweeps: the tiles' start and end.  N = 4096, fixed, one sweep 22.5 and
     // 26.6; N = 2^20 49 and 63, two 84 and 94; FP64 N = 4096 35 and 31, 524,288 53 and 63;
-    // 64 replicas of 16,384 93 and 71, 31 of 40,000 65 and 76, 48 of 65,536 138 and 129.
+    // 64 replicas of 16,384 93 and 71, 31 of 40,000 65 and 76, 48 of 65,536 138 and 129; two
+    // sweeps of eight of 65,536 56 and 61, crowded (cells of 2.5 sigma) 16 of 16,384 113 and
+    // 129, eight 110 and 93.
     const double most = s.R / 24.0;
     if (s.R > 16 && s.tile >= 4500 && s.rounds >= 4) return true;
-    if (n == 2) return s.rounds <= std::max(1.0, most) && !(s.R > 1 && s.R <= 16 && s.tile >= 3500);
+    if (n == 2) return s.rounds <= std::max(1.0, most) && !(s.R > 1 && s.R <= 16 && s.tile >= (s.fixed && s.crowded ? 1200 : 3500));
     return s.rounds <= std::max(s.fixed && !s.crowded && s.R < 16 ? 0.0 : 1.0, most);
 }
 
@@ -74,6 +77,9 @@ inline bool one_launch_pays(const SweepShape& s, int64_t n, bool step) {
     // 1000 (24 sweeps) 1348 and 5696; 76 of 16,384 633 and 636, 200 1635 and 1773; FP64 90 of
     // 1300 347 and 319, 114 of 2000 449 and 467; crowded, cells of 2.5 sigma, 70 of 4096
     // 644 and 707 (FP64 1347 and 1244), 90 of 2000 699 and 820.
+    // A single sweep whose last round of tiles is nearly empty: one replica of 800,000
+    // (1.05 rounds) 55 and 62, 1,500,000 (2.03) 76 and 82; 2^20 (1.5) 65 and 62.
+    if (!step && n == 1 && s.R == 1 && s.rounds > 1.0 && std::ceil(s.rounds) > 1.4 * s.rounds) return false;
     if (s.tile >= 4500) return true;
     const double t = s.tile;
     double most = 0.0;

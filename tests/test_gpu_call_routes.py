@@ -24,7 +24,9 @@ def hd():
 CASES = [
     ("fixed", 4096, 1, 2.0, "run", 1, False), ("fixed", 4096, 1, 2.0, "run", 2, True), ("fp64", 4096, 1, 2.0, "run", 1, True),
     ("fixed", 4096, 1, 2.0, "sweep", 1, True), ("fixed", 1000000, 1, 2.0, "run", 2, False),
-    ("fixed", 1000000, 1, 2.0, "run", 3, True), ("fp64", 524288, 1, 2.0, "sweep", 1, False),
+    ("fixed", 800000, 1, 2.0, "sweep", 1, False), ("fixed", 800000, 1, 2.0, "sweep", 2, True),
+    ("fixed", 1048576, 1, 2.0, "sweep", 1, True), ("fixed", 16384, 16, 2.5, "run", 2, False),
+    ("fixed", 16384, 8, 2.5, "run", 2, True), ("fixed", 1000000, 1, 2.0, "run", 3, True), ("fp64", 524288, 1, 2.0, "sweep", 1, False),
     # more tiles than the SMs take in a few rounds
     ("fixed", 1300, 70, 2.0, "run", 24, True), ("fixed", 1300, 200, 2.0, "run", 24, False),
     ("fixed", 1300, 114, 2.0, "sweep", 24, True), ("fixed", 1300, 200, 2.0, "sweep", 24, False),
